@@ -600,7 +600,8 @@ def measure(args, cfg: int, batch: int, rank: int, world: int, local_rank: int,
     if roof["bound"] == "tensor":
         roof["peak_kind"] = ("sustained: sw_power_cap active in the timed region" if capped
                              else "burst")
-    roof["kernel"] = "tc_search_kernel" if path == "tc" else "simt_search_kernel"
+    roof["kernel"] = ("tc_search_kernel" if path == "tc" else
+                      "f32_search_kernel" if w.dtype == "f32" else "simt_search_kernel")
     roof["kernel_ms_mean"] = statistics.mean(tim["search_ms"])
     roof["kernel_ms_median"] = statistics.median(tim["search_ms"])
     roof["event_pair_us"] = ev_pair_us

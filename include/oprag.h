@@ -348,8 +348,8 @@ OPRAG_API int oprag_index_last_timing(oprag_index *idx, float *lexical_ms, float
 OPRAG_API int oprag_index_buffer_bytes(const oprag_index *idx, int64_t *scratch, int64_t *bounds,
                                        int64_t *lexical);
 
-/* Which kernel family served the last search on this index: 1 SIMT, 2 tensor
- * core, 0 none yet. */
+/* Which kernel family served the last search on this index: 1 CUDA cores (the
+ * fp32 kernel, or the SIMT streaming kernel of a bf16 index), 2 tensor core, 0 none yet. */
 OPRAG_API int oprag_index_last_path(const oprag_index *idx);
 
 /* Launch shape of the last search's main tensor-core kernel: grid (CTAs),

@@ -112,12 +112,22 @@ struct SearchShape {
   bool fused_lex = false;
 };
 
-// --- SIMT streaming search (fp32 or bf16; any q, meant for small q).
-size_t simt_scratch_bytes(int dtype, const SearchShape& s, int grid);
+// --- SIMT streaming search (bf16, on request; any q, meant for small q).
+size_t simt_scratch_bytes(const SearchShape& s, int grid);
 int simt_grid(const SearchShape& s, int num_sms);
-cudaError_t launch_simt_search(int dtype, const void* E, const void* Q, const SearchShape& s,
+cudaError_t launch_simt_search(const void* E, const void* Q, const SearchShape& s,
                                const Fusion& fu, void* scratch, int grid, ListSet* lists,
                                cudaStream_t st);
+
+// --- fp32 search (register-tiled FMA product, search_f32.cuh).
+// slices: corpus slices per query tile.  qfloor / gen (optional): shared
+// k-th score bounds, as for the tensor-core search.
+int f32_slices(const SearchShape& s, int num_sms);
+size_t f32_scratch_bytes(const SearchShape& s, int slices);
+cudaError_t launch_f32_search(const void* E, const void* Q, const SearchShape& s, const Fusion& fu,
+                              void* scratch, int slices, ListSet* lists, cudaStream_t st,
+                              uint64_t* qfloor, uint32_t gen, int* dev_err,
+                              long long wait_limit);
 
 // --- tcgen05 tensor-core search (bf16).
 struct TcPlan {

@@ -55,7 +55,7 @@ struct DeviceGuard {
 };
 
 // bf16 searches always take the tensor-core kernel (measured faster than the
-// SIMT stream even for a single query); fp32 indices take the SIMT kernel.
+// SIMT stream even for a single query); fp32 indices take their own kernel.
 constexpr int kSimtMaxQueriesBf16 = 0;
 // Largest BM25 matrix block (floats) materialised per hybrid pass.
 constexpr int64_t kLexMaxElems = int64_t(1) << 28;
@@ -289,12 +289,12 @@ constexpr int kSampleK = OPRAG_SAMPLE_K;
 
 struct SearchLayout {
   int path = 0;           // 1 SIMT, 2 tensor core
-  int simt_grid = 0;
+  int simt_grid = 0;      // CTAs (bf16) or corpus slices (fp32) of path 1
   TcPlan plan{}, splan{};
   bool sampled = false;
   size_t main_bytes = 0;    // multiple of 256
   size_t sample_bytes = 0;  // 0 unless sampled
-  bool floors = false;      // q shared bounds (register lists on the tensor-core path)
+  bool floors = false;      // q shared bounds (fp32, and register lists on the tensor-core path)
   size_t total() const { return main_bytes + sample_bytes; }
 };
 
@@ -308,8 +308,14 @@ SearchLayout search_layout(oprag_index* idx, int q, int k, int path, int block_n
   s.n_second = path == 2 ? n_second : 0;
   L.path = path;
   if (path == 1) {
-    L.simt_grid = simt_grid(s, idx->num_sms);
-    L.main_bytes = round256(simt_scratch_bytes(idx->dtype, s, L.simt_grid));
+    if (idx->dtype == OPRAG_F32) {
+      L.simt_grid = f32_slices(s, idx->num_sms);
+      L.main_bytes = round256(f32_scratch_bytes(s, L.simt_grid));
+      L.floors = true;
+    } else {
+      L.simt_grid = simt_grid(s, idx->num_sms);
+      L.main_bytes = round256(simt_scratch_bytes(s, L.simt_grid));
+    }
     return L;
   }
   L.plan = tc_plan(s, idx->num_sms, block_n, 1, pair, pair_capacity(idx));
@@ -355,7 +361,10 @@ int launch_search(oprag_index* idx, const SearchLayout& L, const void* Q, int q,
   if (idx->timing) cudaEventRecord(idx->ev[1], st);
   idx->timed_sample = idx->timing && L.sampled;
   if (L.path == 1) {
-    e = launch_simt_search(idx->dtype, idx->emb, Q, s, fu, scratch, L.simt_grid, &lists, st);
+    e = idx->dtype == OPRAG_F32
+            ? launch_f32_search(idx->emb, Q, s, fu, scratch, L.simt_grid, &lists, st, qf, gen,
+                                idx->dev_err, idx->wait_limit)
+            : launch_simt_search(idx->emb, Q, s, fu, scratch, L.simt_grid, &lists, st);
   } else {
     const float* floor = nullptr;
     float* levels = nullptr;
@@ -619,6 +628,10 @@ int oprag_index_reserve(oprag_index* idx, int32_t q_max, int32_t k_max) {
   size_t need = 0;
   for (int kk : {8, 16, 32, 128, 256}) {
     const int k = std::min(kk, kcap);
+    // fp32: the slices depend on the number of query tiles (of 32 at least)
+    if (idx->dtype == OPRAG_F32)
+      for (int64_t qq = 32; qq <= q_max; qq += 32)
+        need = std::max(need, search_layout(idx, static_cast<int>(qq), k, 1, 0, 0).total());
     for (int qq : {static_cast<int>(q_max), std::min<int>(q_max, 128)}) {
       need = std::max(need, search_layout(idx, qq, k, 1, 0, 0).total());
       if (idx->dtype != OPRAG_BF16) continue;
@@ -820,7 +833,7 @@ int oprag_search_two(oprag_index* knowledge, oprag_index* memory, const void* qu
     if ((rc = end_call(memory, st))) return rc;
     return end_call(knowledge, st);
   }
-  // fp32 indices (SIMT kernel): each index's top-k, then one two-list merge.
+  // fp32 indices: each index's top-k, then one two-list merge.
   const int ka = static_cast<int>(std::min<int64_t>(k, knowledge->n));
   const int kb = static_cast<int>(std::min<int64_t>(k, memory->n));
   if ((rc = knowledge->ensure(&knowledge->cand, &knowledge->cand_bytes,

@@ -1,0 +1,456 @@
+// Search of fp32 indices: the query x chunk inner products of Sec. 4.4 as a
+// register-tiled fp32 product on the CUDA cores (the scores must be fp32 sums
+// of fp32 products, which the tensor cores do not give), with the partial
+// top-k selection (Sec. 4.4, Sec. 7) fused behind it.
+//
+// A CTA of 256 threads takes one query tile of TY * TM queries and one
+// contiguous slice of the corpus, in tiles of 4 * TX rows (TX = 256 / TY).
+// Thread (ty, tx) holds the scores of queries ty + TY i (i < TM) and rows
+// tx + TX j (j < 4); a warp covers 4 ty and 8 tx, so that each of its 16-byte
+// shared-memory reads touches at most 128 different bytes (measured: 2.1
+// cycles of the SM each; 4.2 for 16 rows or more).  K blocks of 32 floats of
+// both operands come through a TMA ring (128-byte swizzle: eight rows' reads
+// of one k group touch all banks once) that thread 0 feeds between its own
+// blocks: a ninth warp would cap every thread at 168 registers.  Every two K blocks
+// the sums are folded into one of two second-level sums in turn, so that no
+// chain of additions is longer than 64, or than d / 128 at the second level.
+//
+// What bounds it: from about 16 queries on the FMA pipes and, next to them,
+// the shared-memory reads that feed them (a warp step of four k: 112 FMA issue
+// slots and 11 reads with TM = 7), below that HBM.  The tile shape follows the
+// batch (config_for): TY = 4 (256 corpus rows) up to 32 queries, TY = 8 up to
+// 64, TY = 16 above.  Measured on GB300, 32768 x 768 and k = 10, search kernel,
+// against the streaming kernel this one replaced (each chunk of eight queries
+// streamed the corpus again, five shuffles per score): 1 query 29 (51) us, 16
+// queries 43 (92) us, 100 queries 182 (528) us or 27.7 TFLOP/s, 256 queries
+// 366 (1298) us; 100000 x 768 and 1 query 63 (119) us or 4.9 TB/s; 100 queries
+// and k = 100 272 (1542) us.
+//
+// Selection.  Each query of the tile has a buffer of candidate keys in shared
+// memory.  A score enters it when it reaches the query's floor: the k-th
+// largest of a warp's group maxima in the first tile (k distinct scores reach
+// it), then what compactions prove and what the other slices of the search
+// publish (qfloor).  A buffer that could overflow within the next tile is
+// sorted by one warp and cut to its k best; at the end the buffers are sorted
+// into one list per (query, slice) for the merge kernel.
+#pragma once
+#include "common.cuh"
+#include "internal.h"
+
+namespace oprag {
+namespace f32 {
+
+constexpr int kThreads = 256;
+constexpr int kBK = 32;                    // floats per K block: one 128-byte swizzle row
+constexpr int kRowBytes = kBK * 4;
+constexpr int kRowsPerThread = 4;
+constexpr int kFoldBlocks = 2;             // K blocks between folds
+constexpr int kMaxCap = 512;               // candidate keys per query
+constexpr int kMaxStages = 8;
+constexpr size_t kSmemMax = 226 * 1024;
+
+struct Params {
+  int64_t n;
+  int d;
+  int q;
+  int k;
+  Fusion fu;
+  uint64_t* lists;      // [(tile * G + slice) * TH + query] * stride
+  int stride;
+  int cap;
+  int stages;
+  uint64_t* qfloor;     // optional: shared k-th bounds, tagged gen
+  uint32_t gen;
+  int* dev_err;
+  long long wait_limit;
+};
+
+// Launch shape of one search (host side, also its scratch size).
+struct Config {
+  int TY, TM;
+  int th;        // queries per tile, TY * TM
+  int qt;        // query tiles
+  int G;         // corpus slices
+  int cap, stages;
+  size_t smem;
+};
+
+// Bytes of a ring stage (whole swizzle atoms).
+__host__ __device__ constexpr int stage_bytes(int th, int bn) {
+  return (bn * kRowBytes + th * kRowBytes + 1023) / 1024 * 1024;
+}
+
+// One K block: eight groups of four k (zeros past d), TN of the thread's four
+// rows.  a0 / b0: the thread's first query / corpus row of the stage.
+template <int TY, int TM, int TN>
+__device__ __forceinline__ void mul_block(const unsigned char* a0, const unsigned char* b0, int ty,
+                                          int tx, float (&acc)[TM][kRowsPerThread]) {
+  constexpr int TX = kThreads / TY;
+#pragma unroll
+  for (int s = 0; s < kBK / 4; ++s) {
+    const int ob = (s ^ (tx & 7)) << 4;
+    float4 b[TN];
+#pragma unroll
+    for (int j = 0; j < TN; ++j)
+      b[j] = *reinterpret_cast<const float4*>(b0 + j * TX * kRowBytes + ob);
+#pragma unroll
+    for (int i = 0; i < TM; ++i) {
+      // row ty + TY i of the tile; its swizzle phase alternates when TY = 4
+      const int oa = (s ^ ((ty + TY * i) & 7)) << 4;
+      const float4 a = *reinterpret_cast<const float4*>(a0 + i * TY * kRowBytes + oa);
+#pragma unroll
+      for (int j = 0; j < TN; ++j) acc[i][j] = fmaf(a.x, b[j].x, acc[i][j]);
+#pragma unroll
+      for (int j = 0; j < TN; ++j) acc[i][j] = fmaf(a.y, b[j].y, acc[i][j]);
+#pragma unroll
+      for (int j = 0; j < TN; ++j) acc[i][j] = fmaf(a.z, b[j].z, acc[i][j]);
+#pragma unroll
+      for (int j = 0; j < TN; ++j) acc[i][j] = fmaf(a.w, b[j].w, acc[i][j]);
+    }
+  }
+}
+
+// The warp puts the min(c, k) best of the c keys of a buffer, best first, into
+// dst (which may be the buffer).  Up to 64 keys -- the usual case, a good
+// floor leaves few more than k -- every lane counts the keys above its own
+// ones: no chain of dependent exchanges (14 queries a warp at the end of a
+// search: 1 us instead of 10 us of bitonic sorts).  More keys are sorted.
+template <int E>
+__device__ __noinline__ void sort_best(uint64_t* buf, int c, int k, uint64_t* dst) {
+  const int lane = threadIdx.x & 31;
+  uint64_t v[E];
+#pragma unroll
+  for (int e = 0; e < E; ++e) v[e] = lane * E + e < c ? buf[lane * E + e] : kEmptyKey;
+  warp_sort_desc<E>(v);
+  __syncwarp();
+#pragma unroll
+  for (int e = 0; e < E; ++e)
+    if (lane * E + e < min(c, k)) dst[lane * E + e] = v[e];
+  __syncwarp();
+}
+
+template <int E>
+__device__ __forceinline__ void rank_best(const uint64_t* buf, int c, int k, uint64_t* dst) {
+  const int lane = threadIdx.x & 31;
+  uint64_t v[E];
+  int above[E];
+#pragma unroll
+  for (int e = 0; e < E; ++e) {
+    v[e] = lane + 32 * e < c ? buf[lane + 32 * e] : kEmptyKey;
+    above[e] = 0;
+  }
+#pragma unroll 4
+  for (int i = 0; i < c; ++i) {
+    const uint64_t o = buf[i];
+#pragma unroll
+    for (int e = 0; e < E; ++e) above[e] += o > v[e] ? 1 : 0;
+  }
+  __syncwarp();
+#pragma unroll
+  for (int e = 0; e < E; ++e)
+    if (lane + 32 * e < c && above[e] < k) dst[above[e]] = v[e];
+  __syncwarp();
+}
+
+__device__ __forceinline__ void keep_best(uint64_t* buf, int c, int k, uint64_t* dst) {
+  if (c <= 32) rank_best<1>(buf, c, k, dst);
+  else if (c <= 64) rank_best<2>(buf, c, k, dst);
+  else if (c <= 128) sort_best<4>(buf, c, k, dst);
+  else if (c <= 256) sort_best<8>(buf, c, k, dst);
+  else sort_best<16>(buf, c, k, dst);
+}
+
+// The value of rank r (0-based, descending) among the 8 E values of each group
+// of eight lanes: a bitonic sort, element l E + e in lane l of the group.
+template <int E>
+__device__ __forceinline__ float rank_of_8(float (&v)[E], int r) {
+  const int l = threadIdx.x & 7;
+#pragma unroll
+  for (int size = 2; size <= 8 * E; size <<= 1) {
+#pragma unroll
+    for (int stride = size >> 1; stride > 0; stride >>= 1) {
+      if (stride < E) {
+#pragma unroll
+        for (int e = 0; e < E; ++e)
+          if ((e & stride) == 0) {
+            const bool desc = ((l * E + e) & size) == 0;
+            const float hi = fmaxf(v[e], v[e | stride]), lo = fminf(v[e], v[e | stride]);
+            v[e] = desc ? hi : lo;
+            v[e | stride] = desc ? lo : hi;
+          }
+      } else {
+        const int lm = stride / E;
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+          const bool desc = ((l * E + e) & size) == 0;
+          const float o = __shfl_xor_sync(0xffffffffu, v[e], lm);
+          v[e] = (((l & lm) == 0) == desc) ? fmaxf(v[e], o) : fminf(v[e], o);
+        }
+      }
+    }
+  }
+  float m = v[0];
+#pragma unroll
+  for (int e = 1; e < E; ++e)
+    if (e == (r & (E - 1))) m = v[e];
+  return __shfl_sync(0xffffffffu, m, r / E, 8);
+}
+
+template <int TY, int TM>
+__global__ void __launch_bounds__(kThreads, 1)
+f32_search_kernel(const __grid_constant__ CUtensorMap map_q,
+                  const __grid_constant__ CUtensorMap map_e, const Params p) {
+  constexpr int TX = kThreads / TY;
+  constexpr int BM = TY * TM, BN = TX * kRowsPerThread;
+  constexpr int kStage = stage_bytes(BM, BN);
+  constexpr int WY = TY / 4;                          // warps along the queries
+  extern __shared__ __align__(1024) unsigned char smem_f[];
+  // (an offset, not a rounded pointer: the compiler then still knows that the
+  // ring is shared memory)
+  unsigned char* ring = smem_f + ((1024 - (smem_addr(smem_f) & 1023)) & 1023);
+  uint64_t* buf = reinterpret_cast<uint64_t*>(ring + p.stages * kStage);
+  uint64_t* full = buf + static_cast<size_t>(BM) * p.cap;
+  uint64_t* empty = full + kMaxStages;
+  int* cnt = reinterpret_cast<int*>(empty + kMaxStages);
+  uint32_t* flo = reinterpret_cast<uint32_t*>(cnt + BM);    // score_order of each floor
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(flo + BM);
+
+  // Let the merge kernel get scheduled; it waits for this grid to finish.
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int q0 = blockIdx.y * BM;
+  const int64_t r_begin = p.n * blockIdx.x / gridDim.x;
+  const int64_t r_end = p.n * (blockIdx.x + 1) / gridDim.x;
+  const int tiles = static_cast<int>((r_end - r_begin + BN - 1) / BN);
+  const int nkb = (p.d + kBK - 1) / kBK;
+
+  if (tid == 0) {
+    for (int s = 0; s < p.stages; ++s) {
+      mbar_init(&full[s], 1);
+      mbar_init(&empty[s], kThreads / 32);
+    }
+    *abort_flag = 0;
+    fence_mbar_init();
+    prefetch_map(&map_q);
+    prefetch_map(&map_e);
+  }
+  if (tid < BM) {
+    cnt[tid] = 0;
+    flo[tid] = score_order(-INFINITY);
+  }
+  __syncthreads();
+
+  // Groups of TX rows (1 .. 4) that the tile at row r0 needs.
+  auto groups_of = [&](int64_t r0) {
+    const int64_t left = r_end - r0;
+    return left >= BN ? kRowsPerThread : static_cast<int>((left + TX - 1) / TX);
+  };
+
+  // Loads.  Block m = 8 i + w is issued by lane 0 of warp w, at the start of
+  // the warps' own block m + lag - stages, into the stage that block m - stages
+  // used; with lag 2 its wait for the other warps to leave that stage is
+  // almost never one.  The warps take turns because issuing a block's copies
+  // takes a thread about as long as one of its math steps.
+  const int blocks = tiles * nkb;
+  const int lag = p.stages >= 4 ? 2 : 1;
+  int ld_m = warp, ld_s = warp % p.stages, ld_kb = warp % nkb;
+  uint32_t ld_ph = (warp / p.stages) & 1, issued = 0, parity = 0;
+  int64_t ld_r0 = r_begin + static_cast<int64_t>(warp / nkb) * BN;
+  auto load_next = [&]() {
+    if (lane == 0 && !*abort_flag &&
+        mbar_wait(&empty[ld_s], ld_ph ^ 1u, abort_flag, p.dev_err, p.wait_limit)) {
+      unsigned char* sB = ring + ld_s * kStage;
+      const int tn = groups_of(ld_r0);
+      mbar_arrive_expect_tx(&full[ld_s], static_cast<uint32_t>((tn * TX + BM) * kRowBytes));
+      for (int j = 0; j < tn; ++j)
+        tma_load_2d(sB + j * TX * kRowBytes, &map_e, &full[ld_s], ld_kb * kBK,
+                    static_cast<int>(ld_r0) + j * TX);
+      tma_load_2d(sB + BN * kRowBytes, &map_q, &full[ld_s], ld_kb * kBK, q0);
+      issued |= 1u << ld_s;
+      parity = (parity & ~(1u << ld_s)) | (ld_ph << ld_s);
+    }
+    __syncwarp();
+    ld_m += kThreads / 32;
+    for (ld_s += kThreads / 32; ld_s >= p.stages; ld_s -= p.stages) ld_ph ^= 1u;
+    for (ld_kb += kThreads / 32; ld_kb >= nkb; ld_kb -= nkb) ld_r0 += BN;
+  };
+  if (ld_m < p.stages - lag && ld_m < blocks) load_next();
+
+  // A wait that gives up does not end a warp early (the warps meet at
+  // barriers): it goes on with whatever the stage holds, and every later wait
+  // returns at once because the abort word is set.
+  const int ty = (warp % WY) * 4 + (lane >> 3);
+  const int tx = (warp / WY) * 8 + (lane & 7);
+  float acc[TM][kRowsPerThread], tot[2][TM][kRowsPerThread];
+  int st = 0, blk = 0;
+  uint32_t ph = 0;
+#pragma unroll 1
+  for (int tile = 0; tile < tiles; ++tile) {
+    const int64_t r0 = r_begin + static_cast<int64_t>(tile) * BN;
+    const int tn = groups_of(r0);
+#pragma unroll
+    for (int i = 0; i < TM; ++i)
+#pragma unroll
+      for (int j = 0; j < kRowsPerThread; ++j) acc[i][j] = tot[0][i][j] = tot[1][i][j] = 0.f;
+    // What the other slices have published about this tile's queries.
+    if (p.qfloor != nullptr && tile > 0 && tid < BM && q0 + tid < p.q) {
+      const unsigned long long v =
+          __ldcg(reinterpret_cast<const unsigned long long*>(p.qfloor + q0 + tid));
+      if (static_cast<uint32_t>(v >> 32) == p.gen)
+        atomicMax(flo + tid, static_cast<uint32_t>(v));
+    }
+#pragma unroll 1
+    for (int kb = 0; kb < nkb; ++kb, ++blk) {
+      if (ld_m == blk + p.stages - lag && ld_m < blocks) load_next();
+      mbar_wait(&full[st], ph, abort_flag, p.dev_err, p.wait_limit);
+      __syncwarp();
+      const unsigned char* sB = ring + st * kStage + tx * kRowBytes;
+      const unsigned char* sA = ring + st * kStage + (BN + ty) * kRowBytes;
+      if (tn == 4) mul_block<TY, TM, 4>(sA, sB, ty, tx, acc);
+      else if (tn == 3) mul_block<TY, TM, 3>(sA, sB, ty, tx, acc);
+      else if (tn == 2) mul_block<TY, TM, 2>(sA, sB, ty, tx, acc);
+      else mul_block<TY, TM, 1>(sA, sB, ty, tx, acc);
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&empty[st]);
+      if (++st == p.stages) {
+        st = 0;
+        ph ^= 1u;
+      }
+      if ((kb + 1) % kFoldBlocks == 0 || kb + 1 == nkb) {
+        // the two second-level sums swap, so that each takes every other fold
+#pragma unroll
+        for (int i = 0; i < TM; ++i)
+#pragma unroll
+          for (int j = 0; j < kRowsPerThread; ++j) {
+            const float t = tot[0][i][j] + acc[i][j];
+            tot[0][i][j] = tot[1][i][j];
+            tot[1][i][j] = t;
+            acc[i][j] = 0.f;
+          }
+      }
+    }
+
+    // ---- selection
+    // The scores (in the accumulators' place), -inf where there is none.
+#pragma unroll
+    for (int i = 0; i < TM; ++i) {
+      const int qg = q0 + ty + TY * i;
+      float inv_max = 0.f;
+      const float* brow = nullptr;
+      if (p.fu.bm25 != nullptr && qg < p.q) {
+        const float m = p.fu.bm25_max[qg];
+        inv_max = m > 0.f ? 1.f / m : 0.f;
+        brow = p.fu.bm25 + static_cast<int64_t>(qg) * p.fu.ld;
+      }
+#pragma unroll
+      for (int j = 0; j < kRowsPerThread; ++j) {
+        const int64_t r = r0 + tx + TX * j;
+        float v = tot[0][i][j] + tot[1][i][j];
+        if (brow != nullptr && r < r_end)
+          v = fmaf(p.fu.alpha, v, (1.f - p.fu.alpha) * (brow[r] * inv_max));
+        acc[i][j] = r < r_end && qg < p.q ? v : -INFINITY;
+      }
+    }
+    if (tile == 0 && p.k <= 32 && r_end - r_begin > 64) {
+      // First floors: the k-th largest of the maxima of 8, 16 or 32 groups of
+      // the warp's 32 scores of a query (k distinct scores reach it), then
+      // the best such bound of the CTA and of the slices that are as far.  (A
+      // slice of up to 64 rows takes them all: ranking 64 keys is cheaper.)
+#pragma unroll
+      for (int i = 0; i < TM; ++i) {
+        const int ql = ty + TY * i;
+        float b;
+        if (p.k <= 8) {
+          float m[1] = {fmaxf(fmaxf(acc[i][0], acc[i][1]), fmaxf(acc[i][2], acc[i][3]))};
+          b = rank_of_8<1>(m, p.k - 1);
+        } else if (p.k <= 16) {
+          float m[2] = {fmaxf(acc[i][0], acc[i][1]), fmaxf(acc[i][2], acc[i][3])};
+          b = rank_of_8<2>(m, p.k - 1);
+        } else {
+          float m[4] = {acc[i][0], acc[i][1], acc[i][2], acc[i][3]};
+          b = rank_of_8<4>(m, p.k - 1);
+        }
+        if ((lane & 7) == 0 && b > -INFINITY) atomicMax(flo + ql, score_order(b));
+      }
+      __syncthreads();
+      if (p.qfloor != nullptr && tid < BM && q0 + tid < p.q) {
+        const unsigned long long mine =
+            (static_cast<unsigned long long>(p.gen) << 32) | flo[tid];
+        const unsigned long long old =
+            atomicMax(reinterpret_cast<unsigned long long*>(p.qfloor + q0 + tid), mine);
+        if (old > mine && static_cast<uint32_t>(old >> 32) == p.gen)
+          flo[tid] = static_cast<uint32_t>(old);
+      }
+    }
+    // The previous tile's compactions and the floors are done.
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < TM; ++i) {
+      const int ql = ty + TY * i;
+      const bool qv = q0 + ql < p.q;
+      const float fl = order_score(flo[ql]);
+#pragma unroll
+      for (int j = 0; j < kRowsPerThread; ++j)
+        if (acc[i][j] >= fl && qv && r0 + tx + TX * j < r_end)
+          buf[ql * p.cap + atomicAdd(cnt + ql, 1)] =
+              make_key(acc[i][j], static_cast<uint32_t>(r0 + tx + TX * j));
+    }
+    __syncthreads();
+    // Buffers without room for another tile, or of the last tile: keep the k
+    // best.
+    const bool last = tile + 1 == tiles;
+    for (int ql = warp; ql < BM; ql += kThreads / 32) {
+      if (q0 + ql >= p.q) break;
+      const int c = cnt[ql];
+      uint64_t* b = buf + ql * p.cap;
+      if (last) {
+        uint64_t* dst = p.lists + ((static_cast<int64_t>(blockIdx.y) * gridDim.x + blockIdx.x) * BM +
+                                   ql) * p.stride;
+        keep_best(b, c, p.k, dst);
+        for (int i = c + lane; i < p.k; i += 32) dst[i] = kEmptyKey;
+      } else if (c > p.cap - BN) {
+        keep_best(b, c, p.k, b);
+        if (lane == 0) {
+          cnt[ql] = min(c, p.k);
+          if (c >= p.k) {
+            const uint32_t o = static_cast<uint32_t>(b[p.k - 1] >> 32);
+            atomicMax(flo + ql, o);
+            if (p.qfloor != nullptr)
+              atomicMax(reinterpret_cast<unsigned long long*>(p.qfloor + q0 + ql),
+                        (static_cast<unsigned long long>(p.gen) << 32) | o);
+          }
+        }
+      }
+    }
+  }
+  // After a wait gave up, copies may still fly: the CTA outlives them.
+  if (lane == 0 && *abort_flag)
+    for (int i = 0; i < p.stages; ++i)
+      if (issued & (1u << i)) mbar_drain(&full[i], (parity >> i) & 1u, p.dev_err);
+}
+
+template <int TY, int TM>
+cudaError_t launch_tm(const Config& c, const CUtensorMap& mq, const CUtensorMap& me,
+                      const Params& p, cudaStream_t st) {
+  static bool configured = false;
+  if (!configured) {
+    cudaError_t e = cudaFuncSetAttribute(f32_search_kernel<TY, TM>,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         static_cast<int>(kSmemMax));
+    if (e != cudaSuccess) return e;
+    configured = true;
+  }
+  f32_search_kernel<TY, TM><<<dim3(c.G, c.qt), kThreads, c.smem, st>>>(mq, me, p);
+  return cudaGetLastError();
+}
+
+// Instantiations live in their own translation units (parallel builds).
+cudaError_t launch_ty4(const Config& c, const CUtensorMap& mq, const CUtensorMap& me,
+                       const Params& p, cudaStream_t st);
+cudaError_t launch_ty8(const Config& c, const CUtensorMap& mq, const CUtensorMap& me,
+                       const Params& p, cudaStream_t st);
+cudaError_t launch_ty16(const Config& c, const CUtensorMap& mq, const CUtensorMap& me,
+                        const Params& p, cudaStream_t st);
+
+}  // namespace f32
+}  // namespace oprag

@@ -34,8 +34,7 @@ int simt_grid(const SearchShape& s, int num_sms) {
   return static_cast<int>(grid);
 }
 
-size_t simt_scratch_bytes(int dtype, const SearchShape& s, int grid) {
-  (void)dtype;
+size_t simt_scratch_bytes(const SearchShape& s, int grid) {
   const int QC = qc_for(s);
   const int K = list_len_for(s.k);
   const int64_t chunks = (s.q + QC - 1) / QC;
@@ -44,12 +43,10 @@ size_t simt_scratch_bytes(int dtype, const SearchShape& s, int grid) {
   return bytes;
 }
 
-cudaError_t launch_simt_search(int dtype, const void* E, const void* Q, const SearchShape& s,
+cudaError_t launch_simt_search(const void* E, const void* Q, const SearchShape& s,
                                const Fusion& fu, void* scratch, int grid, ListSet* lists,
                                cudaStream_t st) {
-  const int QC = qc_for(s);
-  return dtype == kF32 ? launch_f32(QC, E, Q, s, fu, scratch, grid, lists, st)
-                       : launch_bf16(QC, E, Q, s, fu, scratch, grid, lists, st);
+  return launch_bf16(qc_for(s), E, Q, s, fu, scratch, grid, lists, st);
 }
 
 }  // namespace oprag

@@ -2,9 +2,8 @@
 // matrix operations over the embedding matrix") with the running partial top-k
 // fused in (Sec. 4.4 / Sec. 7: partial selection instead of a full sort).
 //
-// Used for fp32 indices (whose scores must be exact fp32 FMA sums, which the
-// bf16 tensor path cannot give) and for bf16 searches with very few queries,
-// where the pass is a pure HBM stream and tensor cores buy nothing.
+// The alternative to the tensor-core kernel for bf16 indices
+// (OPRAG_OPT_PATH = 1); fp32 indices have their own kernel (search_f32.cuh).
 //
 // Layout: each warp owns a contiguous range of corpus rows and walks it one
 // row at a time with 16-byte loads spread over its 32 lanes (4 rows in flight
@@ -27,17 +26,6 @@ template <typename T>
 struct Vec;
 
 template <>
-struct Vec<float> {
-  static constexpr int kElems = 4;
-  __device__ __forceinline__ static void unpack(const uint4& v, float (&x)[4]) {
-    x[0] = __uint_as_float(v.x);
-    x[1] = __uint_as_float(v.y);
-    x[2] = __uint_as_float(v.z);
-    x[3] = __uint_as_float(v.w);
-  }
-};
-
-template <>
 struct Vec<__nv_bfloat16> {
   static constexpr int kElems = 8;
   __device__ __forceinline__ static void unpack(const uint4& v, float (&x)[8]) {
@@ -54,8 +42,6 @@ struct Vec<__nv_bfloat16> {
 
 template <typename T>
 __device__ __forceinline__ float to_f32(T v);
-template <>
-__device__ __forceinline__ float to_f32<float>(float v) { return v; }
 template <>
 __device__ __forceinline__ float to_f32<__nv_bfloat16>(__nv_bfloat16 v) {
   return __bfloat162float(v);
@@ -264,8 +250,6 @@ cudaError_t launch_qc(const void* E, const void* Q, const SearchShape& s, const 
   }
 }
 
-cudaError_t launch_f32(int qc, const void* E, const void* Q, const SearchShape& s, const Fusion& fu,
-                       void* scratch, int grid, ListSet* lists, cudaStream_t st);
 cudaError_t launch_bf16(int qc, const void* E, const void* Q, const SearchShape& s,
                         const Fusion& fu, void* scratch, int grid, ListSet* lists,
                         cudaStream_t st);

@@ -219,19 +219,6 @@ constexpr size_t smem_for() {
 
 // ----------------------------------------------------------------- PTX
 
-__device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* map, uint64_t* bar, int x,
-                                            int y) {
-  asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes"
-      " [%0], [%1, {%3, %4}], [%2];" ::"r"(smem_addr(dst)),
-      "l"(reinterpret_cast<uint64_t>(map)), "r"(smem_addr(bar)), "r"(x), "r"(y)
-      : "memory");
-}
-
-__device__ __forceinline__ void prefetch_map(const CUtensorMap* map) {
-  asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(map)) : "memory");
-}
-
 __device__ __forceinline__ void tc_fence_before() {
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
 }
@@ -474,19 +461,6 @@ __device__ __forceinline__ float max32(const float (&v)[32]) {
   const float b0 = fmax3(a[0], a[1], a[2]), b1 = fmax3(a[3], a[4], a[5]);
   const float b2 = fmax3(a[6], a[7], a[8]), b3 = fmax3(a[9], a[10], a[11]);
   return fmaxf(fmax3(b0, b1, b2), b3);
-}
-
-// Waits without looking at the abort word (used to drain in-flight copies and
-// MMAs before the CTA exits); still bounded.
-__device__ __forceinline__ bool mbar_drain(uint64_t* bar, uint32_t parity, int* dev_err) {
-  const long long t0 = clock64();
-  while (!mbar_test(bar, parity)) {
-    if (clock64() - t0 > kWaitLimitCycles) {
-      atomicExch(dev_err, static_cast<int>(kDevErrWaitTimeout));
-      return false;
-    }
-  }
-  return true;
 }
 
 // ----------------------------------------------------------------- lists

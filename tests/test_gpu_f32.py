@@ -1,0 +1,103 @@
+"""GPU parity of the fp32 search (register-tiled FMA kernel) at the edges of
+its tile shapes: query counts around every tile size, corpora around the tile
+height and the slice count, d around the 32-float K block, k around the list
+lengths; ties that fill the candidate buffers; the fused hybrid form."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from oracle import check
+from paper_2608_08340_gb300 import workloads
+from paper_2608_08340_gb300.index import Index
+
+from _gpu import TOL, check_dense, dev_tensor
+
+pytestmark = pytest.mark.gpu
+
+
+def _bound(d):
+    """fp32 error bound of a score of unit vectors: chains of at most 32 and
+    d / 64 + 1 rounded additions, one product rounding (fused), two joins; the
+    sum of |products| is at most 1."""
+    return (32 + d // 64 + 4) * 2.0 ** -24
+
+
+@pytest.mark.parametrize("n,d,q,k", [
+    (1, 8, 1, 1),               # one row, one query, a quarter of a K block
+    (17, 32, 4, 17),            # k = n, one K block, TM = 1
+    (255, 40, 5, 5),            # TM = 2, a partial second K block
+    (3000, 64, 31, 32),         # TM = 8 of 4, the last k of 32-key lists
+    (40000, 72, 32, 5),         # several tiles a slice
+    (4097, 96, 33, 16),         # TY = 8, TM = 5
+    (5000, 128, 64, 33),        # k > 32: query tiles of 32
+    (33000, 200, 64, 32),       # TY = 8, TM = 8, k = W
+    (9000, 136, 65, 16),        # TY = 16, TM = 5, k = W
+    (9000, 136, 65, 32),        # floors from all 32 scores of a warp
+    (70000, 24, 100, 10),       # d below one K block, many tiles a slice
+    (2000, 384, 128, 1),
+    (2000, 264, 129, 8),        # two tiles of 80
+    (300, 64, 700, 100),        # k > 32 with many query tiles
+    (3000, 512, 3, 256),        # K_MAX
+])
+def test_tile_edges(n, d, q, k):
+    rng = np.random.default_rng(n + d + q + k)
+    E = workloads._normalise(rng.standard_normal((n, d)).astype(np.float32))
+    Q = workloads._normalise(rng.standard_normal((q, d)).astype(np.float32))
+    idx = Index(dev_tensor(E))
+    Qd = dev_tensor(Q)
+    for _ in range(2):          # the second search reuses the shared bounds
+        ids, sc = idx.search(Qd, k)
+        check_dense(ids, sc, E, Q, k, f"f32 n={n} d={d} q={q} k={k}")
+        i = ids.cpu().numpy()
+        want = np.einsum("qkd,qd->qk", E.astype(np.float64)[i], Q.astype(np.float64))
+        assert np.abs(sc.cpu().numpy() - want).max() <= _bound(d)
+
+
+@pytest.mark.parametrize("q,k", [(3, 7), (40, 20), (90, 16), (20, 100)])
+def test_equal_scores_fill_every_buffer(q, k):
+    """Every row reaches the floor, so every tile compacts every buffer."""
+    E = np.ones((20000, 16), np.float32)
+    idx = Index(dev_tensor(E))
+    ids, sc = idx.search(dev_tensor(np.ones((q, 16), np.float32)), k)
+    assert ids.cpu().tolist() == [list(range(k))] * q
+    assert (sc.cpu().numpy() == 16).all()
+
+
+def test_rising_scores_replace_every_candidate():
+    """Scores rise with the id: each tile displaces all that came before."""
+    n = 30000
+    E = np.zeros((n, 8), np.float32)
+    E[:, 0] = np.arange(n)
+    Q = np.zeros((70, 8), np.float32)
+    Q[:, 0] = 1 + np.arange(70)
+    ids, sc = Index(dev_tensor(E)).search(dev_tensor(Q), 10)
+    assert ids.cpu().tolist() == [list(range(n - 1, n - 11, -1))] * 70
+    assert (sc.cpu().numpy() == (1 + np.arange(70))[:, None] *
+            np.arange(n - 1, n - 11, -1)[None]).all()
+
+
+@pytest.mark.parametrize("q", [6, 70])
+def test_fused_hybrid(q):
+    w = workloads.make_dense("f32h", 3000, 64, q, 9, "f32", 7)
+    workloads.add_sparse(w, 7)
+    idx = Index(dev_tensor(w.E_data))
+    idx.set_sparse(w.doc_indptr, w.doc_terms, w.vocab, w.k1, w.b)
+    ids, sc = idx.hybrid_search(dev_tensor(w.Q_data), torch.from_numpy(w.q_indptr),
+                                torch.from_numpy(w.q_terms), w.alpha, w.k)
+    o_ids, o_sc, _ = oracle.hybrid_search(w.E_data, w.Q_data, w.doc_indptr, w.doc_terms, w.vocab,
+                                          w.q_indptr, w.q_terms, w.alpha, w.k + 48, w.k1, w.b)
+    check.check_topk(ids.cpu().numpy(), sc.cpu().numpy(), o_ids, o_sc, w.k, TOL, n=w.n,
+                     label=f"f32 hybrid q={q}")
+
+
+@pytest.mark.parametrize("q,k", [(1, 256), (40, 32), (130, 5), (500, 16)])
+def test_reserve_covers_smaller_batches(q, k):
+    rng = np.random.default_rng(q)
+    idx = Index(dev_tensor(rng.standard_normal((6000, 32)).astype(np.float32)))
+    idx.reserve(q, k)
+    before = idx.buffer_bytes()
+    for qq in {1, q // 3 + 1, q // 2 + 1, q}:
+        for kk in {1, k}:
+            idx.search(dev_tensor(rng.standard_normal((qq, 32)).astype(np.float32)), kk)
+    assert idx.buffer_bytes() == before
