@@ -433,7 +433,7 @@ def measure(args, cfg: int, batch: int, rank: int, world: int, local_rank: int,
             last["out"] = (ids, scores)
 
     # our kernels per step: search + merge; k > 32 over many tiles adds the
-    # sampled first pass (search + merge); config 3 adds the BM25 pass
+    # group pass and selection of k > 32; config 3 adds the BM25 pass
     # (dense-first: the rerank), config 4 the upsert scatter.
     for i in range(args.warmup):
         flush.zero_()
@@ -608,7 +608,7 @@ def measure(args, cfg: int, batch: int, rank: int, world: int, local_rank: int,
     roof["merge_ms_mean"] = statistics.mean(tim["merge_ms"])
     roof["merge_ms_median"] = statistics.median(tim["merge_ms"])
     if sampled:
-        # k > 32: the first pass over every 32nd corpus tile and its merge,
+        # k > 32: the group pass over some corpus tiles and its selection,
         # timed apart from the main pass (the dominant kernel above)
         roof["sample_pass_ms_mean"] = statistics.mean(tim["sample_ms"])
         roof["sample_pass_ms_median"] = statistics.median(tim["sample_ms"])

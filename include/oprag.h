@@ -94,7 +94,7 @@ OPRAG_API int oprag_index_get_rows(const oprag_index *idx, int64_t first, int64_
 
 /*
  * Pre-allocates the scratch memory that dense searches of up to q_max queries
- * and k_max results need -- partial lists, the sampled first pass of k > 32,
+ * and k_max results need -- partial lists, the group pass of k > 32,
  * the per-query shared bounds (zeroed here) and, with a sparse side, the
  * lexical block of the hybrid search -- so that later searches of that size
  * allocate nothing and never synchronise the device.  Optional: search calls
@@ -234,8 +234,7 @@ OPRAG_API int oprag_index_update_sparse(oprag_index *idx, const int64_t *ids, in
  * oprag_search).  Order: score descending, then knowledge before memory, then
  * chunk id.  k <= n_knowledge + n_memory.  Asynchronous on `stream`.
  * bf16 indices: one launch of the search kernel scans the knowledge rows
- * followed by the memory rows (plus its sampled first pass when k > 32 over
- * many tiles) and one merge writes the result, using the knowledge index's
+ * followed by the memory rows (plus its group pass when k > 32) and one merge writes the result, using the knowledge index's
  * scratch; fp32 indices: a search per index and a merge of the two lists.
  */
 OPRAG_API int oprag_search_two(oprag_index *knowledge, oprag_index *memory, const void *queries,
@@ -283,7 +282,7 @@ OPRAG_API int oprag_index_set_option(oprag_index *idx, int32_t option, int32_t v
 #define OPRAG_OPT_GRAPH 6
 
 /* OPRAG_OPT_TIMING: 1 makes every later search record CUDA events, on the
- * call's stream, around its lexical (BM25) kernel, its sampled first pass,
+ * call's stream, around its lexical (BM25) kernel, its group pass,
  * its main search kernel and its merge kernel; oprag_index_last_timing()
  * reads them.  0 (default) off. */
 #define OPRAG_OPT_TIMING 3
@@ -332,8 +331,8 @@ OPRAG_API int oprag_index_last_phases(oprag_index *idx, int64_t *out, int32_t ca
 /*
  * Device durations (milliseconds) of the kernels of the last search issued
  * with timing on: lexical_ms (BM25 pass of a hybrid search, 0 for a dense
- * search), sample_ms (the first pass over every 32nd corpus tile and its
- * merge that a search with k > 32 over a large corpus runs first, else 0),
+ * search), sample_ms (the group pass over all or some of the corpus tiles, and
+ * its selection, that a tensor-core search with k > 32 runs first, else 0),
  * search_ms (main pass: score contraction + fused selection), merge_ms
  * (final top-k reduction).  Waits for that search to finish.  Any
  * out-pointer may be NULL.  OPRAG_ERR_NOT_READY if no timed search was issued.
@@ -342,7 +341,7 @@ OPRAG_API int oprag_index_last_timing(oprag_index *idx, float *lexical_ms, float
                                       float *search_ms, float *merge_ms);
 
 /* Bytes currently held by the index's grow-on-demand buffers: the search
- * scratch (partial lists, sampled pass), the shared per-query k-th bounds
+ * scratch (partial lists, group pass), the shared per-query k-th bounds
  * and the lexical block of the hybrid search.  Any out-pointer may be NULL.
  * For tests of oprag_index_reserve. */
 OPRAG_API int oprag_index_buffer_bytes(const oprag_index *idx, int64_t *scratch, int64_t *bounds,
@@ -388,17 +387,17 @@ OPRAG_API int oprag_plan_search(int64_t n, int32_t d, int32_t q, int32_t k, int3
  * synchronisation that cudaMalloc / cudaFree may cause.
  *
  * Same arguments, results and stream semantics as oprag_search, and the same
- * kernels (including the sampled first pass of k > 32 over a large corpus).
+ * kernels (including the group pass of k > 32, unless its maxima are what does
+ * not fit below).
  * Instead of the index's scratch buffer (which oprag_search grows with
- * cudaMalloc), the partial top-k lists, the sampled pass and the per-query
+ * cudaMalloc), the partial top-k lists, the group pass and the per-query
  * shared bounds live in one statically sized device array of 16 MiB that the
  * library holds on every GPU that loads it until the process exits.
  *   - A search that needs more than 16 MiB is refused with
  *     OPRAG_ERR_INVALID_ARG and a message giving the required size; nothing
  *     is launched.  That covers k > 32 over thousands of queries and, since
  *     every CTA then keeps a 128-row list of 256 keys (256 KiB), k > 32 over
- *     a corpus of 128 or more tiles of 128 chunks: the searches for which
- *     oprag_search runs its sampled first pass.
+ *     a corpus of 128 or more tiles of 128 chunks.
  *   - The first call on a device resolves the array's device address (a
  *     runtime query, no allocation) and keeps it for the process; make that
  *     first call before any stream capture.  A cudaDeviceReset invalidates

@@ -110,7 +110,13 @@ struct SearchShape {
   // The lexical part is gathered in the tensor-core epilogue: the plan uses
   // single CTAs with 128-row corpus tiles and one epilogue set.
   bool fused_lex = false;
+  // Group pass of a search with buffered lists: no lists, the maxima of groups
+  // of `group` (8 or 32) scores instead (0: an ordinary search).
+  int group = 0;
 };
+
+// Kept-list length of a pass (0: group pass).
+inline int list_len_of(const SearchShape& s) { return s.group > 0 ? 0 : list_len_for(s.k); }
 
 // --- SIMT streaming search (bf16, on request; any q, meant for small q).
 size_t simt_scratch_bytes(const SearchShape& s, int grid);
@@ -178,10 +184,17 @@ cudaError_t launch_tc_search(const void* E, const void* Q, const SearchShape& s,
                              const void* E2 = nullptr);
 constexpr int kTcPhases = 8;
 
+// Group pass: a search launch whose scratch receives, instead of lists, the
+// group maxima (q rows of tc_group_count floats, see TcParams::gmax).
+int64_t tc_group_count(const SearchShape& s, const TcPlan& p);
+// Per query, the k-th largest of its group maxima (-inf with fewer groups) into
+// kth, and (levels != nullptr) those at ranks level_rank(k, i) with zeroed
+// counters; at most kSelectMaxGroups groups.
+constexpr int kSelectMaxGroups = 4096;
+cudaError_t launch_group_select(const float* gmax, int64_t gld, int groups, int q, int k,
+                                float* kth, float* levels, int* level_cnt, cudaStream_t st);
+
 // --- final merge of partial lists into the sorted top-k per query.
-// kth_out (optional, q floats): the k-th best merged score of every query
-// (-inf when fewer than k candidates exist).  levels_out (optional, q x
-// kLevels floats): the merged scores at ranks level_rank(k, i).
 constexpr int kLevels = 4;
 // Ranks k/16, k/8, k/4, k/2 (at least 1): candidate floors for a search of
 // k > 32 that a first pass over a sample of the corpus tiles proposes.
@@ -190,7 +203,7 @@ inline __host__ __device__ int level_rank(int k, int i) {
   return r < 1 ? 1 : r;
 }
 cudaError_t launch_merge(const ListSet& ls, int q, int k, int64_t* out_ids, float* out_scores,
-                         cudaStream_t st, float* kth_out = nullptr, float* levels_out = nullptr);
+                         cudaStream_t st);
 
 // Two ranked lists per query (a: q x ka, b: q x kb, each sorted score
 // descending then id ascending) into the top-k of both, score descending,

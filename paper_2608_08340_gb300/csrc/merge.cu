@@ -4,9 +4,8 @@
 // local candidates to the global top-k, done inside one GPU: the producers
 // are corpus slices instead of index shards.
 //
-// Four merges: for unsorted lists (buffered tensor-core lists, k > 32) and
-// for sorted lists of at most 32 keys merged into k > 32, one warp per query
-// over all their keys; otherwise for sorted lists, by list count and k, one
+// Four merges: for unsorted lists (buffered tensor-core lists, k > 32) one warp
+// per query over all their keys; otherwise for sorted lists, by list count and k, one
 // warp per query over at most 32 lists (head by head), one to four warps per
 // query over up to 512 lists when k <= 16 (also head by head), and the block
 // merge of merge.cuh (one CTA per query).
@@ -21,20 +20,18 @@ constexpr int kMergeWarps = 8;
 template <int KP>
 __global__ void __launch_bounds__(kMergeWarps * 32)
 merge_kernel(ListSet ls, int q, int k, int64_t* __restrict__ out_ids,
-             float* __restrict__ out_scores, float* __restrict__ kth_out,
-             float* __restrict__ levels_out) {
+             float* __restrict__ out_scores) {
   extern __shared__ __align__(16) uint64_t smem_keys[];
   // Launched as a programmatic dependent of the search kernel: wait until
   // that grid has finished and its lists are visible.
   asm volatile("griddepcontrol.wait;" ::: "memory");
   const int qi = blockIdx.x;
   if (qi >= q) return;
-  merge_one_query<KP>(ls, qi, k, kMergeWarps, out_ids, out_scores, kth_out, levels_out, smem_keys);
+  merge_one_query<KP>(ls, qi, k, kMergeWarps, out_ids, out_scores, smem_keys);
 }
 
 template <int KP>
-cudaError_t launch_merge_kp(const ListSet& ls, int q, int k, int64_t* ids, float* scores,
-                            cudaStream_t st, float* kth_out, float* levels_out) {
+cudaError_t launch_merge_kp(const ListSet& ls, int q, int k, int64_t* ids, float* scores, cudaStream_t st) {
   const size_t smem = static_cast<size_t>(kMergeWarps + 1) * 2 * KP * sizeof(uint64_t);
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3(q);
@@ -46,7 +43,7 @@ cudaError_t launch_merge_kp(const ListSet& ls, int q, int k, int64_t* ids, float
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, merge_kernel<KP>, ls, q, k, ids, scores, kth_out, levels_out);
+  return cudaLaunchKernelEx(&cfg, merge_kernel<KP>, ls, q, k, ids, scores);
 }
 
 // Few lists per query (at most 32): one warp per query merges the sorted
@@ -60,8 +57,7 @@ constexpr int kWayWarps = 2;        // queries per CTA
 
 __global__ void __launch_bounds__(kWayWarps * 32, 16)
 merge_kway_kernel(ListSet ls, int q, int k, int64_t* __restrict__ out_ids,
-                  float* __restrict__ out_scores, float* __restrict__ kth_out,
-                  float* __restrict__ levels_out) {
+                  float* __restrict__ out_scores) {
   asm volatile("griddepcontrol.wait;" ::: "memory");
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int qi = blockIdx.x * kWayWarps + warp;
@@ -105,11 +101,6 @@ merge_kway_kernel(ListSet ls, int q, int k, int64_t* __restrict__ out_ids,
         store_result(ls, out_ids, out_scores, o, mine);
       }
     }
-    if (r == k - 1 && kth_out != nullptr && lane == 0)
-      kth_out[qi] = best == kEmptyKey ? -INFINITY : key_score(best);
-    if (levels_out != nullptr && lane < kLevels && r == level_rank(k, lane) - 1)
-      levels_out[static_cast<int64_t>(qi) * kLevels + lane] =
-          best == kEmptyKey ? -INFINITY : key_score(best);
   }
 }
 
@@ -133,8 +124,7 @@ constexpr int kSmallKeys = 6;
 template <int W>
 __global__ void __launch_bounds__(kSmallThreads, 4)
 merge_small_kernel(ListSet ls, int q, int k, int64_t* __restrict__ out_ids,
-                   float* __restrict__ out_scores, float* __restrict__ kth_out,
-                   float* __restrict__ levels_out) {
+                   float* __restrict__ out_scores) {
   constexpr int kQPerCta = kSmallThreads / 32 / W;
   __shared__ uint64_t heads[2][kSmallThreads / 32];
   asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -203,16 +193,10 @@ merge_small_kernel(ListSet ls, int q, int k, int64_t* __restrict__ out_ids,
         store_result(ls, out_ids, out_scores, o, mine);
       }
     }
-    if (r == k - 1 && kth_out != nullptr && lane == 0)
-      kth_out[qi] = best == kEmptyKey ? -INFINITY : key_score(best);
-    if (levels_out != nullptr && lane < kLevels && r == level_rank(k, lane) - 1)
-      levels_out[static_cast<int64_t>(qi) * kLevels + lane] =
-          best == kEmptyKey ? -INFINITY : key_score(best);
   }
 }
 
-// Unsorted lists (ListSet::counts), k > 32, and short sorted lists merged
-// into k > 32 (read whole, as if unsorted): one warp per query.  The warp
+// Unsorted lists (ListSet::counts), k > 32: one warp per query.  The warp
 // scans the query's list counts into offsets in shared memory, reads the
 // concatenated keys 32 x kUnsortedLoads at a time (a lane's keys come in
 // increasing order, so it finds each key's list by moving a cursor forward
@@ -234,8 +218,7 @@ size_t unsorted_smem_bytes(int P) {
 template <int KP>
 __global__ void __launch_bounds__(kUnsortedWarps * 32)
 merge_unsorted_kernel(ListSet ls, int q, int k, int64_t* __restrict__ out_ids,
-                      float* __restrict__ out_scores, float* __restrict__ kth_out,
-                      float* __restrict__ levels_out) {
+                      float* __restrict__ out_scores) {
   extern __shared__ __align__(16) uint64_t smem_u[];
   asm volatile("griddepcontrol.wait;" ::: "memory");
   constexpr int kCap = 2 * KP;
@@ -246,10 +229,7 @@ merge_unsorted_kernel(ListSet ls, int q, int k, int64_t* __restrict__ out_ids,
   const int np = merge_list_count(ls, tile);
   const int offs_len = (ls.P + 4) / 4 * 4;
   int* offs = reinterpret_cast<int*>(smem_u + kUnsortedWarps * kCap) + warp * offs_len;
-  const int* cnt = ls.counts != nullptr
-                       ? ls.counts + static_cast<int64_t>(tile) * ls.P * ls.TH + row
-                       : nullptr;
-  const int fixed = min(ls.klen, ls.stride);     // keys of a sorted list
+  const int* cnt = ls.counts + static_cast<int64_t>(tile) * ls.P * ls.TH + row;
   const uint64_t* base = ls.keys + (static_cast<int64_t>(tile) * ls.P * ls.TH + row) * ls.stride;
   const int64_t list_step = static_cast<int64_t>(ls.TH) * ls.stride;
 
@@ -257,9 +237,7 @@ merge_unsorted_kernel(ListSet ls, int q, int k, int64_t* __restrict__ out_ids,
   int total = 0;
   for (int p0 = 0; p0 < np; p0 += 32) {
     const int p = p0 + lane;
-    const int c = p >= np          ? 0
-                  : cnt == nullptr ? fixed
-                                   : max(0, min(cnt[static_cast<int64_t>(p) * ls.TH], ls.stride));
+    const int c = p < np ? max(0, min(cnt[static_cast<int64_t>(p) * ls.TH], ls.stride)) : 0;
     int incl = c;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
@@ -294,22 +272,12 @@ merge_unsorted_kernel(ListSet ls, int q, int k, int64_t* __restrict__ out_ids,
       if (g + u * 32 < total) merge_offer32(m, key[u]);
   }
   m.finish();
-  if (kth_out != nullptr && lane == 0) {
-    const uint64_t kk = m.sbuf[k - 1];
-    kth_out[qi] = kk == kEmptyKey ? -INFINITY : key_score(kk);
-  }
-  if (levels_out != nullptr && lane < kLevels) {
-    const uint64_t kk = m.sbuf[level_rank(k, lane) - 1];
-    levels_out[static_cast<int64_t>(qi) * kLevels + lane] =
-        kk == kEmptyKey ? -INFINITY : key_score(kk);
-  }
   for (int i = lane; i < k; i += 32)
     store_result(ls, out_ids, out_scores, static_cast<int64_t>(qi) * k + i, m.sbuf[i]);
 }
 
 template <int KP>
-cudaError_t launch_unsorted_kp(const ListSet& ls, int q, int k, int64_t* ids, float* scores,
-                               cudaStream_t st, float* kth_out, float* levels_out) {
+cudaError_t launch_unsorted_kp(const ListSet& ls, int q, int k, int64_t* ids, float* scores, cudaStream_t st) {
   const size_t smem = unsorted_smem_bytes<KP>(ls.P);
   if (smem > 48 * 1024) {
     const cudaError_t e =
@@ -327,14 +295,12 @@ cudaError_t launch_unsorted_kp(const ListSet& ls, int q, int k, int64_t* ids, fl
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, merge_unsorted_kernel<KP>, ls, q, k, ids, scores, kth_out,
-                            levels_out);
+  return cudaLaunchKernelEx(&cfg, merge_unsorted_kernel<KP>, ls, q, k, ids, scores);
 }
 
 template <typename Kern>
 cudaError_t launch_warp_per_query(Kern kern, int warps, const ListSet& ls, int q, int k,
-                                  int64_t* out_ids, float* out_scores, cudaStream_t st,
-                                  float* kth_out, float* levels_out) {
+                                  int64_t* out_ids, float* out_scores, cudaStream_t st) {
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3((q + warps - 1) / warps);
   cfg.blockDim = dim3(warps * 32);
@@ -345,12 +311,11 @@ cudaError_t launch_warp_per_query(Kern kern, int warps, const ListSet& ls, int q
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kern, ls, q, k, out_ids, out_scores, kth_out, levels_out);
+  return cudaLaunchKernelEx(&cfg, kern, ls, q, k, out_ids, out_scores);
 }
 
 template <int W>
-cudaError_t launch_small_w(const ListSet& ls, int q, int k, int64_t* out_ids, float* out_scores,
-                           cudaStream_t st, float* kth_out, float* levels_out) {
+cudaError_t launch_small_w(const ListSet& ls, int q, int k, int64_t* out_ids, float* out_scores, cudaStream_t st) {
   constexpr int kQPerCta = kSmallThreads / 32 / W;
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3((q + kQPerCta - 1) / kQPerCta);
@@ -362,8 +327,7 @@ cudaError_t launch_small_w(const ListSet& ls, int q, int k, int64_t* out_ids, fl
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, merge_small_kernel<W>, ls, q, k, out_ids, out_scores, kth_out,
-                            levels_out);
+  return cudaLaunchKernelEx(&cfg, merge_small_kernel<W>, ls, q, k, out_ids, out_scores);
 }
 
 // Warps per query of merge_small_kernel: the fewest whose lanes hold all of
@@ -371,14 +335,13 @@ cudaError_t launch_small_w(const ListSet& ls, int q, int k, int64_t* out_ids, fl
 // whatever W is, and with one warp per query the head-by-head rounds need no
 // barrier.  Returns cudaErrorNotSupported when four warps do not suffice (the
 // caller then takes the block merge).
-cudaError_t launch_small(const ListSet& ls, int q, int k, int64_t* out_ids, float* out_scores,
-                         cudaStream_t st, float* kth_out, float* levels_out) {
+cudaError_t launch_small(const ListSet& ls, int q, int k, int64_t* out_ids, float* out_scores, cudaStream_t st) {
   constexpr int kPerWarp = kSmallLists * 32;
   const int W = ls.P <= kPerWarp ? 1 : ls.P <= 2 * kPerWarp ? 2 : 4;
   if (ls.P > W * kPerWarp) return cudaErrorNotSupported;
-  if (W == 4) return launch_small_w<4>(ls, q, k, out_ids, out_scores, st, kth_out, levels_out);
-  if (W == 2) return launch_small_w<2>(ls, q, k, out_ids, out_scores, st, kth_out, levels_out);
-  return launch_small_w<1>(ls, q, k, out_ids, out_scores, st, kth_out, levels_out);
+  if (W == 4) return launch_small_w<4>(ls, q, k, out_ids, out_scores, st);
+  if (W == 2) return launch_small_w<2>(ls, q, k, out_ids, out_scores, st);
+  return launch_small_w<1>(ls, q, k, out_ids, out_scores, st);
 }
 
 }  // namespace
@@ -435,29 +398,25 @@ cudaError_t launch_merge_two(int q, const int64_t* a_ids, const float* a_sc, int
   return cudaGetLastError();
 }
 
-cudaError_t launch_merge(const ListSet& ls, int q, int k, int64_t* out_ids, float* out_scores,
-                         cudaStream_t st, float* kth_out, float* levels_out) {
+cudaError_t launch_merge(const ListSet& ls, int q, int k, int64_t* out_ids, float* out_scores, cudaStream_t st) {
   if (q <= 0) return cudaSuccess;
-  // Unsorted lists, or sorted lists of at most 32 keys merged into more
-  // (the sampled first pass of a search with k > 32): one sort per query
-  // instead of k head-by-head rounds.
-  if (ls.counts != nullptr || (k > 32 && ls.klen <= 32 && ls.stride <= 32)) {
-    if (k <= 64) return launch_unsorted_kp<64>(ls, q, k, out_ids, out_scores, st, kth_out, levels_out);
+  // Unsorted lists: one sort per query instead of k head-by-head rounds.
+  if (ls.counts != nullptr) {
+    if (k <= 64) return launch_unsorted_kp<64>(ls, q, k, out_ids, out_scores, st);
     if (k <= 128)
-      return launch_unsorted_kp<128>(ls, q, k, out_ids, out_scores, st, kth_out, levels_out);
-    return launch_unsorted_kp<256>(ls, q, k, out_ids, out_scores, st, kth_out, levels_out);
+      return launch_unsorted_kp<128>(ls, q, k, out_ids, out_scores, st);
+    return launch_unsorted_kp<256>(ls, q, k, out_ids, out_scores, st);
   }
   if (ls.P <= 32)
-    return launch_warp_per_query(merge_kway_kernel, kWayWarps, ls, q, k, out_ids, out_scores, st,
-                                 kth_out, levels_out);
+    return launch_warp_per_query(merge_kway_kernel, kWayWarps, ls, q, k, out_ids, out_scores, st);
   if (k <= 16) {
-    const cudaError_t e = launch_small(ls, q, k, out_ids, out_scores, st, kth_out, levels_out);
+    const cudaError_t e = launch_small(ls, q, k, out_ids, out_scores, st);
     if (e != cudaErrorNotSupported) return e;
   }
-  if (k <= 32) return launch_merge_kp<32>(ls, q, k, out_ids, out_scores, st, kth_out, levels_out);
-  if (k <= 64) return launch_merge_kp<64>(ls, q, k, out_ids, out_scores, st, kth_out, levels_out);
-  if (k <= 128) return launch_merge_kp<128>(ls, q, k, out_ids, out_scores, st, kth_out, levels_out);
-  return launch_merge_kp<256>(ls, q, k, out_ids, out_scores, st, kth_out, levels_out);
+  if (k <= 32) return launch_merge_kp<32>(ls, q, k, out_ids, out_scores, st);
+  if (k <= 64) return launch_merge_kp<64>(ls, q, k, out_ids, out_scores, st);
+  if (k <= 128) return launch_merge_kp<128>(ls, q, k, out_ids, out_scores, st);
+  return launch_merge_kp<256>(ls, q, k, out_ids, out_scores, st);
 }
 
 }  // namespace oprag

@@ -81,7 +81,6 @@ __device__ __forceinline__ uint64_t merge_floor_key(const ListSet& ls, int qi, i
 template <int KP>
 __device__ __forceinline__ void merge_one_query(const ListSet& ls, int qi, int k, int nw,
                                 int64_t* __restrict__ out_ids, float* __restrict__ out_scores,
-                                float* __restrict__ kth_out, float* __restrict__ levels_out,
                                 uint64_t* smem_keys) {
   constexpr int kCap = 2 * KP;
   constexpr int kUnroll = 4;
@@ -132,15 +131,6 @@ __device__ __forceinline__ void merge_one_query(const ListSet& ls, int qi, int k
       for (int u = 0; u < kUnroll; ++u) merge_offer32(f, key[u]);
     }
     f.finish();
-    if (kth_out != nullptr && lane == 0) {
-      const uint64_t kk = f.sbuf[k - 1];
-      kth_out[qi] = kk == kEmptyKey ? -INFINITY : key_score(kk);
-    }
-    if (levels_out != nullptr && lane < kLevels) {
-      const uint64_t kk = f.sbuf[level_rank(k, lane) - 1];
-      levels_out[static_cast<int64_t>(qi) * kLevels + lane] =
-          kk == kEmptyKey ? -INFINITY : key_score(kk);
-    }
     for (int i = lane; i < k; i += 32) {
       const uint64_t key = f.sbuf[i];
       const int64_t o = static_cast<int64_t>(qi) * k + i;

@@ -135,9 +135,9 @@ struct oprag_index {
   bool timing = false;
   bool timed = false;      // the last search recorded its events
   bool timed_lex = false;  // ... including a lexical pass
-  bool timed_sample = false;  // ... including a sampled first pass
+  bool timed_sample = false;  // ... including a group pass
   // ev[0] before the lexical pass, ev[1] before the search passes, ev[4]
-  // before the main search pass (after the sampled first pass, if any),
+  // before the main search pass (after the group pass, if any),
   // ev[2] before the merge, ev[3] after it.
   cudaEvent_t ev[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};
   // Spin limit (cycles) of the search kernels' mbarrier waits; 0 = default.
@@ -266,32 +266,39 @@ int choose_path(const oprag_index* idx, int q) {
 }
 
 // Scratch of one search, in one block: the main pass's partial lists and,
-// for buffered lists (k > 32) over many corpus tiles, a first pass over every
-// kSampleStride-th corpus tile (its lists, its merged top-k, and per query the
-// k-th score, kLevels counted floors and their counters).  Register lists
-// (k <= 32) also use one 64-bit shared bound per query, kept outside the block.
-#ifndef OPRAG_SAMPLE_STRIDE
-#define OPRAG_SAMPLE_STRIDE 32
-#endif
-constexpr int kSampleStride = OPRAG_SAMPLE_STRIDE;
-// Corpus tiles from which a search with buffered lists runs the first pass.
-constexpr int kSampleMinTiles = 128;
-// Every 32nd corpus tile, lists of 8 keys (two epilogue sets, the cheapest
-// insertions).  Any k-th best of real candidates is a valid floor.  Measured
-// on 1M x 768 with 2048 queries and k = 100: with stride 16, lists of 32 / 16
-// / 8 keys gave a first pass of 395 / 264 / 218 us and the same main pass
-// (2194 us); with lists of 8, strides 8 / 16 / 32 gave steps of 2636 / 2534 /
-// 2470 us (first pass 357 / 220 / 141 us, main pass 2226 / 2256 / 2275 us).
-#ifndef OPRAG_SAMPLE_K
-#define OPRAG_SAMPLE_K 8
-#endif
-constexpr int kSampleK = OPRAG_SAMPLE_K;
+// for buffered lists (k > 32), a group pass over every group_stride-th corpus
+// tile (its group maxima, and per query the floor, kLevels counted floors and
+// their counters).  Register lists (k <= 32) also use one 64-bit shared bound
+// per query, kept outside the block.
+
+// Corpus tiles skipped by the group pass.  Its floor lets about
+// 1.1 k group_stride scores per query into the main pass, so a stride of
+// n / (256 k) lets in about one score in 250 and keeps the main pass's
+// insertions small next to its products; from 32 on the group pass costs too
+// little to thin it further (and a longer stride only where the maxima would
+// not fit the selection kernel).  Measured on GB300 against the first pass it
+// replaced (8-key lists over every 32nd tile, merged, only from 128 tiles on):
+// 32768 x 768, 1024 queries, k = 128 (stride 1) first pass 41 -> 52 us, main
+// pass 508 -> 50 us, merge 64 -> 16 us; 50021 x 392, 300 queries, k = 50
+// (stride 3) 26 -> 28, 41 -> 36 and 25 -> 16 us; 1M x 768, 2048 queries,
+// k = 100 (stride 32) 121 -> 91, 1953 -> 1887 and 41 -> 41 us.
+constexpr int kGroupMaxStride = 32;
+// Counted floors are worth their counting only when the group pass's ranks
+// reach well below rank k of the corpus.
+constexpr int kLevelsMinStride = 4;
+
+int group_stride(int64_t n, int k) {
+  constexpr int64_t kRows = 32 * 4000;      // rows whose groups of 32 fit the selection
+  const int64_t s = std::min<int64_t>(kGroupMaxStride, n / (256 * k));
+  return static_cast<int>(std::max<int64_t>({1, s, (n + kRows - 1) / kRows}));
+}
 
 struct SearchLayout {
   int path = 0;           // 1 SIMT, 2 tensor core
   int simt_grid = 0;      // CTAs (bf16) or corpus slices (fp32) of path 1
   TcPlan plan{}, splan{};
-  bool sampled = false;
+  bool sampled = false;     // a group pass runs first
+  SearchShape gshape{};     // its shape
   size_t main_bytes = 0;    // multiple of 256
   size_t sample_bytes = 0;  // 0 unless sampled
   bool floors = false;      // q shared bounds (fp32, and register lists on the tensor-core path)
@@ -321,19 +328,21 @@ SearchLayout search_layout(oprag_index* idx, int q, int k, int path, int block_n
   L.plan = tc_plan(s, idx->num_sms, block_n, 1, pair, pair_capacity(idx));
   L.main_bytes = round256(tc_scratch_bytes(s, L.plan));
   // Buffered lists collect every score above their floor, and the floor of a
-  // fresh list starts at -inf.  A cheap first pass over every
-  // kSampleStride-th corpus tile with kSampleK-key lists yields, per query, the
-  // k-th best of real corpus scores -- a lower bound of the true k-th best --
-  // which the main pass then uses as the lists' starting floor.
-  L.sampled = list_len_for(k) > 32 && L.plan.nt >= kSampleMinTiles;
+  // fresh list starts at -inf.  A group pass over every group_stride-th corpus
+  // tile keeps only the maxima of groups of 32 scores (8 when 32 would leave
+  // fewer than 4 k groups); the k-th largest of them is a lower bound of the
+  // query's k-th best score, with which the main pass's lists start.
+  L.sampled = list_len_for(k) > 32;
   if (L.sampled) {
-    SearchShape s32 = s;
-    s32.k = kSampleK;
-    L.splan = tc_plan(s32, idx->num_sms, L.plan.block_n, kSampleStride, L.plan.pair,
-                      pair_capacity(idx));
+    L.gshape = s;
+    L.gshape.group = 32;
+    const int stride = group_stride(s.n + s.n_second, k);
+    const int gbn = L.plan.pair == 2 ? L.plan.block_n : block_n;
+    const int gpair = L.plan.pair == 2 ? 2 : pair;
+    L.splan = tc_plan(L.gshape, idx->num_sms, gbn, stride, gpair, pair_capacity(idx));
+    if (tc_group_count(L.gshape, L.splan) < 4 * k) L.gshape.group = 8;
     const size_t per_query_tail = sizeof(float) + kLevels * (sizeof(float) + sizeof(int));
-    L.sample_bytes = round256(tc_scratch_bytes(s32, L.splan)) +
-                     round256(static_cast<size_t>(q) * k * 12) +
+    L.sample_bytes = round256(tc_scratch_bytes(L.gshape, L.splan)) +
                      static_cast<size_t>(q) * per_query_tail + 16;
   }
   L.floors = list_len_for(k) <= 32;
@@ -370,23 +379,21 @@ int launch_search(oprag_index* idx, const SearchLayout& L, const void* Q, int q,
     float* levels = nullptr;
     int* level_cnt = nullptr;
     if (L.sampled) {
-      SearchShape s32 = s;
-      s32.k = kSampleK;
       char* sbase = static_cast<char*>(scratch) + L.main_bytes;
-      const size_t slist = round256(tc_scratch_bytes(s32, L.splan));
-      int64_t* sids = reinterpret_cast<int64_t*>(sbase + slist);
-      float* sscores = reinterpret_cast<float*>(sids + static_cast<size_t>(q) * k);
-      float* kth = reinterpret_cast<float*>(sbase + slist + round256(static_cast<size_t>(q) * k * 12));
-      // 16-byte aligned: each query's kLevels counters are read as one int4.
-      levels = kth + (static_cast<size_t>(q) + 3) / 4 * 4;
-      level_cnt = reinterpret_cast<int*>(levels + static_cast<size_t>(q) * kLevels);
-      ListSet slists{};
-      e = launch_tc_search(idx->emb, Q, s32, fu, L.splan, sbase, idx->dev_err, &slists, st,
+      float* kth = reinterpret_cast<float*>(sbase + round256(tc_scratch_bytes(L.gshape, L.splan)));
+      if (L.splan.tile_stride >= kLevelsMinStride) {
+        // 16-byte aligned: each query's kLevels counters are read as one int4.
+        levels = kth + (static_cast<size_t>(q) + 3) / 4 * 4;
+        level_cnt = reinterpret_cast<int*>(levels + static_cast<size_t>(q) * kLevels);
+      }
+      ListSet none{};
+      e = launch_tc_search(idx->emb, Q, L.gshape, fu, L.splan, sbase, idx->dev_err, &none, st,
                            nullptr, nullptr, 0, nullptr, nullptr, idx->wait_limit, nullptr, E2);
-      if (e == cudaSuccess) e = launch_merge(slists, q, k, sids, sscores, st, kth, levels);
+      const int64_t groups = tc_group_count(L.gshape, L.splan);
       if (e == cudaSuccess)
-        e = cudaMemsetAsync(level_cnt, 0, static_cast<size_t>(q) * kLevels * sizeof(int), st);
-      if (e != cudaSuccess) return cuda_fail(e, "sampling pass");
+        e = launch_group_select(reinterpret_cast<const float*>(sbase), groups,
+                                static_cast<int>(groups), q, k, kth, levels, level_cnt, st);
+      if (e != cudaSuccess) return cuda_fail(e, "group pass");
       floor = kth;
     }
     if (idx->timed_sample) cudaEventRecord(idx->ev[4], st);
@@ -1583,10 +1590,15 @@ extern "C" int oprag_search_noalloc(oprag_index* idx, const void* queries, int32
   void* scratch = nullptr;
   if ((rc = static_scratch(idx->device, &scratch))) return rc;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  // The same passes as oprag_search (with the sampled first pass for k > 32
-  // over many corpus tiles); its shared per-query bounds sit after the lists
-  // and are cleared on every call, since the array is shared by all indexes.
-  const SearchLayout L = search_layout(idx, q, k);
+  // The same passes as oprag_search; its shared per-query bounds sit after
+  // the lists and are cleared on every call, since the array is shared by all
+  // indexes.  Lists that fit the array only without the group pass of k > 32
+  // go without it (same results, more candidates).
+  SearchLayout L = search_layout(idx, q, k);
+  if (L.total() > kStaticScratchBytes && L.main_bytes <= kStaticScratchBytes) {
+    L.sampled = false;
+    L.sample_bytes = 0;
+  }
   const size_t floors = L.floors ? static_cast<size_t>(q) * sizeof(uint64_t) : 0;
   const size_t need = round256(L.total()) + floors;
   if (need > kStaticScratchBytes)

@@ -47,7 +47,7 @@ TcPlan tc_plan(const SearchShape& s, int num_sms, int force_block_n, int tile_st
   // CTA (small batches, where the copies into the SMs, not the MMAs, bound
   // the kernel; measured on 32768 x 768: faster up to 512 queries, slower at
   // 1024); it needs the two epilogue sets of lists of 8 or 16.
-  const bool dual_ok = !s.fused_lex && pl.qt >= 2 && list_len_for(s.k) <= 16 &&
+  const bool dual_ok = !s.fused_lex && pl.qt >= 2 && list_len_of(s) <= 16 &&
                        force_pair != 2 && (force_block_n == 0 || force_block_n == 128);
   const int64_t dual_units =
       static_cast<int64_t>((pl.qt + 1) / 2) * ((s.n + 127) / 128 + (s.n_second + 127) / 128);
@@ -62,7 +62,7 @@ TcPlan tc_plan(const SearchShape& s, int num_sms, int force_block_n, int tile_st
   // (32768 x 1024, 4096 queries, k = 10) pairs are no faster.
   const bool pair = !s.fused_lex && bn == 256 && pair_capacity > 0 &&
                     (force_pair == 2 ||
-                     (force_pair == 0 && list_len_for(s.k) > 32 && pl.qt >= 8));
+                     (force_pair == 0 && list_len_of(s) > 32 && pl.qt >= 8));
   pl.pair = pair ? 2 : 1;
   pl.uqt = pair || pl.dual ? (pl.qt + 1) / 2 : pl.qt;
   pl.tile_stride = tile_stride < 1 ? 1 : tile_stride;
@@ -106,9 +106,9 @@ TcPlan tc_plan(const SearchShape& s, int num_sms, int force_block_n, int tile_st
   for (int j = 0; j < pl.uqt; ++j)
     per_tile = std::max(per_tile, hi[j] - first_cta(j, pl.uqt, C) + 1);
   if (!ok) per_tile = C;  // not expected; every slot then gets a list per tile
-  pl.sets = pl.dual ? 1 : epi_sets(list_len_for(s.k), s.fused_lex);
+  pl.sets = pl.dual ? 1 : epi_sets(list_len_of(s), s.fused_lex);
   pl.pmax = per_tile * pl.sets;
-  const int K = list_len_for(s.k);
+  const int K = list_len_of(s);
   // Shared memory of the launch (the same sum as smem_for<BN, K, pair, dual>).
   const size_t b_stage = static_cast<size_t>(pair ? bn / 2 : bn) * 128;
   const size_t a_stage = kAStageBytes * (pl.dual ? 2 : 1);
@@ -128,8 +128,13 @@ static size_t list_rows(const TcPlan& pl) {
   return static_cast<size_t>(pl.uqt) * (pl.pair == 2 || pl.dual ? 2 : 1) * pl.pmax * kBlockM;
 }
 
+int64_t tc_group_count(const SearchShape& s, const TcPlan& pl) {
+  return static_cast<int64_t>(pl.nt) * (pl.block_n / s.group);
+}
+
 size_t tc_scratch_bytes(const SearchShape& s, const TcPlan& pl) {
-  const int K = list_len_for(s.k);
+  const int K = list_len_of(s);
+  if (K == 0) return static_cast<size_t>(s.q) * tc_group_count(s, pl) * sizeof(float);
   const int stride = K > 32 ? 2 * K : K;
   const size_t rows = list_rows(pl);
   size_t bytes = rows * stride * sizeof(uint64_t);
@@ -173,9 +178,9 @@ cudaError_t launch_tc_search(const void* E, const void* Q, const SearchShape& s,
     maps.qb = maps.q;
     maps.eb = maps.e;
   }
-  const int K = list_len_for(s.k);
+  const int K = list_len_of(s);
   const int stride = K > 32 ? 2 * K : K;
-  const size_t rows = list_rows(pl);
+  const size_t rows = K > 0 ? list_rows(pl) : 0;
   TcParams prm{};
   prm.n = s.n + s.n_second;
   prm.n_first = s.n;
@@ -192,6 +197,11 @@ cudaError_t launch_tc_search(const void* E, const void* Q, const SearchShape& s,
   prm.tile_stride = pl.tile_stride;
   prm.init_floor = init_floor;
   prm.fu = fu;
+  if (K == 0) {
+    prm.gmax = static_cast<float*>(scratch);
+    prm.gld = tc_group_count(s, pl);
+    prm.group = s.group;
+  }
   prm.lists = static_cast<uint64_t*>(scratch);
   prm.meta_worst = prm.lists + rows * stride;
   prm.meta_count = reinterpret_cast<int*>(prm.meta_worst + (K > 32 ? rows : 0));

@@ -96,6 +96,11 @@ struct TcParams {
   int* level_cnt;
   // Optional (measurement): kPhases global-timer stamps per CTA (PhaseMark).
   unsigned long long* phases;
+  // Group pass (K == 0): the maxima of groups of `group` (8 or 32) consecutive
+  // scores, gmax[query * gld + group index], in scanned tile order.
+  float* gmax;
+  int64_t gld;
+  int group;
 };
 
 // Points of a CTA's run whose global-timer values a measurement run records
@@ -530,6 +535,13 @@ struct EpiList<K, false> {
   __device__ __forceinline__ float kth(int) const { return t.floor; }
   __device__ __forceinline__ void sync(bool, bool) {}
   __device__ __forceinline__ void read_ahead() {}
+};
+
+// Group pass: no list.
+template <>
+struct EpiList<0, false> {
+  __device__ __forceinline__ void set_k(int) {}
+  __device__ __forceinline__ void clear() {}
 };
 
 template <int K>
@@ -1160,13 +1172,15 @@ tc_search_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     LexCursor lex;             // hybrid: the query's postings cursors
 
     // This CTA owns the list slots (J, cta - first_cta(J)); empty them first.
-    for (int J = 0; J < p.qt; ++J) {
-      const int qi = qtile(J) * kBlockM + row;
-      if (owns(J) && qi < p.q) list.init_mem(p, list_row(J), qi);
+    if constexpr (K > 0) {
+      for (int J = 0; J < p.qt; ++J) {
+        const int qi = qtile(J) * kBlockM + row;
+        if (owns(J) && qi < p.q) list.init_mem(p, list_row(J), qi);
+      }
     }
 
     int cur_j = -1;
-    int64_t cur_sr = 0;
+    int64_t cur_sr = -1;
     bool cur_valid = false;
     uint32_t acc_ph = 0;                     // phase bit per accumulator (bit acc)
     UnitSeq us;
@@ -1186,15 +1200,19 @@ tc_search_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       const bool valid = j * kBlockM + row < p.q;
       const bool warp_live = j * kBlockM + eg * 32 < p.q;
       if (J != cur_j) {
-        if (cur_j >= 0 && cur_valid) list.save(p, cur_sr);
-        if (!owns(J)) {              // cannot happen when the host plan holds
-          atomicExch(p.dev_err, 2);
-          *abort_flag = 1;
-        }
         cur_j = J;
-        cur_sr = list_row(J);
-        cur_valid = valid && owns(J);
-        if (cur_valid) list.load(p, cur_sr); else list.clear();
+        if constexpr (K > 0) {
+          if (cur_sr >= 0 && cur_valid) list.save(p, cur_sr);
+          if (!owns(J)) {              // cannot happen when the host plan holds
+            atomicExch(p.dev_err, 2);
+            *abort_flag = 1;
+          }
+          cur_sr = list_row(J);
+          cur_valid = valid && owns(J);
+          if (cur_valid) list.load(p, cur_sr); else list.clear();
+        } else {
+          cur_valid = valid;
+        }
         if constexpr (K > 32) list.set_query(p, static_cast<int64_t>(j) * kBlockM + row, cur_valid);
         if constexpr (kHybrid) {
           if (cur_valid) lex.set_query(p, static_cast<int64_t>(j) * kBlockM + row);
@@ -1209,7 +1227,8 @@ tc_search_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       }
       // Shared bound of this query's k-th best score, read while the MMAs run.
       float gfl = -INFINITY;
-      if constexpr (K <= 32) {
+      if constexpr (K == 0) {
+      } else if constexpr (K <= 32) {
         if (p.qfloor != nullptr && act)
           gfl = shared_floor_read(p.qfloor, static_cast<int64_t>(j) * kBlockM + row, p.gen);
       } else {
@@ -1346,6 +1365,41 @@ tc_search_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
               if (id0 + i >= id_end) v[i] = -INFINITY;
           }
         };
+        if constexpr (K == 0) {
+          // Group pass: the maxima of the unit's groups of 8 or 32 scores.
+          static_assert(BN / 32 <= 8, "one 32-byte store of group maxima");
+          const int64_t g0 = (t / p.tile_stride) * (BN / p.group);
+          float* dst = p.gmax + (static_cast<int64_t>(j) * kBlockM + row) * p.gld + g0;
+          uint32_t ra[32];
+          float keep[4];
+#pragma unroll 1
+          for (int c = 0; c < BN / 32; ++c) {
+            tmem_ld32_async(taddr + c * 32, ra);
+            tmem_wait_ld(ra);
+            if (!kHybrid && c + 1 == BN / 32) release_acc();
+            float v[32];
+            scores(ra, c, v);
+            float m[4];
+#pragma unroll
+            for (int g = 0; g < 4; ++g)
+              m[g] = fmax3(fmax3(v[8 * g], v[8 * g + 1], v[8 * g + 2]),
+                           fmax3(v[8 * g + 3], v[8 * g + 4], v[8 * g + 5]),
+                           fmaxf(v[8 * g + 6], v[8 * g + 7]));
+            if (p.group == 8) {
+              if (act) *reinterpret_cast<float4*>(dst + 4 * c) = make_float4(m[0], m[1], m[2], m[3]);
+            } else {
+              // four chunks' maxima per 16-byte store
+              const float w = fmax3(fmaxf(m[0], m[1]), m[2], m[3]);
+#pragma unroll
+              for (int i = 0; i < 4; ++i)
+                if ((c & 3) == i) keep[i] = w;
+              if ((c & 3) == 3 && act)
+                *reinterpret_cast<float4*>(dst + (c & ~3)) =
+                    make_float4(keep[0], keep[1], keep[2], keep[3]);
+            }
+            __syncwarp();
+          }
+        } else {
         // Filters one chunk against max(list floor, unit bound).
         auto process = [&](const uint32_t (&r)[32], int c, float bound) {
           float v[32];
@@ -1498,11 +1552,14 @@ tc_search_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
               shared_floor_raise(p.qfloor, static_cast<int64_t>(j) * kBlockM + row, p.gen, pub);
           }
         }
+        }
       }
       if (!released) release_acc();
       acc_ph ^= 1u << acc;
     }
-    if (cur_j >= 0 && cur_valid) list.save(p, cur_sr);
+    if constexpr (K > 0) {
+      if (cur_sr >= 0 && cur_valid) list.save(p, cur_sr);
+    }
     // The set's last warp to finish (the slots start at zero).
     if (p.phases != nullptr && lane == 0)
       atomicMax(p.phases + static_cast<size_t>(blockIdx.x) * kPhases + kPhEpi0Done + set,
@@ -1597,6 +1654,7 @@ cudaError_t launch_dual_variant(const TcMaps& m, const TcParams& prm, int grid, 
 
 template <int BN, int L>
 cudaError_t launch_bn(const TcMaps& m, const TcParams& prm, int grid, cudaStream_t st) {
+  if (prm.gmax != nullptr) return launch_variant<BN, 0, L>(m, prm, grid, st);
   switch (list_len_for(prm.k)) {
     case 8: return launch_variant<BN, 8, L>(m, prm, grid, st);
     case 16: return launch_variant<BN, 16, L>(m, prm, grid, st);
@@ -1608,6 +1666,7 @@ cudaError_t launch_bn(const TcMaps& m, const TcParams& prm, int grid, cudaStream
 
 template <int L>
 cudaError_t launch_pair(const TcMaps& m, const TcParams& prm, int grid, cudaStream_t st) {
+  if (prm.gmax != nullptr) return launch_pair_variant<256, 0, L>(m, prm, grid, st);
   switch (list_len_for(prm.k)) {
     case 8: return launch_pair_variant<256, 8, L>(m, prm, grid, st);
     case 16: return launch_pair_variant<256, 16, L>(m, prm, grid, st);
@@ -1619,6 +1678,7 @@ cudaError_t launch_pair(const TcMaps& m, const TcParams& prm, int grid, cudaStre
 
 template <int L>
 cudaError_t launch_dual(const TcMaps& m, const TcParams& prm, int grid, cudaStream_t st) {
+  if (prm.gmax != nullptr) return launch_dual_variant<0, L>(m, prm, grid, st);
   switch (list_len_for(prm.k)) {
     case 8: return launch_dual_variant<8, L>(m, prm, grid, st);
     case 16: return launch_dual_variant<16, L>(m, prm, grid, st);

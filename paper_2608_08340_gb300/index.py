@@ -221,7 +221,7 @@ class Index:
 
     def last_timing(self) -> dict:
         """Device milliseconds of the last timed search's kernels: lexical pass,
-        sampled first pass (k > 32 over many tiles), main search pass, merge."""
+        group pass and selection (k > 32), main search pass, merge."""
         a, b, c, m = ctypes.c_float(), ctypes.c_float(), ctypes.c_float(), ctypes.c_float()
         check(self._lib.oprag_index_last_timing(self._h, ctypes.byref(a), ctypes.byref(b),
                                                 ctypes.byref(c), ctypes.byref(m)))

@@ -1,0 +1,89 @@
+"""GPU parity of searches with k > 32, whose floors come from a group pass:
+corpora with fewer groups than k, strides 1, 2, 3 and more, groups of 8 and of
+32, every CTA mode, both lexical forms, two stacked corpora, and scores that
+make every group maximum equal."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from oracle import check
+from paper_2608_08340_gb300 import workloads
+from paper_2608_08340_gb300.index import Index, search_two
+
+from _gpu import TOL, check_dense, dev_tensor
+
+pytestmark = pytest.mark.gpu
+
+
+def _rows(rng, n, d):
+    return workloads.to_bf16_bits(workloads._normalise(rng.standard_normal((n, d)).astype(np.float32)))
+
+
+@pytest.mark.parametrize("n,d,q,k,mode", [
+    (40, 64, 3, 40, None),           # 5 groups of 8 for k = 40: no floor
+    (300, 64, 130, 33, None),        # as many groups as k, about
+    (4096, 64, 257, 256, None),      # groups of 8, k = K_MAX
+    (8300, 72, 5, 100, "single"),    # stride 1, groups of 8, ragged last tile
+    (17000, 64, 300, 64, "dual"),    # stride 1, a dual-mode group pass
+    (20000, 64, 1100, 37, None),     # stride 2, CTA pairs
+    (20000, 64, 1100, 37, "single"),
+    (40000, 64, 40, 50, None),       # stride 3
+    (90000, 64, 150, 40, None),      # stride 8: counted floors
+])
+def test_floors(n, d, q, k, mode):
+    rng = np.random.default_rng(n + q + k)
+    E, Q = _rows(rng, n, d), _rows(rng, q, d)
+    idx = Index(dev_tensor(E))
+    idx.force_pair(mode)
+    Qd = dev_tensor(Q)
+    rows = rng.choice(q, min(q, 150), replace=False)
+    for _ in range(2):
+        ids, sc = idx.search(Qd, k)
+        check_dense(ids, sc, E, Q, k, f"n={n} q={q} k={k} {mode}", rows=np.sort(rows))
+    idx.check()
+
+
+@pytest.mark.parametrize("n,k", [(5000, 40), (70000, 100)])
+def test_equal_scores(n, k):
+    """Every score reaches the floor: lists compact, the lowest ids win."""
+    E = oracle.round_bf16(np.ones((n, 64), np.float32))
+    idx = Index(dev_tensor(E))
+    ids, sc = idx.search(dev_tensor(oracle.round_bf16(np.ones((5, 64), np.float32))), k)
+    assert ids.cpu().tolist() == [list(range(k))] * 5
+    assert (sc.cpu().numpy() == 64).all()
+
+
+@pytest.mark.parametrize("gather", [False, True])
+def test_hybrid(gather):
+    w = workloads.config(3, n=9000, batch=70)
+    idx = Index(dev_tensor(w.E_data))
+    idx.set_sparse(w.doc_indptr, w.doc_terms, w.vocab, w.k1, w.b)
+    idx.gather_lexical(gather)
+    k = 60
+    ids, sc = idx.hybrid_search(dev_tensor(w.Q_data), torch.from_numpy(w.q_indptr),
+                                torch.from_numpy(w.q_terms), w.alpha, k)
+    o_ids, o_sc, _ = oracle.hybrid_search(w.E_data, w.Q_data, w.doc_indptr, w.doc_terms, w.vocab,
+                                          w.q_indptr, w.q_terms, w.alpha, k + 200, w.k1, w.b)
+    check.check_topk(ids.cpu().numpy(), sc.cpu().numpy(), o_ids, o_sc, k, TOL, n=w.n,
+                     label=f"hybrid gather={gather}")
+
+
+def test_two_stacked_corpora():
+    rng = np.random.default_rng(3)
+    A, B, Q = _rows(rng, 5001, 64), _rows(rng, 3002, 64), _rows(rng, 200, 64)
+    k = 77
+    ids, src, sc = search_two(Index(dev_tensor(A)), Index(dev_tensor(B)), dev_tensor(Q), k)
+    stacked = ids + 5001 * (src == 1)
+    check_dense(stacked, sc, np.concatenate([A, B]), Q, k, "two")
+
+
+@pytest.mark.parametrize("q,k", [(1, 256), (130, 100), (1500, 40)])
+def test_reserve_covers_the_group_pass(q, k):
+    rng = np.random.default_rng(q)
+    idx = Index(dev_tensor(_rows(rng, 12000, 64)))
+    idx.reserve(q, k)
+    before = idx.buffer_bytes()
+    for kk in {33, k}:
+        idx.search(dev_tensor(_rows(rng, q, 64)), kk)
+    assert idx.buffer_bytes() == before
