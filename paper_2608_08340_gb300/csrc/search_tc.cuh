@@ -914,8 +914,12 @@ tc_search_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
   const int unit_kb = p.kblocks + (kHybrid ? 1 : 0);
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   if (threadIdx.x == 0) note_phase(p, kPhEntry);
-  unsigned char* base = reinterpret_cast<unsigned char*>(
-      (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
+  // Rounded up by an offset, not as an integer: the compiler then still knows
+  // that everything below is shared memory (the epilogue's staging rows were
+  // accessed through generic loads and stores otherwise: 32768 x 1024 with 4096
+  // queries and k = 10 took 203 instead of 195 us, 256 queries on 32768 x 768
+  // 24.9 instead of 23.7 us).
+  unsigned char* base = smem_raw + ((1024 - (smem_addr(smem_raw) & 1023)) & 1023);
   unsigned char* sA = base;
   unsigned char* sB = sA + S * kAStage;
   float* stage_rows = reinterpret_cast<float*>(sB + S * kBStageBytes);   // epilogue staging
