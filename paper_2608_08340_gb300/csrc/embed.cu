@@ -2,11 +2,19 @@
 // padded batch are mean-pooled over its unmasked tokens and L2-normalised,
 // and the vector is written in the index's dtype, ready for oprag_search.
 //
-// One CTA of 256 threads per batch row.  Thread i accumulates, in fp32, the
-// 16-byte groups i, i + 256, ... of the row's dim elements over the tokens,
-// the loads of kTokenBatch tokens in flight at once (a batch has few rows, so
-// each CTA must keep many bytes in flight); a block reduction of the squared
-// mean gives the norm.  HBM-bound: the unmasked hidden states are read once.
+// One CTA of 256 threads per batch row when the rows fill the SMs twice: thread
+// i accumulates, in fp32, the 16-byte groups i, i + 256, ... of the row's dim
+// elements over the tokens, the loads of kTokenBatch tokens in flight at once;
+// a block reduction of the squared mean gives the norm.  HBM-bound: the
+// unmasked hidden states are read once.
+//
+// Smaller batches leave SMs without loads in flight, so a cluster of S CTAs
+// shares a row: CTA r takes the token blocks r, r + S, ... (a padded row's real
+// tokens, which come first, are spread evenly), leaves its partial sums in
+// shared memory and finishes one S-th of the row: it adds the S partial sums,
+// in CTA order, through distributed shared memory, and the squared norms of
+// the parts are exchanged the same way.
+#include <cooperative_groups.h>
 #include <cuda_bf16.h>
 
 #include "common.cuh"
@@ -44,14 +52,20 @@ struct Group<float> {
   }
 };
 
-template <typename TIn, int R>
+template <typename TIn, int R, bool kSplit>
 __global__ void __launch_bounds__(kPoolThreads)
 embed_pool_kernel(const TIn* __restrict__ hidden, int tokens, int dim,
                   const uint8_t* __restrict__ mask, void* __restrict__ out, int out_bf16) {
+  namespace cg = cooperative_groups;
   constexpr int N = Group<TIn>::kN;
+  extern __shared__ __align__(16) float part[];   // this CTA's partial sums (dim)
   __shared__ float red[kPoolThreads / 32];
-  __shared__ float total;
-  const int b = blockIdx.x;
+  __shared__ float part_ss;                       // squared norm of this CTA's part
+  __shared__ int part_count;
+  cg::cluster_group cluster = cg::this_cluster();
+  const int S = kSplit ? static_cast<int>(cluster.num_blocks()) : 1;
+  const int rank = kSplit ? static_cast<int>(cluster.block_rank()) : 0;
+  const int b = blockIdx.x / S;
   const int groups = dim / N;
   const uint4* row0 = reinterpret_cast<const uint4*>(hidden + static_cast<int64_t>(b) * tokens * dim);
   const uint8_t* mrow = mask + static_cast<int64_t>(b) * tokens;
@@ -60,10 +74,10 @@ embed_pool_kernel(const TIn* __restrict__ hidden, int tokens, int dim,
   for (int r = 0; r < R; ++r)
 #pragma unroll
     for (int i = 0; i < N; ++i) acc[r][i] = 0.f;
-  // Tokens are added in increasing order (a fixed summation order).
+  // Tokens are added in increasing order (a fixed summation order for a given S).
   constexpr int TB = R <= 2 ? kTokenBatch : kTokenBatch / 2;   // register budget
   int count = 0;
-  for (int t = 0; t < tokens; t += TB) {
+  for (int t = rank * TB; t < tokens; t += S * TB) {
     bool m[TB];
 #pragma unroll
     for (int u = 0; u < TB; ++u) {
@@ -85,7 +99,45 @@ embed_pool_kernel(const TIn* __restrict__ hidden, int tokens, int dim,
       for (int r = 0; r < R; ++r)
         if (m[u]) Group<TIn>::add(v[u][r], acc[r]);
   }
-  // Mean, then the block-wide sum of its squares.
+  // This CTA's part of the row: groups [g0, g1), its mean and squared norm.
+  int g0 = 0, g1 = groups;
+  if constexpr (kSplit) {
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      const int g = threadIdx.x + r * kPoolThreads;
+      if (g < groups) {
+#pragma unroll
+        for (int i = 0; i < N; i += 4)
+          *reinterpret_cast<float4*>(part + g * N + i) =
+              make_float4(acc[r][i], acc[r][i + 1], acc[r][i + 2], acc[r][i + 3]);
+      }
+    }
+    if (threadIdx.x == 0) part_count = count;
+    cluster.sync();
+    g0 = groups * rank / S;
+    g1 = groups * (rank + 1) / S;
+    count = 0;
+    for (int s = 0; s < S; ++s) count += *cluster.map_shared_rank(&part_count, s);
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      const int g = g0 + threadIdx.x + r * kPoolThreads;
+#pragma unroll
+      for (int i = 0; i < N; ++i) acc[r][i] = 0.f;
+      if (g < g1) {
+        for (int s = 0; s < S; ++s) {
+          const float* p = cluster.map_shared_rank(part, s) + g * N;
+#pragma unroll
+          for (int i = 0; i < N; i += 4) {
+            const float4 v = *reinterpret_cast<const float4*>(p + i);
+            acc[r][i] += v.x;
+            acc[r][i + 1] += v.y;
+            acc[r][i + 2] += v.z;
+            acc[r][i + 3] += v.w;
+          }
+        }
+      }
+    }
+  }
   const float inv_c = count > 0 ? 1.f / static_cast<float>(count) : 0.f;
   float ss = 0.f;
 #pragma unroll
@@ -100,17 +152,24 @@ embed_pool_kernel(const TIn* __restrict__ hidden, int tokens, int dim,
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = ss;
   __syncthreads();
   if (threadIdx.x == 0) {
-    float s = 0.f;
-    for (int w = 0; w < kPoolThreads / 32; ++w) s += red[w];
-    total = s;
+    float t = 0.f;
+    for (int w = 0; w < kPoolThreads / 32; ++w) t += red[w];
+    part_ss = t;
   }
-  __syncthreads();
+  float total = 0.f;
+  if constexpr (kSplit) {
+    cluster.sync();
+    for (int s = 0; s < S; ++s) total += *cluster.map_shared_rank(&part_ss, s);
+  } else {
+    __syncthreads();
+    total = part_ss;
+  }
   const float norm = sqrtf(total);
   const float scale = count > 0 && norm > 0.f ? 1.f / norm : 0.f;
 #pragma unroll
   for (int r = 0; r < R; ++r) {
-    const int g = threadIdx.x + r * kPoolThreads;
-    if (g >= groups) continue;
+    const int g = g0 + threadIdx.x + r * kPoolThreads;
+    if (g >= g1) continue;
     const int64_t e0 = static_cast<int64_t>(b) * dim + static_cast<int64_t>(g) * N;
     if (out_bf16) {
       __nv_bfloat16* o = static_cast<__nv_bfloat16*>(out) + e0;
@@ -126,25 +185,65 @@ embed_pool_kernel(const TIn* __restrict__ hidden, int tokens, int dim,
                                                         acc[r][i + 2] * scale, acc[r][i + 3] * scale);
     }
   }
+  if constexpr (kSplit) cluster.sync();   // the peers have read this CTA's shared memory
+}
+
+// CTAs per row: as many as keep the batch within two CTAs per SM, at most
+// eight (the portable cluster size) and one per block of tokens.  Measured on
+// GB300 against one CTA per row, bf16: 1 x 512 x 4096 11.8 (41.0) us, 8 x 512 x
+// 4096 13.1 (55.0) us, 64 x 512 x 4096 37.1 (82.0) us, 152 x 512 x 4096 72.5
+// (88.5) us, 1 x 64 x 768 4.3 (5.7) us; 256 x 512 x 4096 stays at one (118 us;
+// split in two 121 us).
+int split_for(int batch, int tokens, int num_sms) {
+  int s = 1;
+  while (s < 8 && static_cast<int64_t>(batch) * 2 * s <= 2 * num_sms &&
+         2 * s * kTokenBatch <= tokens)
+    s *= 2;
+  return s;
+}
+
+template <typename TIn, int R>
+cudaError_t launch_r(const TIn* hidden, int batch, int tokens, int dim, const uint8_t* mask,
+                     void* out, int out_bf16, int split, cudaStream_t st) {
+  if (split == 1) {
+    embed_pool_kernel<TIn, R, false><<<batch, kPoolThreads, 0, st>>>(hidden, tokens, dim, mask, out,
+                                                                     out_bf16);
+    return cudaGetLastError();
+  }
+  const size_t smem = static_cast<size_t>(dim) * sizeof(float);
+  if (smem > 48 * 1024) {
+    const cudaError_t e =
+        cudaFuncSetAttribute(embed_pool_kernel<TIn, R, true>,
+                             cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+    if (e != cudaSuccess) return e;
+  }
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(static_cast<unsigned>(batch) * split);
+  cfg.blockDim = dim3(kPoolThreads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = split;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, embed_pool_kernel<TIn, R, true>, hidden, tokens, dim, mask, out,
+                            out_bf16);
 }
 
 template <typename TIn>
 cudaError_t launch_typed(const void* hidden, int batch, int tokens, int dim, const uint8_t* mask,
-                         void* out, int out_bf16, cudaStream_t st) {
+                         void* out, int out_bf16, int split, cudaStream_t st) {
   const int groups = dim / Group<TIn>::kN;
   const int r = (groups + kPoolThreads - 1) / kPoolThreads;
   const TIn* h = static_cast<const TIn*>(hidden);
-  if (r <= 1)
-    embed_pool_kernel<TIn, 1><<<batch, kPoolThreads, 0, st>>>(h, tokens, dim, mask, out, out_bf16);
-  else if (r <= 2)
-    embed_pool_kernel<TIn, 2><<<batch, kPoolThreads, 0, st>>>(h, tokens, dim, mask, out, out_bf16);
-  else if (r <= 4)
-    embed_pool_kernel<TIn, 4><<<batch, kPoolThreads, 0, st>>>(h, tokens, dim, mask, out, out_bf16);
-  else if (r <= 8)
-    embed_pool_kernel<TIn, 8><<<batch, kPoolThreads, 0, st>>>(h, tokens, dim, mask, out, out_bf16);
-  else
-    return cudaErrorInvalidValue;
-  return cudaGetLastError();
+  if (r <= 1) return launch_r<TIn, 1>(h, batch, tokens, dim, mask, out, out_bf16, split, st);
+  if (r <= 2) return launch_r<TIn, 2>(h, batch, tokens, dim, mask, out, out_bf16, split, st);
+  if (r <= 4) return launch_r<TIn, 4>(h, batch, tokens, dim, mask, out, out_bf16, split, st);
+  if (r <= 8) return launch_r<TIn, 8>(h, batch, tokens, dim, mask, out, out_bf16, split, st);
+  return cudaErrorInvalidValue;
 }
 
 }  // namespace
@@ -153,9 +252,14 @@ cudaError_t launch_embed_pool(int hidden_dtype, const void* hidden, int batch, i
                               const uint8_t* mask, int out_dtype, void* out, cudaStream_t st) {
   if (batch <= 0) return cudaSuccess;
   const int out_bf16 = out_dtype == kBF16 ? 1 : 0;
+  int dev = 0, sms = 1;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (e != cudaSuccess) return e;
+  const int split = split_for(batch, tokens, sms);
   return hidden_dtype == kBF16
-             ? launch_typed<uint16_t>(hidden, batch, tokens, dim, mask, out, out_bf16, st)
-             : launch_typed<float>(hidden, batch, tokens, dim, mask, out, out_bf16, st);
+             ? launch_typed<uint16_t>(hidden, batch, tokens, dim, mask, out, out_bf16, split, st)
+             : launch_typed<float>(hidden, batch, tokens, dim, mask, out, out_bf16, split, st);
 }
 
 }  // namespace oprag
