@@ -5,20 +5,31 @@
 // The per-posting weight idf(t) * tf (k1 + 1) / (tf + k1 (1 - b + b |d| / avgdl))
 // does not depend on the query, so it is computed once on the host when the
 // sparse side is attached; a query's BM25 for chunk d is then the sum of the
-// weights of its terms' postings at d, taken in the order of the query's term
-// list (a repeated term counts again).
+// weights of its terms' postings at d (a repeated term counts again).
 //
-// One CTA per (query, tile of 8192 chunks) accumulates those sums in shared
-// memory, one term at a time in the query's order; a table built with the
-// postings gives where each sparse term's postings enter the tile.  A dense term (held by
-// more than half of the chunks, stored as a row of weights with zeros where
-// absent) is added element-wise with 16-byte loads, each thread keeping the
-// same elements, so consecutive dense terms need no barrier; a sparse term
-// scatters its postings (each chunk at most once per term, so its adds never
-// collide).  Adding a zero weight leaves an fp32 sum unchanged, so both forms
-// give the same sums in the same order.  The CTA writes the tile's row of the
-// q x n BM25 matrix and folds the tile maximum into the per-query maximum
-// that normalises the lexical score.
+// Work items are (tile of 1024 chunks, query), tile-major, in one contiguous
+// share per CTA; a warp takes one item.  Its lanes hold the tile's sums in
+// registers while the query's dense terms (held by more than half of the
+// chunks, stored as rows of weights with zeros where absent) are added, then
+// the sums go to the warp's row in shared memory, where the sparse terms
+// scatter their postings (each chunk at most once per term, so one term's adds
+// never collide); a table built with the postings gives where each sparse
+// term's postings enter the tile.  The order -- dense terms in the query's
+// order, then sparse terms in the query's order -- is the order of the rerank
+// too, so both give the same sums.  Adding a zero weight leaves an fp32 sum
+// unchanged.  The warp writes the tile's row of the q x n BM25 matrix and
+// folds the tile maximum into the per-query maximum that normalises the
+// lexical score.
+//
+// A query holds about four of the thirty or so dense terms, so a CTA with
+// several queries of a tile copies that tile of all dense rows to shared
+// memory once and the items read them there: 1024 queries on 32768 chunks read
+// 19 MB of dense rows from L2 instead of 530 MB.  What is left is the write of
+// the block (134 MB) and the shared-memory passes (about 30 KB per item).
+// Measured on GB300 (8 Zipf terms a query): 64 us instead of 88 us for one CTA
+// per query and tile of 8192 chunks with its sums in shared memory.
+#include <algorithm>
+
 #include "common.cuh"
 #include "internal.h"
 
@@ -27,127 +38,181 @@ namespace oprag {
 namespace {
 
 constexpr int kDocTile = kBm25DocTile;
-constexpr int kBm25Threads = 256;
-constexpr int kTermsPerPass = kBm25Threads / 32;
-constexpr int kScatterUnroll = 4;      // postings loaded per thread before the adds
-constexpr int kDenseBatch = 8;         // dense-row float4 groups loaded per thread before the adds
-constexpr int kSkipTerm = -2;          // term id outside the vocabulary
+constexpr int kBm25Warps = 20;
+constexpr int kBm25Threads = kBm25Warps * 32;
+constexpr int kVec = kDocTile / 4 / 32;      // float4 groups of a tile per lane
+constexpr int kPostBatch = 4;                // postings per lane and chunk
+constexpr int kChunks = 4;                   // chunks loaded before their adds
+// Dense rows kept in shared memory (4 KB each), beside the warps' rows: the
+// commonest terms of a Zipf corpus; others are read from L2.
+constexpr int kBm25MaxRows = 29;
+// Queries of a tile in one CTA from which its dense rows are copied: a query
+// reads about four of them, so below that direct reads move fewer bytes.
+constexpr int kStageMinQueries = 8;
+// Queries and terms of one batch whose lookups are done together.
+constexpr int kBatchQueries = 120;
+constexpr int kBatchTerms = 2048;
 
-__global__ void __launch_bounds__(kBm25Threads)
+// One lane's term of a query: its dense row (-1: postings [lo, hi) of the
+// tile, -2: none).
+struct TermSlot {
+  int slot, lo, hi;
+};
+
+__device__ __forceinline__ TermSlot load_term(const SparseIndex& sp,
+                                              const int32_t* __restrict__ q_terms, int ti, int t1,
+                                              int tile) {
+  TermSlot t{-2, 0, 0};
+  const int32_t term = ti < t1 ? q_terms[ti] : -1;
+  if (term >= 0 && term < sp.vocab) {
+    const int32_t* tp = sp.tile_ptr + static_cast<int64_t>(term) * (sp.ntiles + 1) + tile;
+    t.slot = sp.dense_slot[term];
+    t.lo = tp[0];
+    t.hi = tp[1];
+  }
+  return t;
+}
+
+__global__ void __launch_bounds__(kBm25Threads, 1)
 bm25_matrix_kernel(SparseIndex sp, int64_t n, const int32_t* __restrict__ q_indptr,
-                   const int32_t* __restrict__ q_terms, float* __restrict__ out, int64_t ld,
-                   float* __restrict__ out_max) {
-  __shared__ __align__(16) float acc[kDocTile];
-  __shared__ int64_t rng_lo[kTermsPerPass], rng_hi[kTermsPerPass];
-  __shared__ int slot_of[kTermsPerPass];
-  __shared__ float red[kBm25Threads / 32];
-  const int qi = blockIdx.x;
-  const int64_t d0 = static_cast<int64_t>(blockIdx.y) * kDocTile;
-  const int64_t d1 = min(n, d0 + kDocTile);
-  const int nv = static_cast<int>((d1 - d0 + 3) / 4);     // float4 groups of this tile
+                   const int32_t* __restrict__ q_terms, int q, float* __restrict__ out, int64_t ld,
+                   float* __restrict__ out_max, int rows) {
+  extern __shared__ __align__(16) float smem_b[];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  float4* acc4 = reinterpret_cast<float4*>(acc);
-
-  for (int i = threadIdx.x; i < kDocTile / 4; i += blockDim.x) acc4[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-
-  const int t0 = q_indptr[qi], t1 = q_indptr[qi + 1];
-  bool pending = true;      // element-wise work since the last barrier came from a scatter
-  for (int base = t0; base < t1; base += kTermsPerPass) {
-    // Classify each term of the pass and locate a sparse term's postings
-    // inside [d0, d1) in the per-tile table: one thread per term, its three
-    // loads issued together.
-    const int ti = base + warp;
-    if (ti < t1 && lane == 0) {
-      const int32_t term = q_terms[ti];
-      int slot = kSkipTerm;
-      int64_t lo = 0, hi = 0;
-      if (term >= 0 && term < sp.vocab) {
-        const int64_t* tp = sp.tile_ptr + static_cast<int64_t>(term) * (sp.ntiles + 1) + blockIdx.y;
-        const int64_t a = tp[0], z = tp[1];
-        slot = sp.dense_slot[term];
-        if (slot < 0) {
-          lo = a;
-          hi = z;
-        }
+  float* row = smem_b + warp * kDocTile;
+  float4* row4 = reinterpret_cast<float4*>(row);
+  // Term lookups of the batch, by raw term position, and its query offsets.
+  int* t_slot = reinterpret_cast<int*>(smem_b + kBm25Warps * kDocTile);
+  int* t_lo = t_slot + kBatchTerms;
+  int* t_hi = t_lo + kBatchTerms;
+  int* q_ptr = t_hi + kBatchTerms;
+  float4* dense4 = reinterpret_cast<float4*>(q_ptr + kBatchQueries + 8);
+  const int64_t total = static_cast<int64_t>(sp.ntiles) * q;
+  const int64_t w1 = total * (blockIdx.x + 1) / gridDim.x;
+  int loaded = -1;             // tile whose dense rows are in shared memory
+  for (int64_t w = total * blockIdx.x / gridDim.x; w < w1;) {
+    const int tile = static_cast<int>(w / q);
+    const int qa = static_cast<int>(w - static_cast<int64_t>(tile) * q);
+    const int q_tile = static_cast<int>(min(static_cast<int64_t>(q), qa + (w1 - w)));
+    const int qb = min(q_tile, qa + kBatchQueries);
+    w += qb - qa;
+    const int64_t d0 = static_cast<int64_t>(tile) * kDocTile;
+    const int first_doc = static_cast<int>(d0);
+    const int nv = static_cast<int>((min(n - d0, static_cast<int64_t>(kDocTile)) + 3) / 4);
+    __syncthreads();           // the previous batch has been computed
+    for (int i = threadIdx.x; i <= qb - qa; i += kBm25Threads) q_ptr[i] = q_indptr[qa + i];
+    if (loaded != tile && q_tile - qa >= kStageMinQueries) {
+      for (int i = threadIdx.x; i < rows * (kDocTile / 4); i += kBm25Threads) {
+        const int r = i / (kDocTile / 4), v = i % (kDocTile / 4);
+        if (v < nv)
+          dense4[i] = __ldg(reinterpret_cast<const float4*>(sp.dense_w + r * sp.dense_ld + d0) + v);
       }
-      slot_of[warp] = slot;
-      rng_lo[warp] = lo;
-      rng_hi[warp] = hi;
+      loaded = tile;
     }
+    const int staged = loaded == tile ? rows : 0;
     __syncthreads();
-    pending = false;
-    bool dirty = false;     // unsynchronised adds since the last barrier
-    const int nt = min(kTermsPerPass, t1 - base);
-    for (int w = 0; w < nt; ++w) {
-      const int slot = slot_of[w];
-      if (slot == kSkipTerm) continue;
-      if (slot >= 0) {
-        // Dense term: thread i owns float4 groups i, i + 256, ...; after
-        // another dense term nothing needs ordering.
-        if (pending) __syncthreads();
-        // The row's groups are loaded kDenseBatch at a time, all before the
-        // adds, so a dense term costs one L2 round trip per batch.
-        const float4* row = reinterpret_cast<const float4*>(sp.dense_w + slot * sp.dense_ld + d0);
-        for (int i0 = threadIdx.x; i0 < nv; i0 += kDenseBatch * kBm25Threads) {
-          float4 x[kDenseBatch];
-#pragma unroll
-          for (int u = 0; u < kDenseBatch; ++u) {
-            const int i = i0 + u * kBm25Threads;
-            x[u] = i < nv ? __ldg(row + i) : make_float4(0.f, 0.f, 0.f, 0.f);
-          }
-#pragma unroll
-          for (int u = 0; u < kDenseBatch; ++u) {
-            const int i = i0 + u * kBm25Threads;
-            if (i < nv) {
-              float4 a = acc4[i];
-              a.x += x[u].x;
-              a.y += x[u].y;
-              a.z += x[u].z;
-              a.w += x[u].w;
-              acc4[i] = a;
-            }
-          }
-        }
-        pending = false;
-        dirty = true;
-      } else {
-        if (dirty) __syncthreads();
-        const int64_t lo = rng_lo[w], hi = rng_hi[w];
-        for (int64_t p = lo + threadIdx.x; p < hi; p += kScatterUnroll * blockDim.x) {
-          int2 e[kScatterUnroll];
-#pragma unroll
-          for (int u = 0; u < kScatterUnroll; ++u) {
-            const int64_t pp = p + static_cast<int64_t>(u) * blockDim.x;
-            e[u] = pp < hi ? __ldg(sp.post + pp) : make_int2(-1, 0);
-          }
-#pragma unroll
-          for (int u = 0; u < kScatterUnroll; ++u)
-            if (e[u].x >= 0) acc[e[u].x - d0] += __int_as_float(e[u].y);
-        }
-        pending = true;
-        dirty = true;
+    const int tb = q_ptr[0];
+    const bool listed = q_ptr[qb - qa] - tb <= kBatchTerms;    // else looked up per item
+    if (listed) {
+      for (int i = threadIdx.x; i < q_ptr[qb - qa] - tb; i += kBm25Threads) {
+        const TermSlot t = load_term(sp, q_terms, tb + i, tb + i + 1, tile);
+        t_slot[i] = t.slot;
+        t_lo[i] = t.lo;
+        t_hi[i] = t.hi;
       }
+      __syncthreads();
     }
-    __syncthreads();        // the next pass rewrites the term table; the output reads acc
-  }
-
-  float m = 0.f;
-  float4* orow =
-      out != nullptr ? reinterpret_cast<float4*>(out + static_cast<int64_t>(qi) * ld + d0) : nullptr;
-  for (int i = threadIdx.x; i < nv; i += blockDim.x) {
-    const float4 v = acc4[i];
-    if (orow != nullptr) orow[i] = v;
-    m = fmaxf(fmaxf(m, fmaxf(v.x, v.y)), fmaxf(v.z, v.w));
-  }
+    auto term = [&](int ti, int t1) {
+      if (!listed) return load_term(sp, q_terms, ti, t1, tile);
+      return ti < t1 ? TermSlot{t_slot[ti - tb], t_lo[ti - tb], t_hi[ti - tb]} : TermSlot{-2, 0, 0};
+    };
+    for (int qi = qa + warp; qi < qb; qi += kBm25Warps) {
+      const int b0 = q_ptr[qi - qa], b1 = q_ptr[qi - qa + 1];
+      float4 acc[kVec];
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-  if (lane == 0) red[warp] = m;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    float bm = red[0];
-    for (int w = 1; w < kBm25Threads / 32; ++w) bm = fmaxf(bm, red[w]);
-    // BM25 is never negative, so the float order equals the int order.
-    atomicMax(reinterpret_cast<int*>(out_max + qi), __float_as_int(bm));
+      for (int u = 0; u < kVec; ++u) acc[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+      // Dense terms, 32 of the query's terms at a time.
+      for (int base = b0; base < b1; base += 32) {
+        const int slot = term(base + lane, b1).slot;
+        for (uint32_t m = __ballot_sync(0xffffffffu, slot >= 0); m != 0; m &= m - 1) {
+          const int s = __shfl_sync(0xffffffffu, slot, __ffs(m) - 1);
+          float4 x[kVec];
+          if (s < staged) {
+#pragma unroll
+            for (int u = 0; u < kVec; ++u) x[u] = dense4[s * (kDocTile / 4) + lane + 32 * u];
+          } else {
+            const float4* src = reinterpret_cast<const float4*>(sp.dense_w + s * sp.dense_ld + d0);
+#pragma unroll
+            for (int u = 0; u < kVec; ++u)
+              x[u] = lane + 32 * u < nv ? __ldg(src + lane + 32 * u) : make_float4(0.f, 0.f, 0.f, 0.f);
+          }
+#pragma unroll
+          for (int u = 0; u < kVec; ++u) {
+            acc[u].x += x[u].x;
+            acc[u].y += x[u].y;
+            acc[u].z += x[u].z;
+            acc[u].w += x[u].w;
+          }
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < kVec; ++u) row4[lane + 32 * u] = acc[u];
+      __syncwarp();
+      // Sparse terms: the postings go in chunks of 32 kPostBatch of one term;
+      // kChunks chunks (of one or several terms) are loaded together, then
+      // added one after the other.
+      for (int base = b0; base < b1; base += 32) {
+        const TermSlot t = term(base + lane, b1);
+        uint32_t m = __ballot_sync(0xffffffffu, t.slot == -1 && t.lo < t.hi);
+        int p = 0, hi = 0;       // the current term's postings still to load
+        while (p < hi || m != 0) {
+          int2 e[kChunks][kPostBatch];
+#pragma unroll
+          for (int h = 0; h < kChunks; ++h) {
+            if (p >= hi && m != 0) {
+              const int src = __ffs(m) - 1;
+              p = __shfl_sync(0xffffffffu, t.lo, src);
+              hi = __shfl_sync(0xffffffffu, t.hi, src);
+              m &= m - 1;
+            }
+#pragma unroll
+            for (int u = 0; u < kPostBatch; ++u) {
+              const int i = p + lane + 32 * u;
+              e[h][u] = i < hi ? __ldg(sp.post + i) : make_int2(-1, 0);
+            }
+            p += 32 * kPostBatch;
+          }
+#pragma unroll
+          for (int h = 0; h < kChunks; ++h) {
+            // (one term's chunks are distinct: all reads before the writes)
+            float v[kPostBatch];
+#pragma unroll
+            for (int u = 0; u < kPostBatch; ++u)
+              if (e[h][u].x >= 0) v[u] = row[e[h][u].x - first_doc];
+#pragma unroll
+            for (int u = 0; u < kPostBatch; ++u)
+              if (e[h][u].x >= 0) row[e[h][u].x - first_doc] = v[u] + __int_as_float(e[h][u].y);
+            __syncwarp();
+          }
+        }
+      }
+      float top = 0.f;
+      float4* orow = out != nullptr
+                         ? reinterpret_cast<float4*>(out + static_cast<int64_t>(qi) * ld + d0)
+                         : nullptr;
+#pragma unroll
+      for (int u = 0; u < kVec; ++u) {
+        if (lane + 32 * u < nv) {
+          const float4 v = row4[lane + 32 * u];
+          if (orow != nullptr) orow[lane + 32 * u] = v;
+          top = fmaxf(fmaxf(top, fmaxf(v.x, v.y)), fmaxf(v.z, v.w));
+        }
+      }
+      // BM25 is never negative, so the float order equals the int order.
+      const int bits = __reduce_max_sync(0xffffffffu, __float_as_int(top));
+      if (lane == 0 && bits > 0) atomicMax(reinterpret_cast<int*>(out_max + qi), bits);
+      __syncwarp();            // the row is read before the next item overwrites it
+    }
   }
 }
 
@@ -221,12 +286,26 @@ cudaError_t launch_lex_prep(const int32_t* lex_class, const int64_t* post_ptr, i
 
 cudaError_t launch_bm25_matrix(const SparseIndex& sp, int64_t n, const int32_t* q_indptr,
                                const int32_t* q_terms, int q, float* out, int64_t ld,
-                               float* out_max, cudaStream_t st) {
+                               float* out_max, int num_sms, cudaStream_t st) {
   if (q <= 0) return cudaSuccess;
   cudaError_t e = cudaMemsetAsync(out_max, 0, sizeof(float) * q, st);
   if (e != cudaSuccess) return e;
-  const dim3 grid(q, static_cast<unsigned>((n + kDocTile - 1) / kDocTile));
-  bm25_matrix_kernel<<<grid, kBm25Threads, 0, st>>>(sp, n, q_indptr, q_terms, out, ld, out_max);
+  const int rows = std::min(sp.dense_rows, kBm25MaxRows);
+  constexpr size_t kRow = kDocTile * sizeof(float);
+  constexpr size_t kFixed = kBm25Warps * kRow +
+                            (3 * kBatchTerms + kBatchQueries + 8) * sizeof(int);
+  static bool configured = false;
+  if (!configured) {
+    e = cudaFuncSetAttribute(bm25_matrix_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             static_cast<int>(kFixed + kBm25MaxRows * kRow));
+    if (e != cudaSuccess) return e;
+    configured = true;
+  }
+  // One CTA per SM (its shared memory), fewer when there are fewer items.
+  const int64_t items = static_cast<int64_t>(sp.ntiles) * q;
+  const int grid = static_cast<int>(std::min<int64_t>(items, num_sms));
+  bm25_matrix_kernel<<<grid, kBm25Threads, kFixed + rows * kRow, st>>>(
+      sp, n, q_indptr, q_terms, q, out, ld, out_max, rows);
   return cudaGetLastError();
 }
 

@@ -218,8 +218,8 @@ cudaError_t launch_merge_two(int q, const int64_t* a_ids, const float* a_sc, int
 // Terms held by more than half of the chunks are stored as dense rows of
 // w(t, .) (zero where absent: 4 bytes per chunk instead of 8 per posting, and
 // no scatter); the other terms as postings.
-// Chunks per tile of the BM25 pass (one CTA per query and tile).
-constexpr int kBm25DocTile = 8192;
+// Chunks per tile of the BM25 pass (one warp per query and tile).
+constexpr int kBm25DocTile = 1024;
 
 struct SparseIndex {
   int vocab;
@@ -227,17 +227,18 @@ struct SparseIndex {
   const int64_t* post_ptr;   // device, vocab + 1 (empty range for dense terms)
   const int2* post;          // device, nnz (chunk, weight bits), chunks ascending per term
   const int32_t* dense_slot; // device, vocab: row of a dense term, -1 otherwise
-  const float* dense_w;      // device, rows x dense_ld
+  const float* dense_w;      // device, dense_rows x dense_ld
+  int dense_rows;
   int64_t dense_ld;          // multiple of 4, >= n; zero past n
   // device, vocab x (ntiles + 1): entry (t, b) is the first posting of term t
   // whose chunk is >= b * kBm25DocTile (post_ptr[t + 1] past the last).
-  const int64_t* tile_ptr;
+  const int32_t* tile_ptr;
   int ntiles;
 };
 // out == nullptr computes only the per-query maxima (the gathered form).
 cudaError_t launch_bm25_matrix(const SparseIndex& sp, int64_t n, const int32_t* q_indptr,
                                const int32_t* q_terms, int q, float* out, int64_t ld,
-                               float* out_max, cudaStream_t st);
+                               float* out_max, int num_sms, cudaStream_t st);
 
 // Per-query operands of the gathered lexical part (see Fusion): qcount
 // (q x kLexK bf16), terms (q x kLexRegTerms), mid (q x kLexMidReg) and the
@@ -279,7 +280,7 @@ struct LexBuild {
   float* mid_w;
   int64_t mid_ld;
 };
-cudaError_t launch_lex_build(const LexBuild& lb, int ntiles, int64_t* tile_ptr, cudaStream_t st);
+cudaError_t launch_lex_build(const LexBuild& lb, int ntiles, int32_t* tile_ptr, cudaStream_t st);
 
 // --- lexical rerank of a dense top-N (dense-first hybrid), rerank.cu.
 // cand_ids / cand_scores: q x ncand dense results (id -1 = none), ncand <=

@@ -94,8 +94,9 @@ struct oprag_index {
   int2* post = nullptr;
   int32_t* dense_slot = nullptr;
   float* dense_w = nullptr;
+  int dense_rows = 0;
   int64_t dense_ld = 0;
-  int64_t* tile_ptr = nullptr;
+  int32_t* tile_ptr = nullptr;
   int ntiles = 0;
   void* wsplit = nullptr;      // n x kLexK bf16 head-term weights (high | low halves)
   int32_t* lex_class = nullptr;  // vocab: epilogue class of each term (see rebuild_sparse)
@@ -1117,7 +1118,7 @@ int rebuild_sparse(oprag_index* idx) {
       cudaMalloc(&idx->post, std::max<int64_t>(nnz, 1) * sizeof(int2)) != cudaSuccess ||
       cudaMalloc(&idx->dense_slot, slot.size() * sizeof(int32_t)) != cudaSuccess ||
       cudaMalloc(&idx->dense_w, dense_elems * sizeof(float)) != cudaSuccess ||
-      cudaMalloc(&idx->tile_ptr, tptr_elems * sizeof(int64_t)) != cudaSuccess ||
+      cudaMalloc(&idx->tile_ptr, tptr_elems * sizeof(int32_t)) != cudaSuccess ||
       cudaMalloc(&idx->wsplit, wsplit_elems * sizeof(uint16_t)) != cudaSuccess ||
       cudaMalloc(&idx->lex_class, lex_class.size() * sizeof(int32_t)) != cudaSuccess ||
       cudaMalloc(&idx->mid_w, mid_elems * sizeof(float)) != cudaSuccess ||
@@ -1163,6 +1164,7 @@ int rebuild_sparse(oprag_index* idx) {
     return cuda_fail(e, "building the lexical index");
   }
   idx->nnz = nnz;
+  idx->dense_rows = n_dense;
   idx->dense_ld = dld;
   idx->mid_ld = mld;
   idx->ntiles = ntiles;
@@ -1254,8 +1256,8 @@ int oprag_hybrid_search(oprag_index* idx, const void* queries, int32_t q, const 
     return rc;
   if ((rc = begin_call(idx, st))) return rc;
   const SparseIndex sp{idx->vocab,      idx->nnz,     idx->post_ptr, idx->post,
-                       idx->dense_slot, idx->dense_w, idx->dense_ld, idx->tile_ptr,
-                       idx->ntiles};
+                       idx->dense_slot, idx->dense_w, idx->dense_rows, idx->dense_ld,
+                       idx->tile_ptr,   idx->ntiles};
   char* lex = reinterpret_cast<char*>(idx->lex);
   if (gather) {
     // Gathered form (Sec. 4.4 fusion in the dense epilogue): per-query
@@ -1271,7 +1273,8 @@ int oprag_hybrid_search(oprag_index* idx, const void* queries, int32_t q, const 
     cudaError_t e = launch_lex_prep(idx->lex_class, idx->post_ptr, idx->vocab, q_indptr, q_terms,
                                     q, prep, st);
     if (e == cudaSuccess)
-      e = launch_bm25_matrix(sp, idx->n, q_indptr, q_terms, q, nullptr, 0, bm_max, st);
+      e = launch_bm25_matrix(sp, idx->n, q_indptr, q_terms, q, nullptr, 0, bm_max,
+                             idx->num_sms, st);
     if (e != cudaSuccess) return cuda_fail(e, "BM25 maximum pass");
     Fusion fu{nullptr, 0, bm_max, alpha};
     fu.lex_qcount = prep.qcount;
@@ -1305,7 +1308,7 @@ int oprag_hybrid_search(oprag_index* idx, const void* queries, int32_t q, const 
     if (idx->timing) cudaEventRecord(idx->ev[0], st);
     idx->timed_lex = idx->timing;
     cudaError_t e = launch_bm25_matrix(sp, idx->n, q_indptr + c0, q_terms, qc, block, ld,
-                                       blockmax, st);
+                                       blockmax, idx->num_sms, st);
     if (e != cudaSuccess) return cuda_fail(e, "BM25 kernel");
     const Fusion fu{block, ld, blockmax, alpha};
     if ((rc = run_search(idx, static_cast<const char*>(queries) + c0 * qrow, qc, k, fu,
@@ -1344,8 +1347,8 @@ int oprag_hybrid_search_dense_first(oprag_index* idx, const void* queries, int32
   const Fusion none{nullptr, 0, nullptr, 0.f};
   if ((rc = run_search(idx, queries, q, nc, none, cid, csc, st))) return rc;
   const SparseIndex sp{idx->vocab,      idx->nnz,     idx->post_ptr, idx->post,
-                       idx->dense_slot, idx->dense_w, idx->dense_ld, idx->tile_ptr,
-                       idx->ntiles};
+                       idx->dense_slot, idx->dense_w, idx->dense_rows, idx->dense_ld,
+                       idx->tile_ptr,   idx->ntiles};
   cudaError_t e = launch_rerank(sp, q, nc, cid, csc, q_indptr, q_terms, alpha, k, out_ids,
                                 out_scores, st);
   if (e != cudaSuccess) return cuda_fail(e, "rerank kernel");

@@ -4,9 +4,9 @@
 // Sec. 4.4 and the ranked top-k of the fused scores.
 //
 // One CTA of four warps per query; a thread holds one or two candidates.  A
-// candidate's BM25 is the sum of its query terms' weights in the query's term
-// order: a dense term's weight is read from its row, a sparse term's is found
-// by a binary search of the term's postings.  What bounds it is the latency of
+// candidate's BM25 is the sum of its query terms' weights: a dense term's
+// weight is read from its row, a sparse term's is found by a binary search of
+// the term's postings.  What bounds it is the latency of
 // those dependent loads, so a thread searches kTermBatch terms at once, and
 // the searches of a whole batch of terms take as long as one.  The sums and
 // the fused score are formed exactly as in the BM25 pass and the fused search
@@ -48,21 +48,21 @@ rerank_kernel(SparseIndex sp, int ncand, const int64_t* __restrict__ cand_ids,
     lex[e] = 0.f;
   }
   const int t0 = q_indptr[qi], t1 = q_indptr[qi + 1];
-  for (int base = t0; base < t1; base += kTermBatch) {
+  // Adds the dense and / or the sparse terms of one batch, dense terms first.
+  auto add_batch = [&](int base, bool with_dense, bool with_sparse) {
+    __syncthreads();        // the previous batch's term table has been read
     if (tid < kTermBatch) {
       int slot = -2;
       int64_t lo = 0, hi = 0;
       const int32_t term = base + tid < t1 ? q_terms[base + tid] : -1;
       if (term >= 0 && term < sp.vocab) {
         slot = sp.dense_slot[term];
-        if (slot < 0) {
-          lo = sp.post_ptr[term];
-          hi = sp.post_ptr[term + 1];
-        }
+        lo = sp.post_ptr[term];              // (an empty range for a dense term)
+        hi = sp.post_ptr[term + 1];
       }
-      term_slot[tid] = slot;
+      term_slot[tid] = with_dense ? slot : -2;
       term_lo[tid] = lo;
-      term_hi[tid] = hi;
+      term_hi[tid] = with_sparse ? hi : lo;
     }
     __syncthreads();
     float w[kTermBatch][E];
@@ -99,20 +99,32 @@ rerank_kernel(SparseIndex sp, int ncand, const int64_t* __restrict__ cand_ids,
       }
     }
 #pragma unroll
+    for (int b = 0; b < kTermBatch; ++b)
+#pragma unroll
+      for (int e = 0; e < E; ++e) lex[e] += w[b][e];
+#pragma unroll
     for (int b = 0; b < kTermBatch; ++b) {
       const int len = static_cast<int>(term_hi[b] - term_lo[b]);
 #pragma unroll
-      for (int e = 0; e < E; ++e)
+      for (int e = 0; e < E; ++e) {
+        w[b][e] = 0.f;
         if (doc[e] >= 0 && lo[b][e] < len) {
           const int2 pe = __ldg(sp.post + term_lo[b] + lo[b][e]);
           if (pe.x == doc[e]) w[b][e] = __int_as_float(pe.y);
         }
+      }
     }
 #pragma unroll
     for (int b = 0; b < kTermBatch; ++b)
 #pragma unroll
       for (int e = 0; e < E; ++e) lex[e] += w[b][e];
-    __syncthreads();        // the next batch rewrites the term table
+  };
+  // The BM25 pass's order: all dense terms, then all sparse terms.
+  if (t1 - t0 <= kTermBatch) {
+    add_batch(t0, true, true);
+  } else {
+    for (int base = t0; base < t1; base += kTermBatch) add_batch(base, true, false);
+    for (int base = t0; base < t1; base += kTermBatch) add_batch(base, false, true);
   }
   // BM25 maximum over the candidates (BM25 is never negative).
   float m = 0.f;

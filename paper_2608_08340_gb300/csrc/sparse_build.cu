@@ -59,7 +59,7 @@ __global__ void lex_weights_kernel(LexBuild lb) {
 // One thread per (term, tile boundary b): the first posting of the term whose
 // chunk is >= b * kBm25DocTile.
 __global__ void tile_ptr_kernel(const int64_t* __restrict__ post_ptr, const int2* __restrict__ post,
-                                int vocab, int ntiles, int64_t* __restrict__ tile_ptr) {
+                                int vocab, int ntiles, int32_t* __restrict__ tile_ptr) {
   const int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
   const int64_t per = ntiles + 1;
   if (i >= static_cast<int64_t>(vocab) * per) return;
@@ -70,12 +70,12 @@ __global__ void tile_ptr_kernel(const int64_t* __restrict__ post_ptr, const int2
     const int64_t mid = (lo + hi) >> 1;
     if (post[mid].x < doc0) lo = mid + 1; else hi = mid;
   }
-  tile_ptr[i] = lo;
+  tile_ptr[i] = static_cast<int32_t>(lo);
 }
 
 }  // namespace
 
-cudaError_t launch_lex_build(const LexBuild& lb, int ntiles, int64_t* tile_ptr, cudaStream_t st) {
+cudaError_t launch_lex_build(const LexBuild& lb, int ntiles, int32_t* tile_ptr, cudaStream_t st) {
   if (lb.vocab <= 0) return cudaSuccess;
   const int64_t warps = lb.vocab;
   const int blocks = static_cast<int>(std::min<int64_t>((warps + 7) / 8, 8192));
