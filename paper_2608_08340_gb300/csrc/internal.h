@@ -110,6 +110,8 @@ struct SearchShape {
   // The lexical part is gathered in the tensor-core epilogue: the plan uses
   // single CTAs with 128-row corpus tiles and one epilogue set.
   bool fused_lex = false;
+  // The epilogue reads a materialised BM25 block.
+  bool lex_block = false;
   // Group pass of a search with buffered lists: no lists, the maxima of groups
   // of `group` (8 or 32) scores instead (0: an ordinary search).
   int group = 0;

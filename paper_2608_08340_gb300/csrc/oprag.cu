@@ -308,11 +308,15 @@ struct SearchLayout {
 
 size_t round256(size_t b) { return (b + 255) / 256 * 256; }
 
+// Lexical part of a search: none, a materialised BM25 block, or gathered.
+enum class LexForm { kNone, kBlock, kGather };
+
 SearchLayout search_layout(oprag_index* idx, int q, int k, int path, int block_n, int pair,
-                           bool lex = false, int64_t n_second = 0) {
+                           LexForm lex = LexForm::kNone, int64_t n_second = 0) {
   SearchLayout L;
   SearchShape s{idx->n, idx->d, q, k};
-  s.fused_lex = lex && path == 2;
+  s.fused_lex = lex == LexForm::kGather && path == 2;
+  s.lex_block = lex == LexForm::kBlock && path == 2;
   s.n_second = path == 2 ? n_second : 0;
   L.path = path;
   if (path == 1) {
@@ -350,7 +354,7 @@ SearchLayout search_layout(oprag_index* idx, int q, int k, int path, int block_n
   return L;
 }
 
-SearchLayout search_layout(oprag_index* idx, int q, int k, bool lex = false) {
+SearchLayout search_layout(oprag_index* idx, int q, int k, LexForm lex = LexForm::kNone) {
   return search_layout(idx, q, k, choose_path(idx, q), idx->opt_block_n, idx->opt_pair, lex);
 }
 
@@ -427,7 +431,10 @@ int launch_search(oprag_index* idx, const SearchLayout& L, const void* Q, int q,
 // index's scratch (and shared bounds) on demand.
 int run_search(oprag_index* idx, const void* Q, int q, int k, const Fusion& fu, int64_t* out_ids,
                float* out_scores, cudaStream_t st) {
-  const SearchLayout L = search_layout(idx, q, k, fu.gathered());
+  const SearchLayout L =
+      search_layout(idx, q, k,
+                    fu.gathered() ? LexForm::kGather
+                                  : fu.bm25 != nullptr ? LexForm::kBlock : LexForm::kNone);
   int rc = idx->ensure(&idx->scratch, &idx->scratch_bytes, L.total(), "search scratch");
   if (rc) return rc;
   uint64_t* qf = nullptr;
@@ -671,7 +678,7 @@ int oprag_index_reserve(oprag_index* idx, int32_t q_max, int32_t k_max) {
       const int k = std::min(kk, kcap);
       for (int qq : {static_cast<int>(q_max), std::min<int>(q_max, 128)})
         if (idx->dtype == OPRAG_BF16)
-          need = std::max(need, search_layout(idx, qq, k, 2, 0, 0, true).total());
+          need = std::max(need, search_layout(idx, qq, k, 2, 0, 0, LexForm::kGather).total());
     }
     rc = idx->ensure(&idx->scratch, &idx->scratch_bytes, need, "search scratch");
     if (rc) return rc;
@@ -824,7 +831,7 @@ int oprag_search_two(oprag_index* knowledge, oprag_index* memory, const void* qu
     // the source and the id within it.  Scratch and bounds of the knowledge
     // index.
     const SearchLayout L = search_layout(knowledge, q, k, 2, knowledge->opt_block_n,
-                                         knowledge->opt_pair, false, memory->n);
+                                         knowledge->opt_pair, LexForm::kNone, memory->n);
     if ((rc = knowledge->ensure(&knowledge->scratch, &knowledge->scratch_bytes, L.total(),
                                 "search scratch")))
       return rc;

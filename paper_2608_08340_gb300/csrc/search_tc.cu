@@ -46,12 +46,16 @@ TcPlan tc_plan(const SearchShape& s, int num_sms, int force_block_n, int tile_st
   // when there are at least two query tiles and at most four dual units per
   // CTA (small batches, where the copies into the SMs, not the MMAs, bound
   // the kernel; measured on 32768 x 768: faster up to 512 queries, slower at
-  // 1024); it needs the two epilogue sets of lists of 8 or 16.
+  // 1024); it needs the two epilogue sets of lists of 8 or 16.  With a BM25
+  // block the epilogue's reads of the block bound the kernel, and dual mode's
+  // four accumulators overlap them best at every batch size: 32768 x 768, 256
+  // queries 31 us against 42 (256-row tiles), 1024 queries 72 against 83.
   const bool dual_ok = !s.fused_lex && pl.qt >= 2 && list_len_of(s) <= 16 &&
                        force_pair != 2 && (force_block_n == 0 || force_block_n == 128);
   const int64_t dual_units =
       static_cast<int64_t>((pl.qt + 1) / 2) * ((s.n + 127) / 128 + (s.n_second + 127) / 128);
-  pl.dual = dual_ok && (force_pair == 3 || (force_pair == 0 && dual_units <= 4LL * num_sms));
+  pl.dual = dual_ok && (force_pair == 3 ||
+                        (force_pair == 0 && (s.lex_block || dual_units <= 4LL * num_sms)));
   if (pl.dual) bn = 128;
   pl.block_n = bn;
   // CTA pairs cut the operand bytes each SM loads per MMA by a third; they
@@ -168,10 +172,14 @@ cudaError_t launch_tc_search(const void* E, const void* Q, const SearchShape& s,
         !make_map(&maps.qb, fu.lex_qcount, s.q, kLexK, a_rows) ||
         !make_map(&maps.eb, fu.lex_wsplit, s.n, kLexK, pl.block_n))
       return cudaErrorInvalidValue;
+  } else if (lex == kLexBlock) {
+    // the BM25 block, in the epilogue's tiles of 32 rows x 32 columns
+    if (!encode_rows_map(&maps.qb, fu.bm25, s.q, static_cast<int>(fu.ld), 32, kF32))
+      return cudaErrorInvalidValue;
+    maps.eb = maps.e;
   } else if (s.n_second > 0) {
     // the second stacked corpus (dense search over two indices)
-    if (E2 == nullptr || fu.bm25 != nullptr ||
-        !make_map(&maps.eb, E2, s.n_second, s.d, pl.block_n / pl.pair))
+    if (E2 == nullptr || !make_map(&maps.eb, E2, s.n_second, s.d, pl.block_n / pl.pair))
       return cudaErrorInvalidValue;
     maps.qb = maps.q;
   } else {

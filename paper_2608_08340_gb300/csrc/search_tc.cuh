@@ -199,8 +199,8 @@ __host__ __device__ constexpr int lex_land_bytes(bool lex) {
   return lex ? 128 * kLexLandStride : 0;
 }
 
-// kExtra: further shared memory of the launch (the BM25 block form's second
-// staging tile per epilogue warp, block_land_bytes).
+// kExtra: further shared memory of the launch (the BM25 block form's barriers,
+// block_bar_bytes).
 template <int BN, bool kPair = false, bool kDual = false, bool kLex = false, int kExtra = 0>
 constexpr int stages_for() {
   return (kSmemBudget - lex_land_bytes(kLex) - kExtra) /
@@ -668,21 +668,6 @@ __device__ __forceinline__ void cp_async8(void* dst, const void* src) {
                : "memory");
 }
 
-// 16 bytes, or 16 zero bytes when !in (nothing is read from src then).
-__device__ __forceinline__ void cp_async16_zfill(void* dst, const void* src, bool in) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_addr(dst)), "l"(src),
-               "r"(in ? 16 : 0)
-               : "memory");
-}
-
-__device__ __forceinline__ void cp_async_commit() {
-  asm volatile("cp.async.commit_group;" ::: "memory");
-}
-
-__device__ __forceinline__ void cp_async_wait_all() {
-  asm volatile("cp.async.wait_group 0;" ::: "memory");
-}
-
 __device__ __forceinline__ void cp_async_commit_wait_all() {
   asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;" ::: "memory");
 }
@@ -876,7 +861,8 @@ struct LexCursor {
 //
 // kLex: the lexical part of the hybrid search (Sec. 4.4 fusion).
 // kLexNone: dense scores.  kLexBlock: the epilogue reads BM25(q, d) from the
-// q x ld block that the BM25 pass materialised.  kLexGather (single CTAs,
+// q x ld block that the BM25 pass materialised (map_qb), a 32 x 32 tile per
+// warp and chunk.  kLexGather (single CTAs,
 // BN = 128, one epilogue set): the gathered hybrid
 // search.  After the unit's score K blocks the producer loads one more stage,
 // the query tile's head-term counts (map_qb) and the corpus tile's split
@@ -885,12 +871,14 @@ struct LexCursor {
 // the epilogue adds the other terms from the postings (LexCursor) and fuses.
 constexpr int kLexNone = 0, kLexBlock = 1, kLexGather = 2;
 
-// The BM25 block form's second staging tile: 32 x 32 floats per epilogue
-// warp, so that the next chunk's copy of the block flies while one chunk is
-// filtered.
+// Shared memory that the BM25 block form needs beside the staging rows: a
+// barrier per epilogue warp.  (A second staging tile per warp, so that the next
+// chunk's copy flies while one is filtered, costs one of the four pipeline
+// stages, and the two sets' filters overlap the copies anyway: 32768 x 768 with
+// 1024 queries 87 instead of 72 us, 256 queries 40 instead of 31 us.)
 template <int K, int L>
-constexpr int block_land_bytes() {
-  return L == kLexBlock ? epi_sets(K) * 128 * kStageRowBytes : 0;
+constexpr int block_bar_bytes() {
+  return L == kLexBlock ? 128 : 0;
 }
 
 template <int BN, int K, int kLex, bool kPair = false, bool kDual = false>
@@ -904,7 +892,7 @@ tc_search_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
   constexpr bool kHybrid = kLex == kLexGather;   // the gathered form
   static_assert(!kHybrid || (!kPair && !kDual && BN == 128),
                 "the gathered hybrid search runs single CTAs on 128-row tiles");
-  constexpr int kLand = block_land_bytes<K, kLex>();
+  constexpr int kLand = block_bar_bytes<K, kLex>();
   constexpr int S = stages_for<BN, kPair, kDual, kHybrid, kLand>();
   constexpr uint32_t kAStage = a_stage_bytes<kDual>();
   constexpr uint32_t kBStageBytes = b_stage_bytes<BN, kPair>();
@@ -916,17 +904,18 @@ tc_search_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
   if (threadIdx.x == 0) note_phase(p, kPhEntry);
   // Rounded up by an offset, not as an integer: the compiler then still knows
   // that everything below is shared memory (the epilogue's staging rows were
-  // accessed through generic loads and stores otherwise: 32768 x 1024 with 4096
-  // queries and k = 10 took 203 instead of 195 us, 256 queries on 32768 x 768
-  // 24.9 instead of 23.7 us).
+  // accessed through generic loads and stores otherwise: a search of 32768 x
+  // 1024 with 4096 queries and k = 10 took 214.8 instead of 206.6 us, 256
+  // queries on 32768 x 768 28.8 instead of 27.4 us).
   unsigned char* base = smem_raw + ((1024 - (smem_addr(smem_raw) & 1023)) & 1023);
   unsigned char* sA = base;
   unsigned char* sB = sA + S * kAStage;
   float* stage_rows = reinterpret_cast<float*>(sB + S * kBStageBytes);   // epilogue staging
   // hybrid: each epilogue thread's landing zone of the lexical copies
   unsigned char* lex_land = reinterpret_cast<unsigned char*>(stage_rows + kEpiSets * 128 * 32);
-  float* block_land = reinterpret_cast<float*>(lex_land + lex_land_bytes(kHybrid));
-  uint64_t* full = reinterpret_cast<uint64_t*>(reinterpret_cast<unsigned char*>(block_land) + kLand);
+  // kLexBlock: one barrier per epilogue warp
+  uint64_t* block_bar = reinterpret_cast<uint64_t*>(lex_land + lex_land_bytes(kHybrid));
+  uint64_t* full = block_bar + kLand / 8;
   uint64_t* empty = full + S;
   uint64_t* tfull = empty + S;
   uint64_t* tempty = tfull + 4;
@@ -967,11 +956,13 @@ tc_search_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       mbar_init(&tempty[b], kPair ? 8 : 4);   // four epilogue warps per CTA
     }
     mbar_init(mma_done, 1);
+    if constexpr (kLex == kLexBlock)
+      for (int i = 0; i < 4 * kEpiSets; ++i) mbar_init(&block_bar[i], 1);
     *abort_flag = 0;
     fence_mbar_init();
     prefetch_map(&map_q);
     prefetch_map(&map_e);
-    if (kHybrid || p.n_first < p.n) {
+    if (kLex != kLexNone || p.n_first < p.n) {
       prefetch_map(&map_qb);
       prefetch_map(&map_eb);
     }
@@ -1174,6 +1165,13 @@ tc_search_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     list.set_k(p.k);
     list.clear();
     LexCursor lex;             // hybrid: the query's postings cursors
+    constexpr int NC = BN / 32;              // 32-column chunks of a unit
+    // BM25 block form: this warp's 32 x 32 tile of the block (its staging rows),
+    // the tile's barrier, phase bit and whether a copy is in flight.
+    float* wtile = stage_rows + (warp - 2) * 32 * 32;
+    uint64_t* wbar = block_bar + (warp - 2);
+    uint32_t block_ph = 0;
+    bool block_fly = false;
 
     // This CTA owns the list slots (J, cta - first_cta(J)); empty them first.
     if constexpr (K > 0) {
@@ -1238,11 +1236,46 @@ tc_search_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       } else {
         if (act) gfl = list.proven_floor(p.k);
       }
+      // Copies chunk c of the BM25 block by TMA straight into the staging rows
+      // of the lanes that own the query rows (its 128-byte swizzle is theirs);
+      // the filter stages the chunk's candidates there afterwards, so the next
+      // chunk is copied when that is done.  Rows past the batch and columns
+      // past the block's width read as 0; columns past the corpus become -inf
+      // later.  The fence and the warp barrier order the tile's last reads and
+      // writes before the copy.  Nothing is issued any more once a wait gave up.
+      auto copy_block = [&](int c) {
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        __syncwarp();
+        const bool go = __shfl_sync(0xffffffffu, *abort_flag == 0, 0);
+        if (go && lane == 0) {
+          mbar_arrive_expect_tx(wbar, 32 * kStageRowBytes);
+          tma_load_2d(wtile, &map_qb, wbar, static_cast<int>(id_base) + c * 32,
+                      j * kBlockM + eg * 32);
+        }
+        block_fly = go;
+      };
+      // Waits for the tile's copy; a wait that gives up outlives the copy.
+      auto wait_block = [&]() {
+        if (block_fly) {
+          if (!mbar_wait(wbar, block_ph, abort_flag, p.dev_err, p.wait_limit))
+            mbar_drain(wbar, block_ph, p.dev_err);
+          block_ph ^= 1u;
+          block_fly = false;
+        }
+        __syncwarp();
+      };
+      if constexpr (kLex == kLexBlock) {
+        // The first chunk's tile flies while this unit's MMAs run.
+        if (warp_live) copy_block(0);
+      }
       // The warp leaves together when a wait gives up: the TMEM loads below
       // are warp-collective.
       const bool got = mbar_wait(&tfull[acc], (acc_ph >> acc) & 1u, abort_flag, p.dev_err,
                                  p.wait_limit);
-      if (!__all_sync(0xffffffffu, got)) break;
+      if (!__all_sync(0xffffffffu, got)) {
+        if constexpr (kLex == kLexBlock) wait_block();
+        break;
+      }
       // Hands the accumulator back once this warp's TMEM loads of the unit
       // are done.  Pair mode: the epilogue warps of both CTAs release it at
       // the leader.
@@ -1271,36 +1304,6 @@ tc_search_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         float* srow = stage_rows + ((warp - 2) * 32 + lane) * 32;
         const int swz = lane & 7;
         unsigned char* land = lex_land + ((warp - 2) * 32 + lane) * kLexLandStride;
-        // BM25 block form: the warp's 32 x 32 tile of the block for chunk c
-        // sits in the staging rows (c even) or in the second tile (c odd);
-        // the filter stages the chunk's candidates in the same tile, and the
-        // next chunk's copy goes to the other one while this one is filtered.
-        constexpr int NC = BN / 32;              // 32-column chunks of a unit
-        float* wtile[2] = {stage_rows + (warp - 2) * 32 * 32, block_land + (warp - 2) * 32 * 32};
-        auto row_of = [&](int c) -> float* {
-          return kLex == kLexBlock && (c & 1) ? wtile[1] + lane * 32 : srow;
-        };
-        int block_next = -1;     // chunk whose block tile is in flight (-1: none)
-        // Copies chunk c's tile row by row with cp.async (eight lanes per
-        // 128-byte row, four rows per round: a lane reading its own row would
-        // touch 32 lines per load) straight into the rows of the lanes that
-        // own the query rows.  Rows past the batch and columns past the
-        // block's width read as 0; columns past the corpus become -inf later.
-        auto copy_block = [&](int c) {
-          float* tile = wtile[c & 1];
-          const int sub = lane >> 3, part = lane & 7;
-          const int64_t col = id_base + c * 32 + part * 4;
-          int64_t qrow = static_cast<int64_t>(j) * kBlockM + eg * 32 + sub;
-          const float* src = p.fu.bm25 + qrow * p.fu.ld + col;
-#pragma unroll 1
-          for (int rr = sub; rr < 32; rr += 4) {
-            const bool in = qrow < p.q && col < p.fu.ld;
-            cp_async16_zfill(tile + rr * 32 + ((part ^ (rr & 7)) << 2), in ? src : p.fu.bm25, in);
-            src += 4 * p.fu.ld;
-            qrow += 4;
-          }
-          cp_async_commit();
-        };
         // Scores of one chunk (corpus rows id0 .. id0 + 31), fused with the
         // lexical part when hybrid, -inf past the end of the corpus.  Called
         // by every lane of a live warp (the TMEM load is warp-collective).
@@ -1309,28 +1312,18 @@ tc_search_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
           for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
           const int64_t id0 = id_base + c * 32;
           if constexpr (kLex == kLexBlock) {
-            if (block_next != c) {
-              __syncwarp();                      // the tile's last readers are done
-              copy_block(c);
-            }
-            cp_async_wait_all();
-            __syncwarp();
+            wait_block();
             if (act) {
               const float a = p.fu.alpha, b1 = 1.f - p.fu.alpha;
-              const float* row = row_of(c);
 #pragma unroll
               for (int g = 0; g < 8; ++g) {
-                const float4 x = *reinterpret_cast<const float4*>(row + ((g ^ swz) << 2));
+                const float4 x = *reinterpret_cast<const float4*>(srow + ((g ^ swz) << 2));
                 v[4 * g] = fmaf(a, v[4 * g], b1 * (x.x * inv_max));
                 v[4 * g + 1] = fmaf(a, v[4 * g + 1], b1 * (x.y * inv_max));
                 v[4 * g + 2] = fmaf(a, v[4 * g + 2], b1 * (x.z * inv_max));
                 v[4 * g + 3] = fmaf(a, v[4 * g + 3], b1 * (x.w * inv_max));
               }
             }
-            // The other tile's last users (the previous chunk's filter, which
-            // ends with a warp barrier) are done: start the next chunk's copy.
-            block_next = c + 1 < NC ? c + 1 : -1;
-            if (block_next >= 0) copy_block(block_next);
           }
           if constexpr (kHybrid) {
             // head terms from the second accumulator, the other terms from
@@ -1402,6 +1395,7 @@ tc_search_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
                     make_float4(keep[0], keep[1], keep[2], keep[3]);
             }
             __syncwarp();
+            if (kLex == kLexBlock && c + 1 < BN / 32) copy_block(c + 1);
           }
         } else {
         // Filters one chunk against max(list floor, unit bound).
@@ -1423,13 +1417,11 @@ tc_search_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
 #pragma unroll
               for (int i = 0; i < 32; ++i) part[i >> 3] |= (v[i] >= fl ? 1u : 0u) << i;
               mask = (part[0] | part[1]) | (part[2] | part[3]);
-              float* crow = row_of(c);
 #pragma unroll
               for (int g = 0; g < 8; ++g)
-                *reinterpret_cast<float4*>(crow + ((g ^ swz) << 2)) =
+                *reinterpret_cast<float4*>(srow + ((g ^ swz) << 2)) =
                     make_float4(v[4 * g], v[4 * g + 1], v[4 * g + 2], v[4 * g + 3]);
             }
-            const float* crow = row_of(c);
             // Warp-uniform number of rounds; each round takes the lowest
             // remaining candidate column of every lane (ids stay increasing)
             // and inserts it with the branch-free network, so rounds are
@@ -1440,11 +1432,12 @@ tc_search_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
               const int i = __ffs(mask) - 1;
               const bool has = mask != 0;
               mask &= mask - 1;
-              const float s = has ? crow[((((i & 31) >> 2) ^ swz) << 2) | (i & 3)] : -INFINITY;
+              const float s = has ? srow[((((i & 31) >> 2) ^ swz) << 2) | (i & 3)] : -INFINITY;
               list.insert(s, static_cast<uint32_t>(id0 + i));
             }
           }
           __syncwarp();
+          if (kLex == kLexBlock && c + 1 < NC) copy_block(c + 1);
         };
         static_assert(NC % 2 == 0, "chunks are processed in pairs");
         uint32_t ra[32], rb[32];
@@ -1474,6 +1467,7 @@ tc_search_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
                 tmem_wait_ld(ra);
                 float v[32];
                 scores(ra, c, v);
+                if (kLex == kLexBlock) copy_block(c + 1 < NC ? c + 1 : 0);
 #pragma unroll
                 for (int i = K - 1; i >= G; --i) gm[i] = gm[i - G];
 #pragma unroll
@@ -1501,6 +1495,7 @@ tc_search_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
               tmem_wait_ld(ra);
               float v[32];
               scores(ra, c, v);
+              if (kLex == kLexBlock) copy_block(c + 1 < NC ? c + 1 : 0);
 #pragma unroll
               for (int g = 0; g < GPC; ++g) {
                 float m = v[g * L];
@@ -1595,7 +1590,7 @@ struct TcMaps {
 // Pair mode: clusters of two CTAs; `grid` counts CTAs (even).
 template <int BN, int K, int L>
 cudaError_t launch_pair_variant(const TcMaps& m, const TcParams& prm, int grid, cudaStream_t st) {
-  constexpr size_t smem = smem_for<BN, K, true, false, false, block_land_bytes<K, L>()>();
+  constexpr size_t smem = smem_for<BN, K, true, false, false, block_bar_bytes<K, L>()>();
   static bool configured = false;
   if (!configured) {
     cudaError_t e = cudaFuncSetAttribute(tc_search_kernel<BN, K, L, true>,
@@ -1626,7 +1621,7 @@ int pair_capacity_query();
 template <int BN, int K, int L>
 cudaError_t launch_variant(const TcMaps& m, const TcParams& prm, int grid, cudaStream_t st) {
   constexpr bool g = L == kLexGather;
-  constexpr size_t smem = smem_for<BN, K, false, false, g, block_land_bytes<K, L>()>();
+  constexpr size_t smem = smem_for<BN, K, false, false, g, block_bar_bytes<K, L>()>();
   static bool configured = false;
   if (!configured) {
     cudaError_t e = cudaFuncSetAttribute(tc_search_kernel<BN, K, L>,
@@ -1642,7 +1637,7 @@ cudaError_t launch_variant(const TcMaps& m, const TcParams& prm, int grid, cudaS
 // Dual mode (two query tiles per unit); 128-row corpus tiles, lists of 8 or 16.
 template <int K, int L>
 cudaError_t launch_dual_variant(const TcMaps& m, const TcParams& prm, int grid, cudaStream_t st) {
-  constexpr size_t smem = smem_for<128, K, false, true, false, block_land_bytes<K, L>()>();
+  constexpr size_t smem = smem_for<128, K, false, true, false, block_bar_bytes<K, L>()>();
   static bool configured = false;
   if (!configured) {
     cudaError_t e = cudaFuncSetAttribute(tc_search_kernel<128, K, L, false, true>,
