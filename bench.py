@@ -432,8 +432,8 @@ def measure(args, cfg: int, batch: int, rank: int, world: int, local_rank: int,
             idx.search(Q, w.k, out=(ids, scores))
             last["out"] = (ids, scores)
 
-    # our kernels per step: search + merge; k > 32 over many tiles adds the
-    # group pass and selection of k > 32; config 3 adds the BM25 pass
+    # our kernels per step: search + merge; k > 32 adds its group pass and
+    # selection; config 3 adds the BM25 pass
     # (dense-first: the rerank), config 4 the upsert scatter.
     for i in range(args.warmup):
         flush.zero_()
@@ -442,7 +442,9 @@ def measure(args, cfg: int, batch: int, rank: int, world: int, local_rank: int,
     idx.check()
     t = idx.last_timing()
     sampled = t["sample_ms"] > 0.0
-    launches_per_step = 2 + (2 if sampled else 0) + (1 if cfg in (3, 4) else 0)
+    # (a search of up to 6 queries and k <= 8 merges in its search kernel)
+    inline = idx.last_path == "tc" and w.q <= 6 and w.k <= 8 and cfg != 3
+    launches_per_step = (1 if inline else 2) + (2 if sampled else 0) + (1 if cfg in (3, 4) else 0)
 
     if world > 1:
         torch.distributed.barrier()

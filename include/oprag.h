@@ -261,9 +261,11 @@ OPRAG_API int oprag_index_set_option(oprag_index *idx, int32_t option, int32_t v
  * own (M = 128 MMAs), one query tile per unit.  3 (dual mode) runs every CTA
  * on its own with two query tiles per unit that share each corpus tile
  * (128-row tiles; k <= 16 and more than 128 queries, ignored otherwise).
- * 0 (default) chooses dual mode when its units come to at most four per CTA,
- * CTA pairs for k > 32 with at least 1024 queries on 256-row tiles, single
- * CTAs otherwise. */
+ * 0 (default) chooses a kernel of its own for dense searches of up to 32
+ * queries with k <= 16 (corpus rows on the MMA's M side), dual mode when its
+ * units come to at most four per CTA and for hybrid searches with a BM25
+ * block, CTA pairs for k > 32 with at least 1024 queries on 256-row tiles,
+ * single CTAs otherwise. */
 #define OPRAG_OPT_PAIR 4
 
 /* OPRAG_OPT_BOUND_TAG (test hook): sets the 32-bit tag of the last search's

@@ -186,6 +186,25 @@ cudaError_t launch_tc_search(const void* E, const void* Q, const SearchShape& s,
                              const void* E2 = nullptr);
 constexpr int kTcPhases = 8;
 
+// --- tensor-core search of small batches (search_small.cu): one slice of the
+// corpus per CTA, queries on the MMA's N side.
+constexpr int kSmallMaxQueries = 32;
+struct SmallPlan {
+  int box;            // corpus rows per tile
+  int64_t slice;      // corpus rows per CTA
+  int grid;
+  bool inline_merge;  // the search kernel writes the final results itself
+};
+bool small_applies(const SearchShape& s);
+SmallPlan small_plan(const SearchShape& s, int num_sms);
+size_t small_scratch_bytes(const SearchShape& s, const SmallPlan& pl);
+// done: a zeroed counter that the launches of one index share (it returns to
+// zero by the end of every launch).
+cudaError_t launch_small_search(const void* E, const void* Q, const SearchShape& s,
+                                const SmallPlan& pl, void* scratch, int* dev_err,
+                                unsigned int* done, long long wait_limit, int64_t* out_ids,
+                                float* out_scores, ListSet* lists, cudaStream_t st);
+
 // Group pass: a search launch whose scratch receives, instead of lists, the
 // group maxima (q rows of tc_group_count floats, see TcParams::gmax).
 int64_t tc_group_count(const SearchShape& s, const TcPlan& p);

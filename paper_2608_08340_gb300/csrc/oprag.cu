@@ -70,7 +70,7 @@ struct oprag_index {
   int d = 0;
   int dtype = OPRAG_BF16;
   void* emb = nullptr;
-  int* dev_err = nullptr;
+  int* dev_err = nullptr;        // error word, then the small searches' CTA counter
   int* err_host = nullptr;       // pinned copy of dev_err, read after host-buffer calls
   cudaEvent_t done = nullptr;
 
@@ -298,6 +298,8 @@ struct SearchLayout {
   int path = 0;           // 1 SIMT, 2 tensor core
   int simt_grid = 0;      // CTAs (bf16) or corpus slices (fp32) of path 1
   TcPlan plan{}, splan{};
+  bool small = false;       // small batch (search_small.cu)
+  SmallPlan splan_small{};
   bool sampled = false;     // a group pass runs first
   SearchShape gshape{};     // its shape
   size_t main_bytes = 0;    // multiple of 256
@@ -328,6 +330,14 @@ SearchLayout search_layout(oprag_index* idx, int q, int k, int path, int block_n
       L.simt_grid = simt_grid(s, idx->num_sms);
       L.main_bytes = round256(simt_scratch_bytes(s, L.simt_grid));
     }
+    return L;
+  }
+  // Small batches, unless a tile width, a CTA mode or phase stamps ask for the
+  // general kernel.
+  if (block_n == 0 && pair == 0 && !idx->phases_on && small_applies(s)) {
+    L.small = true;
+    L.splan_small = small_plan(s, idx->num_sms);
+    L.main_bytes = round256(small_scratch_bytes(s, L.splan_small));
     return L;
   }
   L.plan = tc_plan(s, idx->num_sms, block_n, 1, pair, pair_capacity(idx));
@@ -379,6 +389,10 @@ int launch_search(oprag_index* idx, const SearchLayout& L, const void* Q, int q,
             ? launch_f32_search(idx->emb, Q, s, fu, scratch, L.simt_grid, &lists, st, qf, gen,
                                 idx->dev_err, idx->wait_limit)
             : launch_simt_search(idx->emb, Q, s, fu, scratch, L.simt_grid, &lists, st);
+  } else if (L.small) {
+    e = launch_small_search(idx->emb, Q, s, L.splan_small, scratch, idx->dev_err,
+                            reinterpret_cast<unsigned int*>(idx->dev_err) + 1, idx->wait_limit,
+                            out_ids, out_scores, &lists, st);
   } else {
     const float* floor = nullptr;
     float* levels = nullptr;
@@ -414,13 +428,22 @@ int launch_search(oprag_index* idx, const SearchLayout& L, const void* Q, int q,
   }
   if (e != cudaSuccess) return cuda_fail(e, "search kernel");
   if (idx->timing) cudaEventRecord(idx->ev[2], st);
-  note_launch(idx, L.path, L.plan);
+  if (L.small) {
+    idx->last_grid = L.splan_small.grid;
+    idx->last_cluster = 1;
+    idx->last_block_n = 128;
+    idx->last_tiles = 1;
+  } else {
+    note_launch(idx, L.path, L.plan);
+  }
   if (out_src != nullptr) {
     lists.split = idx->n;
     lists.out_src = out_src;
   }
-  e = launch_merge(lists, q, k, out_ids, out_scores, st);
-  if (e != cudaSuccess) return cuda_fail(e, "merge kernel");
+  if (!L.small || !L.splan_small.inline_merge) {
+    e = launch_merge(lists, q, k, out_ids, out_scores, st);
+    if (e != cudaSuccess) return cuda_fail(e, "merge kernel");
+  }
   if (idx->timing) cudaEventRecord(idx->ev[3], st);
   idx->timed = idx->timing;
   idx->last_path = L.path;
@@ -537,7 +560,7 @@ int oprag_index_create(oprag_index** out, const void* emb, int64_t n, int32_t d,
     idx->emb = nullptr;
     return bail(fail(OPRAG_ERR_OOM, "cannot allocate %zu bytes for the index", bytes));
   }
-  if (cudaMalloc(reinterpret_cast<void**>(&idx->dev_err), sizeof(int)) != cudaSuccess) {
+  if (cudaMalloc(reinterpret_cast<void**>(&idx->dev_err), 2 * sizeof(int)) != cudaSuccess) {
     cudaGetLastError();
     idx->dev_err = nullptr;
     return bail(fail(OPRAG_ERR_OOM, "cannot allocate the error word"));
@@ -553,7 +576,7 @@ int oprag_index_create(oprag_index** out, const void* emb, int64_t n, int32_t d,
   cudaStream_t st;
   if ((e = cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking)) != cudaSuccess)
     return bail(cuda_fail(e, "stream"));
-  e = cudaMemsetAsync(idx->dev_err, 0, sizeof(int), st);
+  e = cudaMemsetAsync(idx->dev_err, 0, 2 * sizeof(int), st);
   if (e == cudaSuccess) {
     if (src_dtype == dtype) {
       e = cudaMemcpyAsync(idx->emb, emb, bytes, emb_on_device ? cudaMemcpyDeviceToDevice
