@@ -5,6 +5,7 @@
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
+#include <memory>
 #include <mutex>
 #include <string>
 #include <thread>
@@ -59,6 +60,12 @@ struct DeviceGuard {
 constexpr int kSimtMaxQueriesBf16 = 0;
 // Largest BM25 matrix block (floats) materialised per hybrid pass.
 constexpr int64_t kLexMaxElems = int64_t(1) << 28;
+// Results of a host-buffer search up to this size are written by the device
+// into pinned memory of the index and copied out by the host: no device to
+// host copies to enqueue and to wait for (three of them took 10 us of a 32-query
+// search).
+constexpr size_t kHostResultBytes = 64 * 1024;
+constexpr size_t kHostResultOffset = 64;
 
 }  // namespace
 
@@ -70,8 +77,12 @@ struct oprag_index {
   int d = 0;
   int dtype = OPRAG_BF16;
   void* emb = nullptr;
-  int* dev_err = nullptr;        // error word, then the small searches' CTA counter
-  int* err_host = nullptr;       // pinned copy of dev_err, read after host-buffer calls
+  // Pinned host memory that the device writes: the error word (dev_err is its
+  // device address; kernels write it only when they give up a wait), then the
+  // results of small host-buffer searches (kHostResultOffset).
+  int* err_host = nullptr;
+  int* dev_err = nullptr;
+  unsigned int* cta_count = nullptr;   // the small searches' CTA counter (device)
   cudaEvent_t done = nullptr;
 
   void* scratch = nullptr;     // partial top-k lists
@@ -128,6 +139,7 @@ struct oprag_index {
   size_t qfloor_bytes = 0;
   uint32_t gen = 0;
   int pair_cap = -1;       // clusters of two search CTAs that fit at once (-1: not asked yet)
+  std::shared_ptr<void> layouts;   // LayoutCache: the last searches' layouts
   int last_path = 0;
   int last_grid = 0, last_cluster = 0, last_block_n = 0;   // last main search kernel launch
   int last_tiles = 0;                                         // query tiles per CTA and unit
@@ -313,8 +325,8 @@ size_t round256(size_t b) { return (b + 255) / 256 * 256; }
 // Lexical part of a search: none, a materialised BM25 block, or gathered.
 enum class LexForm { kNone, kBlock, kGather };
 
-SearchLayout search_layout(oprag_index* idx, int q, int k, int path, int block_n, int pair,
-                           LexForm lex = LexForm::kNone, int64_t n_second = 0) {
+SearchLayout plan_layout(oprag_index* idx, int q, int k, int path, int block_n, int pair,
+                         LexForm lex, int64_t n_second) {
   SearchLayout L;
   SearchShape s{idx->n, idx->d, q, k};
   s.fused_lex = lex == LexForm::kGather && path == 2;
@@ -364,6 +376,44 @@ SearchLayout search_layout(oprag_index* idx, int q, int k, int path, int block_n
   return L;
 }
 
+// The layouts of the last few shapes are kept: a plan replays its schedule on
+// the host (2 us at 32768 rows, 28 us at 1M rows and 2048 queries).
+struct LayoutCache {
+  static constexpr int kEntries = 4;
+  struct Entry {
+    int64_t n = -1, n_second = 0;
+    int q = 0, k = 0, path = 0, block_n = 0, pair = 0;
+    LexForm lex = LexForm::kNone;
+    bool phases = false;
+    SearchLayout layout;
+  } entry[kEntries];
+  int next = 0;
+};
+
+SearchLayout search_layout(oprag_index* idx, int q, int k, int path, int block_n, int pair,
+                           LexForm lex = LexForm::kNone, int64_t n_second = 0) {
+  if (!idx->layouts) idx->layouts = std::make_shared<LayoutCache>();
+  LayoutCache& c = *std::static_pointer_cast<LayoutCache>(idx->layouts);
+  for (const LayoutCache::Entry& e : c.entry)
+    if (e.n == idx->n && e.n_second == n_second && e.q == q && e.k == k && e.path == path &&
+        e.block_n == block_n && e.pair == pair && e.lex == lex && e.phases == idx->phases_on)
+      return e.layout;
+  LayoutCache::Entry& e = c.entry[c.next];
+  c.next = (c.next + 1) % LayoutCache::kEntries;
+  e.n = -1;
+  e.layout = plan_layout(idx, q, k, path, block_n, pair, lex, n_second);
+  e.n_second = n_second;
+  e.q = q;
+  e.k = k;
+  e.path = path;
+  e.block_n = block_n;
+  e.pair = pair;
+  e.lex = lex;
+  e.phases = idx->phases_on;
+  e.n = idx->n;
+  return e.layout;
+}
+
 SearchLayout search_layout(oprag_index* idx, int q, int k, LexForm lex = LexForm::kNone) {
   return search_layout(idx, q, k, choose_path(idx, q), idx->opt_block_n, idx->opt_pair, lex);
 }
@@ -391,8 +441,7 @@ int launch_search(oprag_index* idx, const SearchLayout& L, const void* Q, int q,
             : launch_simt_search(idx->emb, Q, s, fu, scratch, L.simt_grid, &lists, st);
   } else if (L.small) {
     e = launch_small_search(idx->emb, Q, s, L.splan_small, scratch, idx->dev_err,
-                            reinterpret_cast<unsigned int*>(idx->dev_err) + 1, idx->wait_limit,
-                            out_ids, out_scores, &lists, st);
+                            idx->cta_count, idx->wait_limit, out_ids, out_scores, &lists, st);
   } else {
     const float* floor = nullptr;
     float* levels = nullptr;
@@ -560,14 +609,16 @@ int oprag_index_create(oprag_index** out, const void* emb, int64_t n, int32_t d,
     idx->emb = nullptr;
     return bail(fail(OPRAG_ERR_OOM, "cannot allocate %zu bytes for the index", bytes));
   }
-  if (cudaMalloc(reinterpret_cast<void**>(&idx->dev_err), 2 * sizeof(int)) != cudaSuccess) {
+  if (cudaMalloc(reinterpret_cast<void**>(&idx->cta_count), sizeof(int)) != cudaSuccess) {
     cudaGetLastError();
-    idx->dev_err = nullptr;
-    return bail(fail(OPRAG_ERR_OOM, "cannot allocate the error word"));
+    idx->cta_count = nullptr;
+    return bail(fail(OPRAG_ERR_OOM, "cannot allocate the CTA counter"));
   }
-  if (cudaMallocHost(reinterpret_cast<void**>(&idx->err_host), sizeof(int)) != cudaSuccess) {
+  if (cudaHostAlloc(reinterpret_cast<void**>(&idx->err_host), kHostResultOffset + kHostResultBytes,
+                    cudaHostAllocMapped) != cudaSuccess ||
+      cudaHostGetDevicePointer(reinterpret_cast<void**>(&idx->dev_err), idx->err_host, 0) !=
+          cudaSuccess) {
     cudaGetLastError();
-    idx->err_host = nullptr;
     return bail(fail(OPRAG_ERR_OOM, "cannot allocate the pinned error word"));
   }
   *idx->err_host = 0;
@@ -576,7 +627,7 @@ int oprag_index_create(oprag_index** out, const void* emb, int64_t n, int32_t d,
   cudaStream_t st;
   if ((e = cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking)) != cudaSuccess)
     return bail(cuda_fail(e, "stream"));
-  e = cudaMemsetAsync(idx->dev_err, 0, 2 * sizeof(int), st);
+  e = cudaMemsetAsync(idx->cta_count, 0, sizeof(int), st);
   if (e == cudaSuccess) {
     if (src_dtype == dtype) {
       e = cudaMemcpyAsync(idx->emb, emb, bytes, emb_on_device ? cudaMemcpyDeviceToDevice
@@ -612,7 +663,7 @@ void oprag_index_destroy(oprag_index* idx) {
   DeviceGuard g(idx->device);
   idx->drain();
   if (idx->emb) cudaFree(idx->emb);
-  if (idx->dev_err) cudaFree(idx->dev_err);
+  if (idx->cta_count) cudaFree(idx->cta_count);
   if (idx->err_host) cudaFreeHost(idx->err_host);
   if (idx->gcache.exec) cudaGraphExecDestroy(idx->gcache.exec);
   if (idx->scratch) cudaFree(idx->scratch);
@@ -970,29 +1021,34 @@ int oprag_search_host(oprag_index* idx, const void* queries, int32_t q, int32_t 
   const size_t q_off = 0;
   const size_t id_off = (qbytes + 255) / 256 * 256;
   const size_t sc_off = id_off + (static_cast<size_t>(q) * k * sizeof(int64_t) + 255) / 256 * 256;
-  const size_t need = sc_off + static_cast<size_t>(q) * k * sizeof(float);
+  const size_t results = static_cast<size_t>(q) * k;
+  const bool direct = results * (sizeof(int64_t) + sizeof(float)) <= kHostResultBytes;
+  const size_t need = direct ? qbytes : sc_off + results * sizeof(float);
   if ((rc = idx->ensure(&idx->stage, &idx->stage_bytes, need, "search staging"))) return rc;
   if ((rc = begin_call(idx, st))) return rc;
   char* stage = static_cast<char*>(idx->stage);
   cudaError_t e = cudaMemcpyAsync(stage + q_off, queries, qbytes, cudaMemcpyHostToDevice, st);
   if (e != cudaSuccess) return cuda_fail(e, "copying queries");
   const Fusion none{nullptr, 0, nullptr, 0.f};
-  if ((rc = run_search(idx, stage + q_off, q, k, none, reinterpret_cast<int64_t*>(stage + id_off),
-                       reinterpret_cast<float*>(stage + sc_off), st)))
-    return rc;
-  e = cudaMemcpyAsync(out_ids, stage + id_off, static_cast<size_t>(q) * k * sizeof(int64_t),
-                      cudaMemcpyDeviceToHost, st);
-  if (e == cudaSuccess)
-    e = cudaMemcpyAsync(out_scores, stage + sc_off, static_cast<size_t>(q) * k * sizeof(float),
-                        cudaMemcpyDeviceToHost, st);
-  // The error word travels with the results, so that the call waits for the
-  // device once.
-  if (e == cudaSuccess)
-    e = cudaMemcpyAsync(idx->err_host, idx->dev_err, sizeof(int), cudaMemcpyDeviceToHost, st);
-  if (e != cudaSuccess) return cuda_fail(e, "copying results");
+  char* result = direct ? reinterpret_cast<char*>(idx->dev_err) + kHostResultOffset : stage + id_off;
+  int64_t* ids = reinterpret_cast<int64_t*>(result);
+  float* scores = reinterpret_cast<float*>(direct ? result + results * sizeof(int64_t)
+                                                  : stage + sc_off);
+  if ((rc = run_search(idx, stage + q_off, q, k, none, ids, scores, st))) return rc;
+  if (!direct) {
+    e = cudaMemcpyAsync(out_ids, ids, results * sizeof(int64_t), cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess)
+      e = cudaMemcpyAsync(out_scores, scores, results * sizeof(float), cudaMemcpyDeviceToHost, st);
+    if (e != cudaSuccess) return cuda_fail(e, "copying results");
+  }
   if ((rc = end_call(idx, st))) return rc;
   if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return cuda_fail(e, "search");
-  return *idx->err_host != 0 ? oprag_index_check(idx) : ok();
+  if (direct) {
+    const char* host = reinterpret_cast<const char*>(idx->err_host) + kHostResultOffset;
+    std::memcpy(out_ids, host, results * sizeof(int64_t));
+    std::memcpy(out_scores, host + results * sizeof(int64_t), results * sizeof(float));
+  }
+  return *static_cast<volatile int*>(idx->err_host) != 0 ? oprag_index_check(idx) : ok();
 }
 
 // Builds the device side of BM25 from the index's host copy of the token
@@ -1412,11 +1468,9 @@ int oprag_index_check(oprag_index* idx) {
   DeviceGuard g(idx->device);
   cudaError_t e = idx->drain();
   if (e != cudaSuccess) return cuda_fail(e, "pending work");
-  int flag = 0;
-  e = cudaMemcpy(&flag, idx->dev_err, sizeof(int), cudaMemcpyDeviceToHost);
-  if (e != cudaSuccess) return cuda_fail(e, "reading the error word");
+  const int flag = *static_cast<volatile int*>(idx->err_host);
   if (flag != 0) {
-    cudaMemset(idx->dev_err, 0, sizeof(int));
+    *idx->err_host = 0;
     return fail(OPRAG_ERR_DEVICE, "a kernel gave up a bounded wait (code %d)", flag);
   }
   return ok();

@@ -21,7 +21,9 @@ _DT = {torch.float32: OPRAG_F32, torch.bfloat16: OPRAG_BF16}
 
 def _stream_ptr(stream) -> int:
     if stream is None:
-        stream = torch.cuda.current_stream()
+        # torch.cuda.current_stream().cuda_stream without its Stream object
+        # (3 us of a call, as long as the search call itself takes the host).
+        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
     return int(stream.cuda_stream)
 
 
