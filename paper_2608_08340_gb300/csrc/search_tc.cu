@@ -34,11 +34,19 @@ TcPlan tc_plan(const SearchShape& s, int num_sms, int force_block_n, int tile_st
   } else if (force_block_n == 128 || force_block_n == 256) {
     bn = force_block_n;
   } else {
-    // Few units (small query batches): 128-row tiles give every SM more of
-    // them; the MMA rate per row is the same for N = 128 and N = 256.
-    const int64_t units256 =
-      static_cast<int64_t>(pl.qt) * ((s.n + 255) / 256 + (s.n_second + 255) / 256);
-    if (units256 < 4LL * num_sms) bn = 128;
+    // 256-row tiles (half the query tile copies per row) unless there are few
+    // units and the busiest CTA would scan a fifth fewer rows in 128-row tiles.
+    // Measured, search kernel with 128- / 256-row tiles: 32768 x 768, 40 queries
+    // (2 x 128 rows against 256) 21.0 / 18.7 us; 50021 x 392, 40 queries (3 x
+    // 128 against 2 x 256) 21.0 / 24.5 us; 50021 x 392, 300 queries, k = 50 (as
+    // many rows) 35.5 / 31.4 us, 600 queries (7% fewer) 53.2 / 45.7 us.  With a
+    // BM25 block small batches keep 128 (32768 x 768, 64 queries: 23.2 / 25.2).
+    auto units = [&](int b) {
+      const int64_t tiles = (s.n + b - 1) / b + (s.n_second + b - 1) / b;
+      return pl.qt * ((tiles + tile_stride - 1) / tile_stride);
+    };
+    auto rows = [&](int b) { return (units(b) + num_sms - 1) / num_sms * b; };
+    if (units(256) < 4LL * num_sms && (s.lex_block || rows(128) * 5 < rows(256) * 4)) bn = 128;
   }
   // Dual mode: every unit takes two query tiles and one 128-row corpus tile,
   // so a CTA reads each corpus tile once for 256 queries, and its four
