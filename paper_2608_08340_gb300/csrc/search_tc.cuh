@@ -1161,6 +1161,8 @@ tc_search_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       const int pc = cta - first_cta(J, p.qt, C);
       return pc >= 0 && pc < per_tile;
     };
+    // The floors of a preceding selection kernel (see dependent_attr).
+    if constexpr (K > 32) asm volatile("griddepcontrol.wait;" ::: "memory");
     EpiList<K> list;
     list.set_k(p.k);
     list.clear();
@@ -1587,6 +1589,16 @@ struct TcMaps {
   CUtensorMap q, e, qb, eb;
 };
 
+// The main pass of a search with a group pass is a programmatic dependent of
+// the selection kernel: its copies and MMAs start while the floors are still
+// being selected, and its epilogue waits for them (griddepcontrol.wait).
+inline cudaLaunchAttribute dependent_attr() {
+  cudaLaunchAttribute a{};
+  a.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  a.val.programmaticStreamSerializationAllowed = 1;
+  return a;
+}
+
 // Pair mode: clusters of two CTAs; `grid` counts CTAs (even).
 template <int BN, int K, int L>
 cudaError_t launch_pair_variant(const TcMaps& m, const TcParams& prm, int grid, cudaStream_t st) {
@@ -1604,13 +1616,14 @@ cudaError_t launch_pair_variant(const TcMaps& m, const TcParams& prm, int grid, 
   cfg.blockDim = dim3(threads_for(K));
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = 2;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
+  attr[1] = dependent_attr();
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = prm.init_floor != nullptr ? 2 : 1;
   return cudaLaunchKernelEx(&cfg, tc_search_kernel<BN, K, L, true>, m.q, m.e, m.qb, m.eb, prm);
 }
 
@@ -1630,8 +1643,15 @@ cudaError_t launch_variant(const TcMaps& m, const TcParams& prm, int grid, cudaS
     if (e != cudaSuccess) return e;
     configured = true;
   }
-  tc_search_kernel<BN, K, L><<<grid, threads_for(K, g), smem, st>>>(m.q, m.e, m.qb, m.eb, prm);
-  return cudaGetLastError();
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(threads_for(K, g));
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1] = {dependent_attr()};
+  cfg.attrs = attr;
+  cfg.numAttrs = prm.init_floor != nullptr ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, tc_search_kernel<BN, K, L>, m.q, m.e, m.qb, m.eb, prm);
 }
 
 // Dual mode (two query tiles per unit); 128-row corpus tiles, lists of 8 or 16.

@@ -30,7 +30,9 @@ group_select_kernel(const float* __restrict__ gmax, int64_t gld, int groups, int
   __shared__ int part[2][kSelWarps];
   __shared__ uint32_t top[kSelTop];
   __shared__ int ntop;
-  // Launched as a programmatic dependent of the group pass.
+  // Launched as a programmatic dependent of the group pass; the main pass may
+  // start once every CTA of this grid has.
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   asm volatile("griddepcontrol.wait;" ::: "memory");
   const int qi = blockIdx.x, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const float* g = gmax + static_cast<int64_t>(qi) * gld;
