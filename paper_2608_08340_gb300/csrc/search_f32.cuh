@@ -21,10 +21,10 @@
 // batch (config_for): TY = 4 (256 corpus rows) up to 32 queries, TY = 8 up to
 // 64, TY = 16 above.  Measured on GB300, 32768 x 768 and k = 10, search kernel,
 // against the streaming kernel this one replaced (each chunk of eight queries
-// streamed the corpus again, five shuffles per score): 1 query 29 (51) us, 16
-// queries 43 (92) us, 100 queries 182 (528) us or 27.7 TFLOP/s, 256 queries
-// 366 (1298) us; 100000 x 768 and 1 query 63 (119) us or 4.9 TB/s; 100 queries
-// and k = 100 272 (1542) us.
+// streamed the corpus again, five shuffles per score): 1 query 28 (51) us, 16
+// queries 42 (92) us, 100 queries 176 (528) us or 28.5 TFLOP/s, 256 queries
+// 356 (1298) us; 100000 x 768 and 1 query 63 (119) us or 4.9 TB/s; 100 queries
+// and k = 100 270 (1542) us.
 //
 // Selection.  Each query of the tile has a buffer of candidate keys in shared
 // memory.  A score enters it when it reaches the query's floor: the k-th
@@ -317,16 +317,25 @@ f32_search_kernel(const __grid_constant__ CUtensorMap map_q,
         ph ^= 1u;
       }
       if ((kb + 1) % kFoldBlocks == 0 || kb + 1 == nkb) {
-        // the two second-level sums swap, so that each takes every other fold
+        // Every other fold goes to the other second-level sum.  (A branch: the
+        // swap of the two arrays in registers took 6% of the kernel.)
+        if ((kb / kFoldBlocks) & 1) {
 #pragma unroll
-        for (int i = 0; i < TM; ++i)
+          for (int i = 0; i < TM; ++i)
 #pragma unroll
-          for (int j = 0; j < kRowsPerThread; ++j) {
-            const float t = tot[0][i][j] + acc[i][j];
-            tot[0][i][j] = tot[1][i][j];
-            tot[1][i][j] = t;
-            acc[i][j] = 0.f;
-          }
+            for (int j = 0; j < kRowsPerThread; ++j) {
+              tot[1][i][j] += acc[i][j];
+              acc[i][j] = 0.f;
+            }
+        } else {
+#pragma unroll
+          for (int i = 0; i < TM; ++i)
+#pragma unroll
+            for (int j = 0; j < kRowsPerThread; ++j) {
+              tot[0][i][j] += acc[i][j];
+              acc[i][j] = 0.f;
+            }
+        }
       }
     }
 
@@ -384,16 +393,31 @@ f32_search_kernel(const __grid_constant__ CUtensorMap map_q,
     }
     // The previous tile's compactions and the floors are done.
     __syncthreads();
+    // One slot reservation per thread and query, all of them in flight before
+    // the first key is stored (a returning atomic per score took 5 us more of
+    // 100 queries' search).
+    int at[TM];
+    uint32_t take = 0;                 // bit 4 i + j: the score enters
+    static_assert(TM * kRowsPerThread <= 32, "one mask bit per score");
 #pragma unroll
     for (int i = 0; i < TM; ++i) {
       const int ql = ty + TY * i;
-      const bool qv = q0 + ql < p.q;
       const float fl = order_score(flo[ql]);
+      uint32_t m = 0;
 #pragma unroll
       for (int j = 0; j < kRowsPerThread; ++j)
-        if (acc[i][j] >= fl && qv && r0 + tx + TX * j < r_end)
-          buf[ql * p.cap + atomicAdd(cnt + ql, 1)] =
-              make_key(acc[i][j], static_cast<uint32_t>(r0 + tx + TX * j));
+        if (acc[i][j] >= fl && r0 + tx + TX * j < r_end) m |= 1u << j;
+      if (q0 + ql >= p.q) m = 0;
+      at[i] = m != 0 ? atomicAdd(cnt + ql, __popc(m)) : 0;
+      take |= m << (kRowsPerThread * i);
+    }
+#pragma unroll
+    for (int i = 0; i < TM; ++i) {
+      uint64_t* b = buf + (ty + TY * i) * p.cap + at[i];
+#pragma unroll
+      for (int j = 0; j < kRowsPerThread; ++j)
+        if ((take >> (kRowsPerThread * i + j)) & 1u)
+          *b++ = make_key(acc[i][j], static_cast<uint32_t>(r0 + tx + TX * j));
     }
     __syncthreads();
     // Buffers without room for another tile, or of the last tile: keep the k
