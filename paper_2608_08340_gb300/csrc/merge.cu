@@ -4,47 +4,14 @@
 // local candidates to the global top-k, done inside one GPU: the producers
 // are corpus slices instead of index shards.
 //
-// Four merges: for unsorted lists (buffered tensor-core lists, k > 32) one warp
-// per query over all their keys; otherwise for sorted lists, by list count and k, one
-// warp per query over at most 32 lists (head by head), one to four warps per
-// query over up to 512 lists when k <= 16 (also head by head), and the block
-// merge of merge.cuh (one CTA per query).
+// Three merges: for unsorted lists (buffered tensor-core lists, k > 32) one warp
+// per query over all their keys; for sorted lists head by head, one warp per
+// query over at most 32 lists, one to four warps per query over up to 512.
 #include "merge.cuh"
 
 namespace oprag {
 
 namespace {
-
-constexpr int kMergeWarps = 8;
-
-template <int KP>
-__global__ void __launch_bounds__(kMergeWarps * 32)
-merge_kernel(ListSet ls, int q, int k, int64_t* __restrict__ out_ids,
-             float* __restrict__ out_scores) {
-  extern __shared__ __align__(16) uint64_t smem_keys[];
-  // Launched as a programmatic dependent of the search kernel: wait until
-  // that grid has finished and its lists are visible.
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-  const int qi = blockIdx.x;
-  if (qi >= q) return;
-  merge_one_query<KP>(ls, qi, k, kMergeWarps, out_ids, out_scores, smem_keys);
-}
-
-template <int KP>
-cudaError_t launch_merge_kp(const ListSet& ls, int q, int k, int64_t* ids, float* scores, cudaStream_t st) {
-  const size_t smem = static_cast<size_t>(kMergeWarps + 1) * 2 * KP * sizeof(uint64_t);
-  cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3(q);
-  cfg.blockDim = dim3(kMergeWarps * 32);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, merge_kernel<KP>, ls, q, k, ids, scores);
-}
 
 // Few lists per query (at most 32): one warp per query merges the sorted
 // lists directly.  Lane l holds the head of list l (with the next keys
@@ -104,19 +71,21 @@ merge_kway_kernel(ListSet ls, int q, int k, int64_t* __restrict__ out_ids,
   }
 }
 
-// More than 32 lists and k <= 16, at most kSmallLists lists per lane: W
-// warps per query (W = 1, 2 or 4 by list count; CTAs of four warps, 4 / W
-// queries each).
-// Launched early (programmatic dependent
-// launch), a CTA waits in place and starts as soon as the search grid ends.
-// Lane l of warp w holds lists p = 32 w + l + 32 W u (u < kSmallLists): the
-// first kSmallKeys keys of each, fetched with 16-byte loads all issued
-// together.  Then the query's 32 W lanes take the k best head by head:
-// each round the lanes' best heads go through a warp maximum (and, when
-// W > 1, a maximum over the query's warps in shared memory); keys are
-// unique, so one lane owns the winner and advances that list (fetching its
-// next keys once the held ones are used up, which only k > kSmallKeys can
-// need).
+// More than 32 sorted lists, at most kSmallLists lists per lane: W warps per
+// query (W = 1, 2 or 4 by list count; CTAs of four warps, 4 / W queries each).
+// Launched early (programmatic dependent launch), a CTA waits in place and
+// starts as soon as the search grid ends.  Lane l of warp w holds lists p =
+// 32 w + l + 32 W u (u < kSmallLists): the first kSmallKeys keys of each,
+// fetched with 16-byte loads all issued together.  Then the query's 32 W lanes
+// take the k best head by head: each round the lanes' best heads go through a
+// warp maximum (and, when W > 1, a maximum over the query's warps in shared
+// memory); keys are unique, so one lane owns the winner and advances that list
+// (fetching its next keys once the held ones are used up, which only k >
+// kSmallKeys can need).  A round takes about 0.15 us, and few lists are drawn
+// on beyond their first keys, so this holds up to k = 256: measured on GB300,
+// 16 queries over 152 lists, against a CTA per query that filtered all P k keys
+// through sorted buffers: k = 32 13 (56) us, k = 100 27 (76) us, k = 256 60
+// (191) us; 1000 queries k = 32 11 (224) us.
 constexpr int kSmallThreads = 128;
 constexpr int kSmallLists = 4;
 constexpr int kSmallKeys = 6;
@@ -333,12 +302,12 @@ cudaError_t launch_small_w(const ListSet& ls, int q, int k, int64_t* out_ids, fl
 // Warps per query of merge_small_kernel: the fewest whose lanes hold all of
 // a query's lists (kSmallLists each).  The lists' loads are issued together
 // whatever W is, and with one warp per query the head-by-head rounds need no
-// barrier.  Returns cudaErrorNotSupported when four warps do not suffice (the
-// caller then takes the block merge).
+// barrier.
 cudaError_t launch_small(const ListSet& ls, int q, int k, int64_t* out_ids, float* out_scores, cudaStream_t st) {
   constexpr int kPerWarp = kSmallLists * 32;
   const int W = ls.P <= kPerWarp ? 1 : ls.P <= 2 * kPerWarp ? 2 : 4;
-  if (ls.P > W * kPerWarp) return cudaErrorNotSupported;
+  // (at most three slices or two epilogue sets per SM: 456 lists on 152 SMs)
+  if (ls.P > W * kPerWarp) return cudaErrorInvalidValue;
   if (W == 4) return launch_small_w<4>(ls, q, k, out_ids, out_scores, st);
   if (W == 2) return launch_small_w<2>(ls, q, k, out_ids, out_scores, st);
   return launch_small_w<1>(ls, q, k, out_ids, out_scores, st);
@@ -409,14 +378,7 @@ cudaError_t launch_merge(const ListSet& ls, int q, int k, int64_t* out_ids, floa
   }
   if (ls.P <= 32)
     return launch_warp_per_query(merge_kway_kernel, kWayWarps, ls, q, k, out_ids, out_scores, st);
-  if (k <= 16) {
-    const cudaError_t e = launch_small(ls, q, k, out_ids, out_scores, st);
-    if (e != cudaErrorNotSupported) return e;
-  }
-  if (k <= 32) return launch_merge_kp<32>(ls, q, k, out_ids, out_scores, st);
-  if (k <= 64) return launch_merge_kp<64>(ls, q, k, out_ids, out_scores, st);
-  if (k <= 128) return launch_merge_kp<128>(ls, q, k, out_ids, out_scores, st);
-  return launch_merge_kp<256>(ls, q, k, out_ids, out_scores, st);
+  return launch_small(ls, q, k, out_ids, out_scores, st);
 }
 
 }  // namespace oprag

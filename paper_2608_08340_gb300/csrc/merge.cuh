@@ -1,12 +1,5 @@
-// Block merge of one query's partial lists (the global top-k reduction of
-// Op_retrieve, Sec. 3.2 / Sec. 4.1 Retrieval), run by the merge kernel with
-// one CTA per query.
-//
-// The P * kl candidate keys of the query (the first kl of each producer's
-// sorted list) are split evenly over the CTA's warps; a warp fetches four
-// 32-key groups at once (independent loads, so L2 latency is paid once per
-// group of four) and filters them against its running k-th best.  Warp 0 then
-// merges the warps' results and writes the query's ranked top-k.
+// Pieces of the merges of a query's partial lists (the global top-k reduction
+// of Op_retrieve, Sec. 3.2 / Sec. 4.1 Retrieval).
 #pragma once
 #include "common.cuh"
 #include "internal.h"
@@ -74,70 +67,6 @@ __device__ __forceinline__ uint64_t merge_floor_key(const ListSet& ls, int qi, i
     }
   }
   return kEmptyKey;
-}
-
-// Shared memory: (nw + 1) * 2 * KP keys.  All threads of the CTA call this;
-// it ends with a barrier, so the buffer can be reused.
-template <int KP>
-__device__ __forceinline__ void merge_one_query(const ListSet& ls, int qi, int k, int nw,
-                                int64_t* __restrict__ out_ids, float* __restrict__ out_scores,
-                                uint64_t* smem_keys) {
-  constexpr int kCap = 2 * KP;
-  constexpr int kUnroll = 4;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int tile = qi / ls.TH, row = qi % ls.TH;
-  const uint64_t* base = ls.keys + (static_cast<int64_t>(tile) * ls.P * ls.TH + row) * ls.stride;
-  const int64_t list_step = static_cast<int64_t>(ls.TH) * ls.stride;
-  const int np = merge_list_count(ls, tile);
-  const int kl = min(k, ls.klen);         // keys read from each list
-  const int total = np * kl;
-  const int lo = static_cast<int>(static_cast<int64_t>(total) * warp / nw);
-  const int hi = static_cast<int>(static_cast<int64_t>(total) * (warp + 1) / nw);
-
-  WarpMerger<KP> m;
-  m.init(smem_keys + warp * kCap, k);
-  for (int g = lo; g < hi; g += 32 * kUnroll) {
-    uint64_t key[kUnroll];
-#pragma unroll
-    for (int u = 0; u < kUnroll; ++u) {
-      const int i = g + u * 32 + lane;
-      key[u] = kEmptyKey;
-      if (i < hi) {
-        const int p = i / kl;
-        key[u] = base[p * list_step + (i - p * kl)];
-      }
-    }
-#pragma unroll
-    for (int u = 0; u < kUnroll; ++u) merge_offer32(m, key[u]);
-  }
-  m.finish();
-  __syncthreads();
-  if (warp == 0) {
-    WarpMerger<KP> f;
-    f.init(smem_keys + nw * kCap, k);
-    const int all = nw * k;
-    for (int g = 0; g < all; g += 32 * kUnroll) {
-      uint64_t key[kUnroll];
-#pragma unroll
-      for (int u = 0; u < kUnroll; ++u) {
-        const int i = g + u * 32 + lane;
-        key[u] = kEmptyKey;
-        if (i < all) {
-          const int w = i / k;
-          key[u] = smem_keys[w * kCap + (i - w * k)];
-        }
-      }
-#pragma unroll
-      for (int u = 0; u < kUnroll; ++u) merge_offer32(f, key[u]);
-    }
-    f.finish();
-    for (int i = lane; i < k; i += 32) {
-      const uint64_t key = f.sbuf[i];
-      const int64_t o = static_cast<int64_t>(qi) * k + i;
-      store_result(ls, out_ids, out_scores, o, key);
-    }
-  }
-  __syncthreads();
 }
 
 }  // namespace oprag
