@@ -6,15 +6,16 @@
 // One CTA of four warps per query; a thread holds one or two candidates.  A
 // candidate's BM25 is the sum of its query terms' weights: a dense term's
 // weight is read from its row, a sparse term's is found by a binary search of
-// the term's postings.  What bounds it is the latency of
-// those dependent loads, so a thread searches kTermBatch terms at once, and
-// the searches of a whole batch of terms take as long as one.  The sums and
-// the fused score are formed exactly as in the BM25 pass and the fused search
-// epilogue, so with every chunk a candidate the result equals the full hybrid
-// search bit for bit.  A candidate's rank is counted against the other keys
-// in shared memory (no chain of exchanges).  Measured on GB300, 32768 chunks,
-// 1024 queries of 8 terms, 128 candidates: the search with its rerank takes
-// 140 us instead of 174 us with one warp per query and one term at a time.
+// the term's postings in the candidate's 1024-chunk tile (the table of the BM25
+// pass gives their range).  The searches' scattered reads of L2 bound the
+// kernel, and their latency, so a thread searches kTermBatch terms at once.
+// The sums and the fused score are formed exactly as in the BM25 pass and the
+// fused search epilogue, so with every chunk a candidate the result equals the
+// full hybrid search bit for bit.  A candidate's rank is counted against the
+// other keys in shared memory (no chain of exchanges).  Measured on GB300,
+// 32768 chunks, 1024 queries of 8 terms, 128 candidates: 21.7 us; a term's
+// whole list searched instead, 24 us; one warp per query and one term at a
+// time, 58 us.
 #include "common.cuh"
 #include "internal.h"
 
@@ -32,7 +33,7 @@ rerank_kernel(SparseIndex sp, int ncand, const int64_t* __restrict__ cand_ids,
               const int32_t* __restrict__ q_terms, float alpha, int k,
               int64_t* __restrict__ out_ids, float* __restrict__ out_scores) {
   __shared__ int term_slot[kTermBatch];            // dense row, -1: postings, -2: no term
-  __shared__ int64_t term_lo[kTermBatch], term_hi[kTermBatch];
+  __shared__ int64_t term_row[kTermBatch];         // the term's row of the tile table
   __shared__ uint64_t keys[kRerankThreads * E];
   __shared__ float warp_max[kRerankThreads / 32];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -53,47 +54,49 @@ rerank_kernel(SparseIndex sp, int ncand, const int64_t* __restrict__ cand_ids,
     __syncthreads();        // the previous batch's term table has been read
     if (tid < kTermBatch) {
       int slot = -2;
-      int64_t lo = 0, hi = 0;
       const int32_t term = base + tid < t1 ? q_terms[base + tid] : -1;
-      if (term >= 0 && term < sp.vocab) {
-        slot = sp.dense_slot[term];
-        lo = sp.post_ptr[term];              // (an empty range for a dense term)
-        hi = sp.post_ptr[term + 1];
-      }
-      term_slot[tid] = with_dense ? slot : -2;
-      term_lo[tid] = lo;
-      term_hi[tid] = with_sparse ? hi : lo;
+      if (term >= 0 && term < sp.vocab) slot = sp.dense_slot[term];
+      term_slot[tid] = slot >= 0 ? (with_dense ? slot : -2) : (with_sparse ? slot : -2);
+      term_row[tid] = static_cast<int64_t>(term) * (sp.ntiles + 1);
     }
     __syncthreads();
+    // Dense weights, and each candidate's part of the sparse terms' postings:
+    // those of the candidate's tile of chunks.
     float w[kTermBatch][E];
-    int lo[kTermBatch][E], hi[kTermBatch][E];       // offsets from term_lo
-    int longest = 0;
+    int lo[kTermBatch][E], hi[kTermBatch][E], end[kTermBatch][E];
 #pragma unroll
     for (int b = 0; b < kTermBatch; ++b) {
       const int slot = term_slot[b];
-      const int len = static_cast<int>(term_hi[b] - term_lo[b]);
-      longest = max(longest, len);
+      const int32_t* tp = sp.tile_ptr + term_row[b];
 #pragma unroll
       for (int e = 0; e < E; ++e) {
         w[b][e] = 0.f;
-        if (slot >= 0 && doc[e] >= 0) w[b][e] = __ldg(sp.dense_w + slot * sp.dense_ld + doc[e]);
-        lo[b][e] = 0;
-        hi[b][e] = doc[e] >= 0 ? len : 0;
+        lo[b][e] = hi[b][e] = 0;
+        if (doc[e] < 0) continue;
+        if (slot >= 0) w[b][e] = __ldg(sp.dense_w + slot * sp.dense_ld + doc[e]);
+        if (slot == -1) {
+          lo[b][e] = __ldg(tp + doc[e] / kBm25DocTile);
+          hi[b][e] = __ldg(tp + doc[e] / kBm25DocTile + 1);
+        }
       }
     }
-    // Lower bound of each candidate in each term's (ascending) postings: the
-    // interval of a search halves per step, so the longest list gives the
-    // number of steps.
-    for (int left = longest; left > 0; left >>= 1) {
+#pragma unroll
+    for (int b = 0; b < kTermBatch; ++b)
+#pragma unroll
+      for (int e = 0; e < E; ++e) end[b][e] = hi[b][e];
+    // Lower bound of each candidate in each range (chunks ascending).
+    bool more = true;
+    while (more) {
+      more = false;
 #pragma unroll
       for (int b = 0; b < kTermBatch; ++b) {
-        const int2* post = sp.post + term_lo[b];
 #pragma unroll
         for (int e = 0; e < E; ++e) {
           if (lo[b][e] < hi[b][e]) {
-            const int mid = (lo[b][e] + hi[b][e]) >> 1;
-            if (__ldg(&post[mid].x) < doc[e]) lo[b][e] = mid + 1;
+            const int mid = lo[b][e] + ((hi[b][e] - lo[b][e]) >> 1);
+            if (__ldg(&sp.post[mid].x) < doc[e]) lo[b][e] = mid + 1;
             else hi[b][e] = mid;
+            more |= lo[b][e] < hi[b][e];
           }
         }
       }
@@ -104,12 +107,11 @@ rerank_kernel(SparseIndex sp, int ncand, const int64_t* __restrict__ cand_ids,
       for (int e = 0; e < E; ++e) lex[e] += w[b][e];
 #pragma unroll
     for (int b = 0; b < kTermBatch; ++b) {
-      const int len = static_cast<int>(term_hi[b] - term_lo[b]);
 #pragma unroll
       for (int e = 0; e < E; ++e) {
         w[b][e] = 0.f;
-        if (doc[e] >= 0 && lo[b][e] < len) {
-          const int2 pe = __ldg(sp.post + term_lo[b] + lo[b][e]);
+        if (lo[b][e] < end[b][e]) {
+          const int2 pe = __ldg(sp.post + lo[b][e]);
           if (pe.x == doc[e]) w[b][e] = __int_as_float(pe.y);
         }
       }
