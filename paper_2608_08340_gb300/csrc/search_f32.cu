@@ -32,9 +32,15 @@ Config config_for(const SearchShape& s, int G) {
   // buffers, counts and floors, barriers and the abort word, ring alignment
   const size_t fixed = static_cast<size_t>(c.th) * (c.cap * sizeof(uint64_t) + 8) +
                        2 * kMaxStages * sizeof(uint64_t) + 16 + 1024;
-  const size_t stage = stage_bytes(c.th, bn);
-  c.stages = static_cast<int>(std::min<size_t>(kMaxStages, (kSmemMax - fixed) / stage));
-  c.smem = fixed + c.stages * stage;
+  // A stage holds the corpus rows of the widest tile of a slice (short slices
+  // then have more K blocks in flight) and the queries, in whole swizzle atoms.
+  const int tx = kThreads / c.TY;
+  const int64_t rows = (s.n + G - 1) / G;
+  const int groups = static_cast<int>(std::min<int64_t>(kRowsPerThread, (rows + tx - 1) / tx));
+  c.b_bytes = groups * tx * kRowBytes;
+  c.stage = (c.b_bytes + c.th * kRowBytes + 1023) / 1024 * 1024;
+  c.stages = static_cast<int>(std::min<size_t>(kMaxStages, (kSmemMax - fixed) / c.stage));
+  c.smem = fixed + c.stages * static_cast<size_t>(c.stage);
   return c;
 }
 
@@ -84,6 +90,8 @@ cudaError_t launch_f32_search(const void* E, const void* Q, const SearchShape& s
   p.stride = list_len_for(s.k);
   p.cap = c.cap;
   p.stages = c.stages;
+  p.stage = c.stage;
+  p.b_bytes = c.b_bytes;
   p.qfloor = qfloor;
   p.gen = gen;
   p.dev_err = dev_err;

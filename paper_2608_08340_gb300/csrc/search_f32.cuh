@@ -46,7 +46,7 @@ constexpr int kRowBytes = kBK * 4;
 constexpr int kRowsPerThread = 4;
 constexpr int kFoldBlocks = 2;             // K blocks between folds
 constexpr int kMaxCap = 512;               // candidate keys per query
-constexpr int kMaxStages = 8;
+constexpr int kMaxStages = 16;
 constexpr size_t kSmemMax = 226 * 1024;
 
 struct Params {
@@ -59,6 +59,8 @@ struct Params {
   int stride;
   int cap;
   int stages;
+  int stage;            // bytes of a ring stage: b_bytes of corpus rows, then the queries
+  int b_bytes;
   uint64_t* qfloor;     // optional: shared k-th bounds, tagged gen
   uint32_t gen;
   int* dev_err;
@@ -71,14 +73,9 @@ struct Config {
   int th;        // queries per tile, TY * TM
   int qt;        // query tiles
   int G;         // corpus slices
-  int cap, stages;
+  int cap, stages, stage, b_bytes;
   size_t smem;
 };
-
-// Bytes of a ring stage (whole swizzle atoms).
-__host__ __device__ constexpr int stage_bytes(int th, int bn) {
-  return (bn * kRowBytes + th * kRowBytes + 1023) / 1024 * 1024;
-}
 
 // One K block: eight groups of four k (zeros past d), TN of the thread's four
 // rows.  a0 / b0: the thread's first query / corpus row of the stage.
@@ -202,13 +199,12 @@ f32_search_kernel(const __grid_constant__ CUtensorMap map_q,
                   const __grid_constant__ CUtensorMap map_e, const Params p) {
   constexpr int TX = kThreads / TY;
   constexpr int BM = TY * TM, BN = TX * kRowsPerThread;
-  constexpr int kStage = stage_bytes(BM, BN);
   constexpr int WY = TY / 4;                          // warps along the queries
   extern __shared__ __align__(1024) unsigned char smem_f[];
   // (an offset, not a rounded pointer: the compiler then still knows that the
   // ring is shared memory)
   unsigned char* ring = smem_f + ((1024 - (smem_addr(smem_f) & 1023)) & 1023);
-  uint64_t* buf = reinterpret_cast<uint64_t*>(ring + p.stages * kStage);
+  uint64_t* buf = reinterpret_cast<uint64_t*>(ring + p.stages * p.stage);
   uint64_t* full = buf + static_cast<size_t>(BM) * p.cap;
   uint64_t* empty = full + kMaxStages;
   int* cnt = reinterpret_cast<int*>(empty + kMaxStages);
@@ -259,13 +255,13 @@ f32_search_kernel(const __grid_constant__ CUtensorMap map_q,
   auto load_next = [&]() {
     if (lane == 0 && !*abort_flag &&
         mbar_wait(&empty[ld_s], ld_ph ^ 1u, abort_flag, p.dev_err, p.wait_limit)) {
-      unsigned char* sB = ring + ld_s * kStage;
+      unsigned char* sB = ring + ld_s * p.stage;
       const int tn = groups_of(ld_r0);
       mbar_arrive_expect_tx(&full[ld_s], static_cast<uint32_t>((tn * TX + BM) * kRowBytes));
       for (int j = 0; j < tn; ++j)
         tma_load_2d(sB + j * TX * kRowBytes, &map_e, &full[ld_s], ld_kb * kBK,
                     static_cast<int>(ld_r0) + j * TX);
-      tma_load_2d(sB + BN * kRowBytes, &map_q, &full[ld_s], ld_kb * kBK, q0);
+      tma_load_2d(sB + p.b_bytes, &map_q, &full[ld_s], ld_kb * kBK, q0);
       issued |= 1u << ld_s;
       parity = (parity & ~(1u << ld_s)) | (ld_ph << ld_s);
     }
@@ -274,7 +270,7 @@ f32_search_kernel(const __grid_constant__ CUtensorMap map_q,
     for (ld_s += kThreads / 32; ld_s >= p.stages; ld_s -= p.stages) ld_ph ^= 1u;
     for (ld_kb += kThreads / 32; ld_kb >= nkb; ld_kb -= nkb) ld_r0 += BN;
   };
-  if (ld_m < p.stages - lag && ld_m < blocks) load_next();
+  while (ld_m < p.stages - lag && ld_m < blocks) load_next();
 
   // A wait that gives up does not end a warp early (the warps meet at
   // barriers): it goes on with whatever the stage holds, and every later wait
@@ -304,8 +300,8 @@ f32_search_kernel(const __grid_constant__ CUtensorMap map_q,
       if (ld_m == blk + p.stages - lag && ld_m < blocks) load_next();
       mbar_wait(&full[st], ph, abort_flag, p.dev_err, p.wait_limit);
       __syncwarp();
-      const unsigned char* sB = ring + st * kStage + tx * kRowBytes;
-      const unsigned char* sA = ring + st * kStage + (BN + ty) * kRowBytes;
+      const unsigned char* sB = ring + st * p.stage + tx * kRowBytes;
+      const unsigned char* sA = ring + st * p.stage + p.b_bytes + ty * kRowBytes;
       if (tn == 4) mul_block<TY, TM, 4>(sA, sB, ty, tx, acc);
       else if (tn == 3) mul_block<TY, TM, 3>(sA, sB, ty, tx, acc);
       else if (tn == 2) mul_block<TY, TM, 2>(sA, sB, ty, tx, acc);
