@@ -4,10 +4,11 @@
 // local candidates to the global top-k, done inside one GPU: the producers
 // are corpus slices instead of index shards.
 //
-// Three merges: for unsorted lists (buffered tensor-core lists, k > 32) one warp
+// Three merges: for unsorted lists (buffered tensor-core lists, k > 32) a CTA
 // per query over all their keys; for sorted lists head by head, one warp per
 // query over at most 32 lists, one to four warps per query over up to 512.
 #include "merge.cuh"
+#include "oprag.h"
 
 namespace oprag {
 
@@ -165,106 +166,238 @@ merge_small_kernel(ListSet ls, int q, int k, int64_t* __restrict__ out_ids,
   }
 }
 
-// Unsorted lists (ListSet::counts), k > 32: one warp per query.  The warp
-// scans the query's list counts into offsets in shared memory, reads the
-// concatenated keys 32 x kUnsortedLoads at a time (a lane's keys come in
-// increasing order, so it finds each key's list by moving a cursor forward
-// over the offsets, rarely more than one step), drops keys below the counted floor and
-// keeps the rest in a WarpMerger, whose buffer is sorted only when it fills
-// up and once at the end.  A good floor leaves a few hundred keys of the
-// several thousand read, so a query usually costs one sort; the warps of
-// different queries share nothing and need no barrier.
-constexpr int kUnsortedWarps = 4;
-constexpr int kUnsortedLoads = 8;
+// Unsorted lists (ListSet::counts), k > 32: W warps per query, a CTA of their
+// own.  What bounds it is a chain of dependent steps on few keys, so each step
+// is taken by all threads at once: the lists' counts are scanned into offsets
+// in shared memory, every thread reads kUnsortedLoads of the concatenated keys
+// (a binary search of the offsets finds a key's list), and the keys above the
+// floor go to a buffer, which is cut down when the next round of keys might
+// not fit and ranked at the end.  A good floor leaves little more than k keys.
+// Measured on GB300 (event pairs of 2 us included), against a warp per query
+// that sorts its buffer: 300 queries of 32768 x 256, k = 50 10 (14) us, of
+// 300000 x 128 12 (20) us; 33 queries of 300000 x 128, k = 100 14 (33) us, 4000
+// queries of 32768 x 256, k = 100 18 (29) us; 32768 rows in ascending order of
+// their scores, 33 queries, k = 256 62 (381) us.
+constexpr int kUnsortedLoads = 4;
+constexpr int kRankMax = 256;       // keys that rank_buffer takes
+static_assert(kRankMax >= OPRAG_K_MAX, "the k best can be ranked");
+// Up to this many queries, whose CTAs the SMs hold all at once (ten of four
+// warps each), four warps a query; above, two.  Four against two warps,
+// event-timed, k = 100: 300 queries of 300000 x 128 12 / 16 us, 1024 queries 16
+// / 16 us, 4000 queries 35 / 31 us; 2048 queries of 1048576 x 768 27 / 23 us.
+constexpr int kUnsortedWideQueries = 1520;
 
-// Shared memory of merge_unsorted_kernel: a merger buffer and P + 1
-// offsets per warp.
-template <int KP>
-size_t unsorted_smem_bytes(int P) {
-  return kUnsortedWarps * (2 * KP * sizeof(uint64_t) + (static_cast<size_t>(P) + 4) / 4 * 16);
+template <int W>
+struct Unsorted {
+  static constexpr int kThreads = 32 * W;
+  static constexpr int kRound = kThreads * kUnsortedLoads;   // keys read at a time
+  static constexpr int kCap = 2 * kRound;                    // keys in the buffer
+  static_assert(kCap - kRound >= kRankMax, "a cut buffer leaves room for a round");
+};
+
+// Drops the smallest of the buffer's c > limit keys (all different) until
+// between k and limit are left, and returns how many; keys up to the new
+// `floor` are not among the k best.  A bisection between the smallest and the
+// largest key: a few rounds, where a sort takes some fifty.
+template <int W>
+__device__ __forceinline__ int cut_buffer(uint64_t* buf, int c, int k, int limit, uint64_t& floor) {
+  constexpr int T = Unsorted<W>::kThreads, E = Unsorted<W>::kCap / T;
+  __shared__ uint64_t ends[2][W];
+  __shared__ int part[2][W];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  uint64_t v[E], lo = ~0ull, hi = 0;
+#pragma unroll
+  for (int e = 0; e < E; ++e) {
+    const bool in = tid + e * T < c;
+    v[e] = in ? buf[tid + e * T] : kEmptyKey;
+    lo = umin64(lo, in ? v[e] : ~0ull);
+    hi = umax64(hi, v[e]);
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    lo = umin64(lo, __shfl_xor_sync(0xffffffffu, lo, o));
+    hi = umax64(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+  }
+  if (lane == 0) {
+    ends[0][warp] = lo;
+    ends[1][warp] = hi;
+  }
+  __syncthreads();          // also: every key of the buffer is in a register
+#pragma unroll
+  for (int w = 0; w < W; ++w) {
+    lo = umin64(lo, ends[0][w]);
+    hi = umax64(hi, ends[1][w]);
+  }
+  // c > limit keys are >= lo, and none is > hi; as no two are equal, some
+  // value in (lo, hi] has exactly k keys at or above it.
+  int kept = c, round = 0, before = 0;
+  uint64_t mid = lo;
+  while (lo < hi) {
+    mid = lo + ((hi - lo) >> 1) + ((hi - lo) & 1);
+    int mine = 0;
+#pragma unroll
+    for (int e = 0; e < E; ++e) mine += v[e] >= mid ? 1 : 0;
+    mine = __reduce_add_sync(0xffffffffu, mine);
+    if (lane == 0) part[round][warp] = mine;
+    __syncthreads();
+    kept = before = 0;
+#pragma unroll
+    for (int w = 0; w < W; ++w) {
+      if (w < warp) before += part[round][w];
+      kept += part[round][w];
+    }
+    round ^= 1;             // written again only after the next barrier
+    if (kept > limit) lo = mid;
+    else if (kept < k) hi = mid - 1;
+    else break;
+  }
+#pragma unroll
+  for (int e = 0; e < E; ++e) {
+    const uint32_t bits = __ballot_sync(0xffffffffu, v[e] >= mid);
+    const int at = before + __popc(bits & ((1u << lane) - 1u));
+    if (v[e] >= mid && at < limit) buf[at] = v[e];
+    before += __popc(bits);
+  }
+  floor = mid - 1;
+  __syncthreads();
+  return min(kept, limit);
 }
 
-template <int KP>
-__global__ void __launch_bounds__(kUnsortedWarps * 32)
-merge_unsorted_kernel(ListSet ls, int q, int k, int64_t* __restrict__ out_ids,
+// Sorts the buffer's c <= kRankMax keys, best first: every thread counts the
+// keys above its own ones, with no barrier between.
+template <int T, int E>
+__device__ __forceinline__ void rank_buffer(uint64_t* buf, int c) {
+  uint64_t v[E];
+  int above[E];
+#pragma unroll
+  for (int e = 0; e < E; ++e) {
+    const int i = threadIdx.x + e * T;
+    v[e] = i < c ? buf[i] : kEmptyKey;
+    above[e] = 0;
+  }
+#pragma unroll 8
+  for (int i = 0; i < c; ++i) {
+    const uint64_t o = buf[i];
+#pragma unroll
+    for (int e = 0; e < E; ++e) above[e] += o > v[e] ? 1 : 0;
+  }
+  __syncthreads();
+#pragma unroll
+  for (int e = 0; e < E; ++e)
+    if (static_cast<int>(threadIdx.x) + e * T < c) buf[above[e]] = v[e];
+  __syncthreads();
+}
+
+template <int W>
+__global__ void __launch_bounds__(Unsorted<W>::kThreads)
+merge_unsorted_kernel(ListSet ls, int k, int64_t* __restrict__ out_ids,
                       float* __restrict__ out_scores) {
-  extern __shared__ __align__(16) uint64_t smem_u[];
+  constexpr int T = Unsorted<W>::kThreads, kRound = Unsorted<W>::kRound, kCap = Unsorted<W>::kCap;
+  extern __shared__ int offs[];                     // P: keys of the lists before p
+  __shared__ uint64_t buf[kCap];
+  __shared__ int warp_sum[W];
+  __shared__ int count;
   asm volatile("griddepcontrol.wait;" ::: "memory");
-  constexpr int kCap = 2 * KP;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int qi = blockIdx.x * kUnsortedWarps + warp;
-  if (qi >= q) return;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int qi = blockIdx.x;
   const int tile = qi / ls.TH, row = qi % ls.TH;
   const int np = merge_list_count(ls, tile);
-  const int offs_len = (ls.P + 4) / 4 * 4;
-  int* offs = reinterpret_cast<int*>(smem_u + kUnsortedWarps * kCap) + warp * offs_len;
   const int* cnt = ls.counts + static_cast<int64_t>(tile) * ls.P * ls.TH + row;
   const uint64_t* base = ls.keys + (static_cast<int64_t>(tile) * ls.P * ls.TH + row) * ls.stride;
   const int64_t list_step = static_cast<int64_t>(ls.TH) * ls.stride;
+  uint64_t worst = merge_floor_key(ls, qi, k);      // the same in every thread
 
-  // offs[p]: keys of the lists before p (exclusive scan, 32 lists a round)
-  int total = 0;
-  for (int p0 = 0; p0 < np; p0 += 32) {
-    const int p = p0 + lane;
-    const int c = p < np ? max(0, min(cnt[static_cast<int64_t>(p) * ls.TH], ls.stride)) : 0;
+  auto list_count = [&](int p) {
+    return p < np ? max(0, min(cnt[static_cast<int64_t>(p) * ls.TH], ls.stride)) : 0;
+  };
+  if (tid == 0) count = 0;
+  int total = 0, next = list_count(tid);
+  for (int p0 = 0; p0 < np; p0 += T) {
+    const int c = next;
+    next = list_count(p0 + T + tid);
     int incl = c;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
       const int t = __shfl_up_sync(0xffffffffu, incl, o);
       if (lane >= o) incl += t;
     }
-    if (p < np) offs[p] = total + incl - c;
-    total += __shfl_sync(0xffffffffu, incl, 31);
+    if (lane == 31) warp_sum[warp] = incl;
+    __syncthreads();
+    int before = total;
+#pragma unroll
+    for (int w = 0; w < W; ++w) {
+      if (w < warp) before += warp_sum[w];
+      total += warp_sum[w];
+    }
+    if (p0 + tid < np) offs[p0 + tid] = before + incl - c;
+    __syncthreads();        // warp_sum has been read; the offsets are written
   }
-  if (lane == 0) offs[np] = total;
-  __syncwarp();
 
-  WarpMerger<KP> m;
-  m.init(smem_u + warp * kCap, k);
-  m.worst = merge_floor_key(ls, qi, k);
-  int cur = 0;      // this lane's list: offs[cur] <= its next key's index
-  for (int g = 0; g < total; g += 32 * kUnsortedLoads) {
+  for (int g = 0; g < total; g += kRound) {
     uint64_t key[kUnsortedLoads];
 #pragma unroll
     for (int u = 0; u < kUnsortedLoads; ++u) {
-      const int i = g + u * 32 + lane;
+      const int i = g + u * T + tid;
       key[u] = kEmptyKey;
       if (i < total) {
-        // the list holding key i: the last p with offs[p] <= i (offs[np] =
-        // total > i ends the walk)
-        while (offs[cur + 1] <= i) ++cur;
-        key[u] = base[cur * list_step + (i - offs[cur])];
+        int lo = 0, hi = np;                        // the last list with offs[p] <= i
+        while (hi - lo > 1) {
+          const int mid = (lo + hi) >> 1;
+          if (offs[mid] <= i) lo = mid;
+          else hi = mid;
+        }
+        key[u] = base[lo * list_step + (i - offs[lo])];
       }
     }
+    uint32_t bits[kUnsortedLoads];
+    int pass = 0;
 #pragma unroll
-    for (int u = 0; u < kUnsortedLoads; ++u)
-      if (g + u * 32 < total) merge_offer32(m, key[u]);
+    for (int u = 0; u < kUnsortedLoads; ++u) {
+      bits[u] = __ballot_sync(0xffffffffu, key[u] > worst);
+      pass += __popc(bits[u]);
+    }
+    if (pass != 0) {
+      int slot = 0;
+      if (lane == 0) slot = atomicAdd(&count, pass);
+      slot = __shfl_sync(0xffffffffu, slot, 0);
+#pragma unroll
+      for (int u = 0; u < kUnsortedLoads; ++u) {
+        if (key[u] > worst) buf[slot + __popc(bits[u] & ((1u << lane) - 1u))] = key[u];
+        slot += __popc(bits[u]);
+      }
+    }
+    __syncthreads();
+    const int c = count;
+    if (g + kRound < total && c > kCap - kRound) {
+      const int kept = cut_buffer<W>(buf, c, k, kRankMax, worst);
+      if (tid == 0) count = kept;
+    }
+    __syncthreads();
   }
-  m.finish();
-  for (int i = lane; i < k; i += 32)
-    store_result(ls, out_ids, out_scores, static_cast<int64_t>(qi) * k + i, m.sbuf[i]);
+  int c = count;
+  const int limit = k <= 7 * kRankMax / 16 ? kRankMax / 2 : kRankMax;
+  if (c > limit) c = cut_buffer<W>(buf, c, k, limit, worst);
+  if (c <= kRankMax / 2) rank_buffer<T, kRankMax / 2 / T>(buf, c);
+  else if (c <= 3 * kRankMax / 4) rank_buffer<T, (3 * kRankMax / 4 + T - 1) / T>(buf, c);
+  else rank_buffer<T, kRankMax / T>(buf, c);
+  for (int i = tid; i < k; i += T)
+    store_result(ls, out_ids, out_scores, static_cast<int64_t>(qi) * k + i,
+                 i < c ? buf[i] : kEmptyKey);
 }
 
-template <int KP>
-cudaError_t launch_unsorted_kp(const ListSet& ls, int q, int k, int64_t* ids, float* scores, cudaStream_t st) {
-  const size_t smem = unsorted_smem_bytes<KP>(ls.P);
-  if (smem > 48 * 1024) {
-    const cudaError_t e =
-        cudaFuncSetAttribute(merge_unsorted_kernel<KP>,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
-    if (e != cudaSuccess) return e;
-  }
+template <int W>
+cudaError_t launch_unsorted(const ListSet& ls, int q, int k, int64_t* ids, float* scores, cudaStream_t st) {
   cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3((q + kUnsortedWarps - 1) / kUnsortedWarps);
-  cfg.blockDim = dim3(kUnsortedWarps * 32);
-  cfg.dynamicSmemBytes = smem;
+  cfg.gridDim = dim3(q);
+  cfg.blockDim = dim3(Unsorted<W>::kThreads);
+  cfg.dynamicSmemBytes = static_cast<size_t>(ls.P) * sizeof(int);
   cfg.stream = st;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, merge_unsorted_kernel<KP>, ls, q, k, ids, scores);
+  return cudaLaunchKernelEx(&cfg, merge_unsorted_kernel<W>, ls, k, ids, scores);
 }
 
 template <typename Kern>
@@ -369,13 +502,9 @@ cudaError_t launch_merge_two(int q, const int64_t* a_ids, const float* a_sc, int
 
 cudaError_t launch_merge(const ListSet& ls, int q, int k, int64_t* out_ids, float* out_scores, cudaStream_t st) {
   if (q <= 0) return cudaSuccess;
-  // Unsorted lists: one sort per query instead of k head-by-head rounds.
-  if (ls.counts != nullptr) {
-    if (k <= 64) return launch_unsorted_kp<64>(ls, q, k, out_ids, out_scores, st);
-    if (k <= 128)
-      return launch_unsorted_kp<128>(ls, q, k, out_ids, out_scores, st);
-    return launch_unsorted_kp<256>(ls, q, k, out_ids, out_scores, st);
-  }
+  if (ls.counts != nullptr)
+    return q <= kUnsortedWideQueries ? launch_unsorted<4>(ls, q, k, out_ids, out_scores, st)
+                                     : launch_unsorted<2>(ls, q, k, out_ids, out_scores, st);
   if (ls.P <= 32)
     return launch_warp_per_query(merge_kway_kernel, kWayWarps, ls, q, k, out_ids, out_scores, st);
   return launch_small(ls, q, k, out_ids, out_scores, st);

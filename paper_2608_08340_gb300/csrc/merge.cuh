@@ -6,17 +6,6 @@
 
 namespace oprag {
 
-template <int KP>
-__device__ __forceinline__ void merge_offer32(WarpMerger<KP>& m, uint64_t key) {
-  const int lane = threadIdx.x & 31;
-  const bool pass = key > m.worst;
-  const uint32_t bits = __ballot_sync(0xffffffffu, pass);
-  if (bits == 0) return;
-  if (m.count > WarpMerger<KP>::kCap - 32) m.compact();
-  if (pass) m.sbuf[m.count + __popc(bits & ((1u << lane) - 1u))] = key;
-  m.count += __popc(bits);
-}
-
 // Writes result o of the merge: a key's id (split into the corpus and the id
 // within it for a search over two stacked corpora) and score, or the empty
 // result (-1, -inf).
@@ -56,15 +45,19 @@ __device__ __forceinline__ int merge_list_count(const ListSet& ls, int tile) {
 // counted floors.
 __device__ __forceinline__ uint64_t merge_floor_key(const ListSet& ls, int qi, int k) {
   if (ls.levels == nullptr || ls.level_cnt == nullptr) return kEmptyKey;
+  int cnt[kLevels];
+  float floors[kLevels];
+#pragma unroll
+  for (int i = 0; i < kLevels; ++i) {       // all loads before the first use
+    const int64_t o = static_cast<int64_t>(qi) * kLevels + i;
+    cnt[i] = ls.level_cnt[o];
+    floors[i] = ls.levels[o];
+  }
   int sum = 0;
 #pragma unroll
   for (int i = 0; i < kLevels; ++i) {
-    const int64_t o = static_cast<int64_t>(qi) * kLevels + i;
-    sum += ls.level_cnt[o];
-    if (sum >= k) {
-      const float f = ls.levels[o];
-      return f > -INFINITY ? make_key(f, kNoId) : kEmptyKey;
-    }
+    sum += cnt[i];
+    if (sum >= k) return floors[i] > -INFINITY ? make_key(floors[i], kNoId) : kEmptyKey;
   }
   return kEmptyKey;
 }
