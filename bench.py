@@ -50,9 +50,9 @@ sys.path.insert(0, ROOT)
 from paper_2608_08340_gb300 import workloads  # noqa: E402
 
 L2_FLUSH_BYTES = 512 << 20
-# Files that define the search kernel whose DRAM traffic profiles/ncu_traffic.json
+# Files that define the search kernels whose DRAM traffic profiles/ncu_traffic.json
 # records; the hash covers their code with comments and blank space removed.
-KERNEL_SOURCES = ["common.cuh", "search_tc.cuh", "search_tc.cu"]
+KERNEL_SOURCES = ["common.cuh", "search_tc.cuh", "search_tc.cu", "search_small.cu"]
 
 
 def _code_only(text: str) -> str:
@@ -442,8 +442,11 @@ def measure(args, cfg: int, batch: int, rank: int, world: int, local_rank: int,
     idx.check()
     t = idx.last_timing()
     sampled = t["sample_ms"] > 0.0
-    # (a search of up to 6 queries and k <= 8 merges in its search kernel)
-    inline = idx.last_path == "tc" and w.q <= 6 and w.k <= 8 and cfg != 3
+    # (a small batch has a kernel of its own, which up to 6 queries and k <= 8
+    # merges its lists too)
+    small = (idx.last_path == "tc" and w.q <= 32 and w.k <= 16 and cfg != 3
+             and args.pair == "auto" and not args.block_n and not args.phases)
+    inline = small and w.q <= 6 and w.k <= 8
     launches_per_step = (1 if inline else 2) + (2 if sampled else 0) + (1 if cfg in (3, 4) else 0)
 
     if world > 1:
@@ -602,7 +605,7 @@ def measure(args, cfg: int, batch: int, rank: int, world: int, local_rank: int,
     if roof["bound"] == "tensor":
         roof["peak_kind"] = ("sustained: sw_power_cap active in the timed region" if capped
                              else "burst")
-    roof["kernel"] = ("tc_search_kernel" if path == "tc" else
+    roof["kernel"] = ("small_search_kernel" if small else "tc_search_kernel" if path == "tc" else
                       "f32_search_kernel" if w.dtype == "f32" else "simt_search_kernel")
     roof["kernel_ms_mean"] = statistics.mean(tim["search_ms"])
     roof["kernel_ms_median"] = statistics.median(tim["search_ms"])
