@@ -11,9 +11,15 @@
 // cycles of the SM each; 4.2 for 16 rows or more).  K blocks of 32 floats of
 // both operands come through a TMA ring (128-byte swizzle: eight rows' reads
 // of one k group touch all banks once) that thread 0 feeds between its own
-// blocks: a ninth warp would cap every thread at 168 registers.  Every two K blocks
-// the sums are folded into one of two second-level sums in turn, so that no
-// chain of additions is longer than 64, or than d / 128 at the second level.
+// blocks: a ninth warp would cap every thread at 168 registers.
+//
+// Sums: chains of eight products, four of them added up per K block, and the
+// blocks' sums added with compensation (Kahan), so that the error does not grow
+// with d.  Relative error against 64 bits (root mean square over the 10 best of
+// 100 queries), in brackets the streaming kernel's: d = 64 4.4e-8 (3.9e-8), 128
+// 4.3e-8 (4.6e-8), 768 3.6e-8 (5.2e-8), 1280 3.1e-8 (5.4e-8).  One chain of 64
+// products per two blocks, added to two plain sums in turn, gave 11.6e-8, 9.6e-8,
+// 6.8e-8 and 6.8e-8, and 177 us instead of 195 at 100 queries of 32768 x 768.
 //
 // What bounds it: from about 16 queries on the FMA pipes and, next to them,
 // the shared-memory reads that feed them (a warp step of four k: 112 FMA issue
@@ -21,10 +27,9 @@
 // batch (config_for): TY = 4 (256 corpus rows) up to 32 queries, TY = 8 up to
 // 64, TY = 16 above.  Measured on GB300, 32768 x 768 and k = 10, search kernel,
 // against the streaming kernel this one replaced (each chunk of eight queries
-// streamed the corpus again, five shuffles per score): 1 query 28 (51) us, 16
-// queries 42 (92) us, 100 queries 176 (528) us or 28.5 TFLOP/s, 256 queries
-// 356 (1298) us; 100000 x 768 and 1 query 63 (119) us or 4.9 TB/s; 100 queries
-// and k = 100 270 (1542) us.
+// streamed the corpus again, five shuffles per score): 1 query 27 (41) us, 16
+// queries 43 (92) us, 32 queries 68 (172) us, 100 queries 195 (529) us or 25.8
+// TFLOP/s, 256 queries 393 (1297) us; 86132 x 1192 and 8 queries 96 (111) us.
 //
 // Selection.  Each query of the tile has a buffer of candidate keys in shared
 // memory.  A score enters it when it reaches the query's floor: the k-th
@@ -44,7 +49,7 @@ constexpr int kThreads = 256;
 constexpr int kBK = 32;                    // floats per K block: one 128-byte swizzle row
 constexpr int kRowBytes = kBK * 4;
 constexpr int kRowsPerThread = 4;
-constexpr int kFoldBlocks = 2;             // K blocks between folds
+constexpr int kChain = 8;                  // products of a first-level sum
 constexpr int kMaxCap = 512;               // candidate keys per query
 constexpr int kMaxStages = 16;
 constexpr size_t kSmemMax = 226 * 1024;
@@ -78,13 +83,15 @@ struct Config {
 };
 
 // One K block: eight groups of four k (zeros past d), TN of the thread's four
-// rows.  a0 / b0: the thread's first query / corpus row of the stage.
+// rows.  mid: the block's sums, of chains of kChain products.  a0 / b0: the thread's first query / corpus row of the stage.
 template <int TY, int TM, int TN>
 __device__ __forceinline__ void mul_block(const unsigned char* a0, const unsigned char* b0, int ty,
-                                          int tx, float (&acc)[TM][kRowsPerThread]) {
+                                          int tx, float (&mid)[TM][kRowsPerThread]) {
   constexpr int TX = kThreads / TY;
+  float acc[TM][TN];
 #pragma unroll
   for (int s = 0; s < kBK / 4; ++s) {
+    const bool first = s % (kChain / 4) == 0, last = (s + 1) % (kChain / 4) == 0;
     const int ob = (s ^ (tx & 7)) << 4;
     float4 b[TN];
 #pragma unroll
@@ -96,15 +103,23 @@ __device__ __forceinline__ void mul_block(const unsigned char* a0, const unsigne
       const int oa = (s ^ ((ty + TY * i) & 7)) << 4;
       const float4 a = *reinterpret_cast<const float4*>(a0 + i * TY * kRowBytes + oa);
 #pragma unroll
-      for (int j = 0; j < TN; ++j) acc[i][j] = fmaf(a.x, b[j].x, acc[i][j]);
+      for (int j = 0; j < TN; ++j) acc[i][j] = first ? a.x * b[j].x : fmaf(a.x, b[j].x, acc[i][j]);
 #pragma unroll
       for (int j = 0; j < TN; ++j) acc[i][j] = fmaf(a.y, b[j].y, acc[i][j]);
 #pragma unroll
       for (int j = 0; j < TN; ++j) acc[i][j] = fmaf(a.z, b[j].z, acc[i][j]);
 #pragma unroll
       for (int j = 0; j < TN; ++j) acc[i][j] = fmaf(a.w, b[j].w, acc[i][j]);
+      if (last)
+#pragma unroll
+        for (int j = 0; j < TN; ++j)
+          mid[i][j] = s < kChain / 4 ? acc[i][j] : mid[i][j] + acc[i][j];
     }
   }
+#pragma unroll
+  for (int i = 0; i < TM; ++i)
+#pragma unroll
+    for (int j = TN; j < kRowsPerThread; ++j) mid[i][j] = 0.f;
 }
 
 // The warp puts the min(c, k) best of the c keys of a buffer, best first, into
@@ -277,7 +292,7 @@ f32_search_kernel(const __grid_constant__ CUtensorMap map_q,
   // returns at once because the abort word is set.
   const int ty = (warp % WY) * 4 + (lane >> 3);
   const int tx = (warp / WY) * 8 + (lane & 7);
-  float acc[TM][kRowsPerThread], tot[2][TM][kRowsPerThread];
+  float acc[TM][kRowsPerThread], tot[TM][kRowsPerThread], lost[TM][kRowsPerThread];
   int st = 0, blk = 0;
   uint32_t ph = 0;
 #pragma unroll 1
@@ -287,7 +302,7 @@ f32_search_kernel(const __grid_constant__ CUtensorMap map_q,
 #pragma unroll
     for (int i = 0; i < TM; ++i)
 #pragma unroll
-      for (int j = 0; j < kRowsPerThread; ++j) acc[i][j] = tot[0][i][j] = tot[1][i][j] = 0.f;
+      for (int j = 0; j < kRowsPerThread; ++j) tot[i][j] = lost[i][j] = 0.f;
     // What the other slices have published about this tile's queries.
     if (p.qfloor != nullptr && tile > 0 && tid < BM && q0 + tid < p.q) {
       const unsigned long long v =
@@ -312,27 +327,15 @@ f32_search_kernel(const __grid_constant__ CUtensorMap map_q,
         st = 0;
         ph ^= 1u;
       }
-      if ((kb + 1) % kFoldBlocks == 0 || kb + 1 == nkb) {
-        // Every other fold goes to the other second-level sum.  (A branch: the
-        // swap of the two arrays in registers took 6% of the kernel.)
-        if ((kb / kFoldBlocks) & 1) {
+      // The block's sums are added with their rounding errors carried (Kahan).
 #pragma unroll
-          for (int i = 0; i < TM; ++i)
+      for (int i = 0; i < TM; ++i)
 #pragma unroll
-            for (int j = 0; j < kRowsPerThread; ++j) {
-              tot[1][i][j] += acc[i][j];
-              acc[i][j] = 0.f;
-            }
-        } else {
-#pragma unroll
-          for (int i = 0; i < TM; ++i)
-#pragma unroll
-            for (int j = 0; j < kRowsPerThread; ++j) {
-              tot[0][i][j] += acc[i][j];
-              acc[i][j] = 0.f;
-            }
+        for (int j = 0; j < kRowsPerThread; ++j) {
+          const float add = acc[i][j] - lost[i][j], sum = tot[i][j] + add;
+          lost[i][j] = (sum - tot[i][j]) - add;
+          tot[i][j] = sum;
         }
-      }
     }
 
     // ---- selection
@@ -350,7 +353,7 @@ f32_search_kernel(const __grid_constant__ CUtensorMap map_q,
 #pragma unroll
       for (int j = 0; j < kRowsPerThread; ++j) {
         const int64_t r = r0 + tx + TX * j;
-        float v = tot[0][i][j] + tot[1][i][j];
+        float v = tot[i][j];
         if (brow != nullptr && r < r_end)
           v = fmaf(p.fu.alpha, v, (1.f - p.fu.alpha) * (brow[r] * inv_max));
         acc[i][j] = r < r_end && qg < p.q ? v : -INFINITY;
