@@ -10,8 +10,8 @@
 // shared-memory reads touches at most 128 different bytes (measured: 2.1
 // cycles of the SM each; 4.2 for 16 rows or more).  K blocks of 32 floats of
 // both operands come through a TMA ring (128-byte swizzle: eight rows' reads
-// of one k group touch all banks once) that thread 0 feeds between its own
-// blocks: a ninth warp would cap every thread at 168 registers.
+// of one k group touch all banks once) that the warps feed in turn, every eighth
+// block each: a ninth warp would cap every thread at 168 registers.
 //
 // Sums: chains of eight products, four of them added up per K block, and the
 // blocks' sums added with compensation (Kahan), so that the error does not grow
