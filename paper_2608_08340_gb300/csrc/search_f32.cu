@@ -81,6 +81,8 @@ cudaError_t launch_f32_search(const void* E, const void* Q, const SearchShape& s
       !encode_rows_map(&me, E, s.n, s.d, kThreads / c.TY, kF32))
     return cudaErrorInvalidValue;
   Params p{};
+  p.E = static_cast<const float*>(E);
+  p.Q = static_cast<const float*>(Q);
   p.n = s.n;
   p.d = s.d;
   p.q = s.q;

@@ -39,6 +39,8 @@
 // sorted by one warp and cut to its k best; at the end the buffers are sorted
 // into one list per (query, slice) for the merge kernel.
 #pragma once
+#include <cfloat>
+
 #include "common.cuh"
 #include "internal.h"
 
@@ -55,6 +57,8 @@ constexpr int kMaxStages = 16;
 constexpr size_t kSmemMax = 226 * 1024;
 
 struct Params {
+  const float* E;       // n x d
+  const float* Q;       // q x d
   int64_t n;
   int d;
   int q;
@@ -120,6 +124,57 @@ __device__ __forceinline__ void mul_block(const unsigned char* a0, const unsigne
   for (int i = 0; i < TM; ++i)
 #pragma unroll
     for (int j = TN; j < kRowsPerThread; ++j) mid[i][j] = 0.f;
+}
+
+// max(m, |a|, |b|), NaN when one of them is.
+__device__ __forceinline__ float max_abs_nan(float m, float a, float b) {
+  asm("max.NaN.f32 %0, %0, %1, %2;" : "+f"(m) : "f"(fabsf(a)), "f"(fabsf(b)));
+  return m;
+}
+
+// Scores that passed the fp32 range: the carried errors of the sums turn an
+// infinite sum into NaN, so those scores are formed again as plain sums in the
+// order of the dimensions, where an overflowed sum of finite products keeps its
+// infinity.  Looked for once per tile (a check in each K block, to drop the
+// carried errors there, took 6 of 204 us at 100 queries of 32768 x 768).
+// r0, q0: the thread's first corpus row and query; rows end at r_end.
+template <int TY, int TM>
+__device__ __forceinline__ void redo_overflowed(const Params& p, int64_t r0, int64_t r_end, int q0,
+                                                float (&tot)[TM][kRowsPerThread]) {
+  constexpr int TX = kThreads / TY;
+  float worst = 0.f;
+#pragma unroll
+  for (int i = 0; i < TM; ++i)
+#pragma unroll
+    for (int j = 0; j < kRowsPerThread; j += 2)
+      worst = max_abs_nan(worst, tot[i][j], tot[i][j + 1]);
+  if (worst <= FLT_MAX) return;
+  uint32_t redo = 0;                   // bit 4 i + j
+#pragma unroll
+  for (int i = 0; i < TM; ++i)
+#pragma unroll
+    for (int j = 0; j < kRowsPerThread; ++j)
+      if (!(fabsf(tot[i][j]) <= FLT_MAX) && r0 + TX * j < r_end && q0 + TY * i < p.q)
+        redo |= 1u << (kRowsPerThread * i + j);
+#pragma unroll 1
+  for (; redo != 0; redo &= redo - 1) {
+    const int at = __ffs(redo) - 1;
+    const float4* e = reinterpret_cast<const float4*>(
+        p.E + (r0 + TX * (at % kRowsPerThread)) * p.d);
+    const float4* q = reinterpret_cast<const float4*>(
+        p.Q + static_cast<int64_t>(q0 + TY * (at / kRowsPerThread)) * p.d);
+    float s = 0.f;
+#pragma unroll 2
+    for (int t = 0; t < p.d / 4; ++t) {
+      const float4 x = __ldg(e + t), y = __ldg(q + t);
+      s = fmaf(x.w, y.w, fmaf(x.z, y.z, fmaf(x.y, y.y, fmaf(x.x, y.x, s))));
+    }
+#pragma unroll
+    for (int i = 0; i < TM; ++i)
+#pragma unroll
+      for (int j = 0; j < kRowsPerThread; ++j)
+        if (at == kRowsPerThread * i + j) tot[i][j] = s;
+  }
 }
 
 // The warp puts the min(c, k) best of the c keys of a buffer, best first, into
@@ -337,6 +392,8 @@ f32_search_kernel(const __grid_constant__ CUtensorMap map_q,
           tot[i][j] = sum;
         }
     }
+
+    redo_overflowed<TY, TM>(p, r0 + tx, r_end, q0 + ty, tot);
 
     // ---- selection
     // The scores (in the accumulators' place), -inf where there is none.

@@ -77,6 +77,44 @@ def test_rising_scores_replace_every_candidate():
             np.arange(n - 1, n - 11, -1)[None]).all()
 
 
+@pytest.mark.parametrize("q", [3, 40, 100])        # the three tile shapes
+@pytest.mark.parametrize("d", [32, 64, 256, 1000])
+@pytest.mark.parametrize("k", [5, 40])
+def test_overflowing_scores_keep_their_infinity(q, d, k):
+    """Finite rows whose product with a query passes the fp32 range rank first,
+    whether the sum overflows in the first, a middle or the last K block, and a
+    partial sum of the other sign that overflows later does not remove them."""
+    n = 3000
+    rng = np.random.default_rng(d)
+    E = rng.standard_normal((n, d)).astype(np.float32)
+    Q = np.ones((q, d), np.float32)
+    top = [5, 700, 1500, 2999]
+    E[top] = 0
+    E[5] = 3e38
+    E[700, :8] = 3e38
+    E[1500, d // 2:d // 2 + 4] = 3e38
+    E[2999, -2:] = 3e38
+    if d >= 256:                 # both signs, blocks apart
+        top.append(2000)
+        E[2000] = np.where(np.arange(d) < d // 2, 3e38, -3e38)
+    low = 1111
+    E[low] = -3e38
+    idx = Index(dev_tensor(E))
+    ids, sc = idx.search(dev_tensor(Q), k)
+    m = min(k, len(top))
+    assert ids.cpu()[:, :m].tolist() == [sorted(top)[:m]] * q
+    assert torch.isposinf(sc[:, :m]).all() and torch.isfinite(sc[:, m:]).all()
+    assert not (ids == low).any()
+    rest = np.setdiff1d(np.arange(n), top + [low])
+    want = np.sort((E[rest].astype(np.float64).sum(1)))[::-1][:k - m]
+    np.testing.assert_allclose(sc.cpu().numpy()[:, m:], np.broadcast_to(want, (q, k - m)),
+                               rtol=0, atol=2.0 ** -20 * d)
+    idx.check()
+    E[:] = 3e38                  # every score overflows: the lowest ids win
+    ids, sc = Index(dev_tensor(E)).search(dev_tensor(Q), k)
+    assert ids.cpu().tolist() == [list(range(k))] * q and torch.isposinf(sc).all()
+
+
 @pytest.mark.parametrize("q", [6, 70])
 def test_fused_hybrid(q):
     w = workloads.make_dense("f32h", 3000, 64, q, 9, "f32", 7)
