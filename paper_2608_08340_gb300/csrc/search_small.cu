@@ -27,6 +27,7 @@
 // selection of a CTA's queries by its six warps costs more than it saves: 64
 // queries 37 against 31 us.
 #include <algorithm>
+#include <cfloat>
 
 #include "merge.cuh"
 #include "search_tc.cuh"
@@ -285,12 +286,15 @@ small_search_kernel(const __grid_constant__ CUtensorMap map_q,
       __syncwarp();
       if (lane == 0) mbar_arrive(&tempty[acc]);
       if (tile < 2) {
-        // Fixed slots of the first two tiles.
+        // Fixed slots of the first two tiles.  A score of -inf (one that
+        // overflowed) is no result, as in the general kernel.
 #pragma unroll
         for (int i = 0; i < N; ++i)
-          if (i < p.q)
+          if (i < p.q) {
+            const float s = __uint_as_float(v[i]);
             buf[i * kSmallCap + tile * kBlockM + row] =
-                valid ? make_key(__uint_as_float(v[i]), static_cast<uint32_t>(r)) : kEmptyKey;
+                valid && s > -INFINITY ? make_key(s, static_cast<uint32_t>(r)) : kEmptyKey;
+          }
       } else {
 #pragma unroll
         for (int i = 0; i < N; ++i) {
@@ -311,7 +315,7 @@ small_search_kernel(const __grid_constant__ CUtensorMap map_q,
             small_best(b, have, p.k, b);
             if (lane == 0) {
               cnt[c] = p.k;
-              flo[c] = key_floor(b[p.k - 1]);
+              flo[c] = fmaxf(key_floor(b[p.k - 1]), -FLT_MAX);
             }
           }
         }

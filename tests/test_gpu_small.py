@@ -60,3 +60,22 @@ def test_equal_and_rising_scores(q, k):
     ids, sc = idx.search(dev_tensor(Q), k)
     top = (n - 1) // 256 * 256
     assert ids.cpu().tolist() == [list(range(top, top + k))] * q
+
+
+@pytest.mark.parametrize("n", [20, 30000, 60000])         # one, two and four tiles a slice
+@pytest.mark.parametrize("q,k", [(3, 5), (3, 8), (30, 16)])
+def test_scores_of_minus_infinity_are_no_results(n, q, k):
+    """Finite rows whose score overflows to -inf: as in the general kernel, they
+    leave empty results behind the finite scores."""
+    E = np.full((n, 64), -3e38, np.float32)
+    keep = np.linspace(0, n - 1, 7).astype(int)
+    E[keep] = 0
+    E[keep, 0] = np.arange(7) - 3
+    idx = Index(dev_tensor(oracle.round_bf16(E)))
+    Q = dev_tensor(oracle.round_bf16(np.ones((q, 64), np.float32)))
+    want = (keep[::-1].tolist() + [-1] * k)[:k]
+    for mode in (None, "single"):
+        idx.force_pair(mode)
+        ids, sc = idx.search(Q, k)
+        assert ids.cpu().tolist() == [want] * q
+        assert sc.cpu().tolist() == [([3.0, 2, 1, 0, -1, -2, -3] + [-np.inf] * k)[:k]] * q
