@@ -302,7 +302,8 @@ f32_search_kernel(const __grid_constant__ CUtensorMap map_q,
   }
   if (tid < BM) {
     cnt[tid] = 0;
-    flo[tid] = score_order(-INFINITY);
+    // (up to 32 results a score of -inf, one that overflowed, is none)
+    flo[tid] = score_order(p.k <= 32 ? -FLT_MAX : -INFINITY);
   }
   __syncthreads();
 
@@ -424,16 +425,19 @@ f32_search_kernel(const __grid_constant__ CUtensorMap map_q,
 #pragma unroll
       for (int i = 0; i < TM; ++i) {
         const int ql = ty + TY * i;
-        float b;
+        float b, v[kRowsPerThread];
+        // NaN counts for nothing: the sorts' minima and maxima would put a
+        // second copy of another score in its place.
+#pragma unroll
+        for (int j = 0; j < kRowsPerThread; ++j) v[j] = fmaxf(acc[i][j], -INFINITY);
         if (p.k <= 8) {
-          float m[1] = {fmaxf(fmaxf(acc[i][0], acc[i][1]), fmaxf(acc[i][2], acc[i][3]))};
+          float m[1] = {fmaxf(fmaxf(v[0], v[1]), fmaxf(v[2], v[3]))};
           b = rank_of_8<1>(m, p.k - 1);
         } else if (p.k <= 16) {
-          float m[2] = {fmaxf(acc[i][0], acc[i][1]), fmaxf(acc[i][2], acc[i][3])};
+          float m[2] = {fmaxf(v[0], v[1]), fmaxf(v[2], v[3])};
           b = rank_of_8<2>(m, p.k - 1);
         } else {
-          float m[4] = {acc[i][0], acc[i][1], acc[i][2], acc[i][3]};
-          b = rank_of_8<4>(m, p.k - 1);
+          b = rank_of_8<4>(v, p.k - 1);
         }
         if ((lane & 7) == 0 && b > -INFINITY) atomicMax(flo + ql, score_order(b));
       }

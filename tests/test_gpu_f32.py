@@ -115,6 +115,24 @@ def test_overflowing_scores_keep_their_infinity(q, d, k):
     assert ids.cpu().tolist() == [list(range(k))] * q and torch.isposinf(sc).all()
 
 
+@pytest.mark.parametrize("q", [3, 40, 100])
+@pytest.mark.parametrize("n", [20, 30000])
+def test_scores_of_minus_infinity_are_no_results(q, n):
+    """Up to 32 results, as with a bf16 index; above, they rank last."""
+    E = np.full((n, 64), -3e38, np.float32)
+    keep = np.linspace(0, n - 1, 7).astype(int)
+    E[keep] = 0
+    E[keep, 0] = np.arange(7) - 3
+    idx = Index(dev_tensor(E))
+    Q = dev_tensor(np.ones((q, 64), np.float32))
+    low = np.setdiff1d(np.arange(n), keep)
+    for k in (5, 12, 20) if n == 20 else (5, 16, 32, 40):
+        want = (keep[::-1].tolist() + ([-1] * k if k <= 32 else low.tolist()))[:k]
+        ids, sc = idx.search(Q, k)
+        assert ids.cpu().tolist() == [want] * q
+        assert sc.cpu().tolist() == [([3.0, 2, 1, 0, -1, -2, -3] + [-np.inf] * k)[:k]] * q
+
+
 @pytest.mark.parametrize("q", [6, 70])
 def test_fused_hybrid(q):
     w = workloads.make_dense("f32h", 3000, 64, q, 9, "f32", 7)
