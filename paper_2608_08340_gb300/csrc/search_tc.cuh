@@ -1483,6 +1483,10 @@ tc_search_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
             tmem_st32_async(taddr + c * 32, v);
           }
         };
+        // A group of NaN scores (a fused score may be one: a dense weight of 0
+        // times a score that overflowed) bounds nothing; in the sort it would
+        // leave a second copy of another maximum.
+        auto group_max = [](float m) { return kLex == kLexNone ? m : fmaxf(m, -INFINITY); };
         // (Hybrid: no group bound for a fresh list, whose scores would need
         // a second walk of the postings.)
         if constexpr (K <= 32 && !kHybrid) {
@@ -1518,7 +1522,7 @@ tc_search_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
 #pragma unroll
                   for (int i = 1; i + 1 < L; i += 2) m = fmax3(m, v[g * L + i], v[g * L + i + 1]);
                   if constexpr (L % 2 == 0) m = fmaxf(m, v[g * L + L - 1]);
-                  gm[g] = m;
+                  gm[g] = group_max(m);
                 }
               }
               // The k-th largest group maximum (K groups, k <= K).
@@ -1544,7 +1548,7 @@ tc_search_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
 #pragma unroll
                 for (int i = 1; i + 1 < L; i += 2) m = fmax3(m, v[g * L + i], v[g * L + i + 1]);
                 if constexpr (L % 2 == 0) m = fmaxf(m, v[g * L + L - 1]);
-                gm[c * GPC + g] = m;
+                gm[c * GPC + g] = group_max(m);
               }
             }
             fused = kLex == kLexBlock;

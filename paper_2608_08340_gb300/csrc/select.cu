@@ -44,7 +44,8 @@ group_select_kernel(const float* __restrict__ gmax, int64_t gld, int groups, int
 #pragma unroll
   for (int r = 0; r < R; ++r) {
     const int i = r * kSelThreads + tid;
-    v[r] = i < groups ? score_order(__ldcs(g + i)) : 0u;
+    // (NaN, the maximum of a group of NaN scores, holds no score)
+    v[r] = i < groups ? score_order(fmaxf(__ldcs(g + i), -INFINITY)) : 0u;
   }
   const uint32_t none = score_order(-INFINITY);     // a group past the corpus's end
   uint32_t reached = none;

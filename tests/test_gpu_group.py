@@ -87,3 +87,33 @@ def test_reserve_covers_the_group_pass(q, k):
     for kk in {33, k}:
         idx.search(dev_tensor(_rows(rng, q, 64)), kk)
     assert idx.buffer_bytes() == before
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("few", [False, True])
+@pytest.mark.parametrize("q,k", [(3, 5), (40, 12), (100, 30), (40, 50), (300, 200)])
+def test_scores_that_are_not_a_number_prove_no_floor(q, k, few, dtype):
+    """Hybrid with a dense weight of 0: overflowed products give 0 * inf, not a
+    number.  Such chunks are no results, and whole groups of them push no other
+    chunk out."""
+    n = 4000
+    E = np.zeros((n, 64), np.float32)
+    bad = np.arange(64, 224) if few else np.arange(64, 3000)
+    E[bad] = 3e38
+    # Term 1 once in every chunk; its weight falls with the chunk's length, and
+    # each group of eight chunks holds one of the shortest.
+    lens = 1 + np.arange(n) % 8 * 500 + np.arange(n) // 16
+    indptr = np.concatenate([[0], np.cumsum(lens)]).astype(np.int32)
+    terms = np.full(indptr[-1], 2, np.int32)
+    terms[indptr[:-1]] = 1
+    Q = np.ones((q, 64), np.float32)
+    if dtype == "bf16":
+        E, Q = oracle.round_bf16(E), oracle.round_bf16(Q)
+    idx = Index(dev_tensor(E))
+    idx.set_sparse(indptr, terms, 8)
+    ids, sc = idx.hybrid_search(dev_tensor(Q), torch.arange(q + 1, dtype=torch.int32),
+                                torch.ones(q, dtype=torch.int32), 0.0, k)
+    want = np.argsort(lens, kind="stable")
+    want = want[~np.isin(want, bad)][:k]
+    assert ids.cpu().tolist() == [want.tolist()] * q
+    assert torch.isfinite(sc).all()
