@@ -1,5 +1,5 @@
 // Host side of the fp32 search of search_f32.cuh: tile shape, corpus slices and
-// scratch size; query tiles of up to 128 (TY = 16).
+// scratch size.
 #include <algorithm>
 
 #include "search_f32.cuh"
@@ -8,6 +8,23 @@
 namespace oprag {
 
 using namespace f32;
+
+namespace f32 {
+
+extern template cudaError_t launch_ty<4, false>(const Config&, const CUtensorMap&,
+                                                const CUtensorMap&, const Params&, cudaStream_t);
+extern template cudaError_t launch_ty<4, true>(const Config&, const CUtensorMap&,
+                                               const CUtensorMap&, const Params&, cudaStream_t);
+extern template cudaError_t launch_ty<8, false>(const Config&, const CUtensorMap&,
+                                                const CUtensorMap&, const Params&, cudaStream_t);
+extern template cudaError_t launch_ty<8, true>(const Config&, const CUtensorMap&,
+                                               const CUtensorMap&, const Params&, cudaStream_t);
+extern template cudaError_t launch_ty<16, false>(const Config&, const CUtensorMap&,
+                                                 const CUtensorMap&, const Params&, cudaStream_t);
+extern template cudaError_t launch_ty<16, true>(const Config&, const CUtensorMap&,
+                                                const CUtensorMap&, const Params&, cudaStream_t);
+
+}  // namespace f32
 
 namespace {
 
@@ -103,22 +120,12 @@ cudaError_t launch_f32_search(const void* E, const void* Q, const SearchShape& s
   lists->TH = c.th;
   lists->stride = p.stride;
   lists->klen = p.stride;
-  if (c.TY == 4) return launch_ty4(c, mq, me, p, st);
-  if (c.TY == 8) return launch_ty8(c, mq, me, p, st);
-  return launch_ty16(c, mq, me, p, st);
+  const bool fine = s.d <= kFineDim;
+  if (c.TY == 4)
+    return fine ? launch_ty<4, true>(c, mq, me, p, st) : launch_ty<4, false>(c, mq, me, p, st);
+  if (c.TY == 8)
+    return fine ? launch_ty<8, true>(c, mq, me, p, st) : launch_ty<8, false>(c, mq, me, p, st);
+  return fine ? launch_ty<16, true>(c, mq, me, p, st) : launch_ty<16, false>(c, mq, me, p, st);
 }
 
-namespace f32 {
-
-cudaError_t launch_ty16(const Config& c, const CUtensorMap& mq, const CUtensorMap& me,
-                       const Params& p, cudaStream_t st) {
-  switch (c.TM) {
-    case 5: return launch_tm<16, 5>(c, mq, me, p, st);
-    case 6: return launch_tm<16, 6>(c, mq, me, p, st);
-    case 7: return launch_tm<16, 7>(c, mq, me, p, st);
-    default: return launch_tm<16, 8>(c, mq, me, p, st);
-  }
-}
-
-}  // namespace f32
 }  // namespace oprag

@@ -15,11 +15,17 @@
 //
 // Sums: chains of eight products, four of them added up per K block, and the
 // blocks' sums added with compensation (Kahan), so that the error does not grow
-// with d.  Relative error against 64 bits (root mean square over the 10 best of
-// 100 queries), in brackets the streaming kernel's: d = 64 4.4e-8 (3.9e-8), 128
-// 4.3e-8 (4.6e-8), 768 3.6e-8 (5.2e-8), 1280 3.1e-8 (5.4e-8).  One chain of 64
-// products per two blocks, added to two plain sums in turn, gave 11.6e-8, 9.6e-8,
-// 6.8e-8 and 6.8e-8, and 177 us instead of 195 at 100 queries of 32768 x 768.
+// with d.  Up to d = kFineDim the streaming kernel, whose lanes then held one
+// chain of four products each, was closer to 64 bits than that; there the
+// chains have four products and four of them (two up to d = 32) are added up
+// before each compensated addition.  Relative error against 64 bits (root mean
+// square, 1e-8, over the 10 best of 100 queries), in brackets the streaming
+// kernel's: d = 16 4.3 (4.2; 40 queries 4.2 and 4.3), 32 4.0 (4.4), 64 3.9 (4.3),
+// 128 4.0 (4.7), 136 4.2 (4.5), 768 3.3 (5.1), 1280 3.5 (5.9).  With chains of
+// eight throughout 4.7, 4.8, 4.6 and 4.5 up to d = 128, and 263 instead of 285 us
+// (100000 x 64, 256 queries), 66 instead of 73 us (32768 x 64, 100 queries).
+// One chain of 64 products per two blocks, added to two plain sums in turn, gave
+// 6.8 at d = 768 and 177 instead of 195 us at 100 queries of 32768 x 768.
 //
 // What bounds it: from about 16 queries on the FMA pipes and, next to them,
 // the shared-memory reads that feed them (a warp step of four k: 112 FMA issue
@@ -51,7 +57,7 @@ constexpr int kThreads = 256;
 constexpr int kBK = 32;                    // floats per K block: one 128-byte swizzle row
 constexpr int kRowBytes = kBK * 4;
 constexpr int kRowsPerThread = 4;
-constexpr int kChain = 8;                  // products of a first-level sum
+constexpr int kFineDim = 128;              // dimensions of the finer sums
 constexpr int kMaxCap = 512;               // candidate keys per query
 constexpr int kMaxStages = 16;
 constexpr size_t kSmemMax = 226 * 1024;
@@ -86,12 +92,34 @@ struct Config {
   size_t smem;
 };
 
+// Adds sums to the scores with their rounding errors carried (Kahan).
+template <int TM, int TN>
+__device__ __forceinline__ void add_sums(const float (&s)[TM][kRowsPerThread],
+                                         float (&tot)[TM][kRowsPerThread],
+                                         float (&lost)[TM][kRowsPerThread]) {
+#pragma unroll
+  for (int i = 0; i < TM; ++i)
+#pragma unroll
+    for (int j = 0; j < TN; ++j) {
+      const float add = s[i][j] - lost[i][j], sum = tot[i][j] + add;
+      lost[i][j] = (sum - tot[i][j]) - add;
+      tot[i][j] = sum;
+    }
+}
+
 // One K block: eight groups of four k (zeros past d), TN of the thread's four
-// rows.  mid: the block's sums, of chains of kChain products.  a0 / b0: the thread's first query / corpus row of the stage.
-template <int TY, int TM, int TN>
+// rows.  mid: the block's sums, of four chains of eight products, 0 for the
+// other rows.  kFine: chains of four, four of them added up in mid (two when
+// `finest`) and then to the scores.  a0 / b0: the thread's first query / corpus
+// row of the stage.
+template <int TY, int TM, int TN, bool kFine>
 __device__ __forceinline__ void mul_block(const unsigned char* a0, const unsigned char* b0, int ty,
-                                          int tx, float (&mid)[TM][kRowsPerThread]) {
+                                          int tx, float (&mid)[TM][kRowsPerThread],
+                                          float (&tot)[TM][kRowsPerThread],
+                                          float (&lost)[TM][kRowsPerThread], bool finest) {
   constexpr int TX = kThreads / TY;
+  constexpr int kChain = kFine ? 4 : 8;
+  constexpr int kSum = 4 * kChain / 4;              // steps of a second-level sum
   float acc[TM][TN];
 #pragma unroll
   for (int s = 0; s < kBK / 4; ++s) {
@@ -117,13 +145,22 @@ __device__ __forceinline__ void mul_block(const unsigned char* a0, const unsigne
       if (last)
 #pragma unroll
         for (int j = 0; j < TN; ++j)
-          mid[i][j] = s < kChain / 4 ? acc[i][j] : mid[i][j] + acc[i][j];
+          mid[i][j] = s % kSum < kChain / 4 ? acc[i][j] : mid[i][j] + acc[i][j];
+    }
+    if (kFine && (s + 1) % kSum == 0) add_sums<TM, TN>(mid, tot, lost);
+    if (kFine && (s + 1) % kSum == kSum / 2 && finest) {
+      add_sums<TM, TN>(mid, tot, lost);
+#pragma unroll
+      for (int i = 0; i < TM; ++i)
+#pragma unroll
+        for (int j = 0; j < TN; ++j) mid[i][j] = 0.f;
     }
   }
+  if (!kFine)
 #pragma unroll
-  for (int i = 0; i < TM; ++i)
+    for (int i = 0; i < TM; ++i)
 #pragma unroll
-    for (int j = TN; j < kRowsPerThread; ++j) mid[i][j] = 0.f;
+      for (int j = TN; j < kRowsPerThread; ++j) mid[i][j] = 0.f;
 }
 
 // max(m, |a|, |b|), NaN when one of them is.
@@ -263,7 +300,7 @@ __device__ __forceinline__ float rank_of_8(float (&v)[E], int r) {
   return __shfl_sync(0xffffffffu, m, r / E, 8);
 }
 
-template <int TY, int TM>
+template <int TY, int TM, bool kFine>
 __global__ void __launch_bounds__(kThreads, 1)
 f32_search_kernel(const __grid_constant__ CUtensorMap map_q,
                   const __grid_constant__ CUtensorMap map_e, const Params p) {
@@ -289,6 +326,7 @@ f32_search_kernel(const __grid_constant__ CUtensorMap map_q,
   const int64_t r_end = p.n * (blockIdx.x + 1) / gridDim.x;
   const int tiles = static_cast<int>((r_end - r_begin + BN - 1) / BN);
   const int nkb = (p.d + kBK - 1) / kBK;
+  const bool finest = nkb == 1;
 
   if (tid == 0) {
     for (int s = 0; s < p.stages; ++s) {
@@ -373,25 +411,17 @@ f32_search_kernel(const __grid_constant__ CUtensorMap map_q,
       __syncwarp();
       const unsigned char* sB = ring + st * p.stage + tx * kRowBytes;
       const unsigned char* sA = ring + st * p.stage + p.b_bytes + ty * kRowBytes;
-      if (tn == 4) mul_block<TY, TM, 4>(sA, sB, ty, tx, acc);
-      else if (tn == 3) mul_block<TY, TM, 3>(sA, sB, ty, tx, acc);
-      else if (tn == 2) mul_block<TY, TM, 2>(sA, sB, ty, tx, acc);
-      else mul_block<TY, TM, 1>(sA, sB, ty, tx, acc);
+      if (tn == 4) mul_block<TY, TM, 4, kFine>(sA, sB, ty, tx, acc, tot, lost, finest);
+      else if (tn == 3) mul_block<TY, TM, 3, kFine>(sA, sB, ty, tx, acc, tot, lost, finest);
+      else if (tn == 2) mul_block<TY, TM, 2, kFine>(sA, sB, ty, tx, acc, tot, lost, finest);
+      else mul_block<TY, TM, 1, kFine>(sA, sB, ty, tx, acc, tot, lost, finest);
       __syncwarp();
       if (lane == 0) mbar_arrive(&empty[st]);
       if (++st == p.stages) {
         st = 0;
         ph ^= 1u;
       }
-      // The block's sums are added with their rounding errors carried (Kahan).
-#pragma unroll
-      for (int i = 0; i < TM; ++i)
-#pragma unroll
-        for (int j = 0; j < kRowsPerThread; ++j) {
-          const float add = acc[i][j] - lost[i][j], sum = tot[i][j] + add;
-          lost[i][j] = (sum - tot[i][j]) - add;
-          tot[i][j] = sum;
-        }
+      if (!kFine) add_sums<TM, kRowsPerThread>(acc, tot, lost);
     }
 
     redo_overflowed<TY, TM>(p, r0 + tx, r_end, q0 + ty, tot);
@@ -513,28 +543,39 @@ f32_search_kernel(const __grid_constant__ CUtensorMap map_q,
       if (issued & (1u << i)) mbar_drain(&full[i], (parity >> i) & 1u, p.dev_err);
 }
 
-template <int TY, int TM>
+template <int TY, int TM, bool kFine>
 cudaError_t launch_tm(const Config& c, const CUtensorMap& mq, const CUtensorMap& me,
                       const Params& p, cudaStream_t st) {
   static bool configured = false;
   if (!configured) {
-    cudaError_t e = cudaFuncSetAttribute(f32_search_kernel<TY, TM>,
+    cudaError_t e = cudaFuncSetAttribute(f32_search_kernel<TY, TM, kFine>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          static_cast<int>(kSmemMax));
     if (e != cudaSuccess) return e;
     configured = true;
   }
-  f32_search_kernel<TY, TM><<<dim3(c.G, c.qt), kThreads, c.smem, st>>>(mq, me, p);
+  f32_search_kernel<TY, TM, kFine><<<dim3(c.G, c.qt), kThreads, c.smem, st>>>(mq, me, p);
   return cudaGetLastError();
 }
 
-// Instantiations live in their own translation units (parallel builds).
-cudaError_t launch_ty4(const Config& c, const CUtensorMap& mq, const CUtensorMap& me,
-                       const Params& p, cudaStream_t st);
-cudaError_t launch_ty8(const Config& c, const CUtensorMap& mq, const CUtensorMap& me,
-                       const Params& p, cudaStream_t st);
-cudaError_t launch_ty16(const Config& c, const CUtensorMap& mq, const CUtensorMap& me,
-                        const Params& p, cudaStream_t st);
+// Query tiles of up to 8 TY queries.  Instantiated in translation units of
+// their own (parallel builds).
+template <int TY, bool kFine>
+cudaError_t launch_ty(const Config& c, const CUtensorMap& mq, const CUtensorMap& me,
+                      const Params& p, cudaStream_t st) {
+  if constexpr (TY == 4) {
+    if (c.TM == 1) return launch_tm<TY, 1, kFine>(c, mq, me, p, st);
+    if (c.TM == 2) return launch_tm<TY, 2, kFine>(c, mq, me, p, st);
+    if (c.TM == 3) return launch_tm<TY, 3, kFine>(c, mq, me, p, st);
+    if (c.TM == 4) return launch_tm<TY, 4, kFine>(c, mq, me, p, st);
+  }
+  switch (c.TM) {
+    case 5: return launch_tm<TY, 5, kFine>(c, mq, me, p, st);
+    case 6: return launch_tm<TY, 6, kFine>(c, mq, me, p, st);
+    case 7: return launch_tm<TY, 7, kFine>(c, mq, me, p, st);
+    default: return launch_tm<TY, 8, kFine>(c, mq, me, p, st);
+  }
+}
 
 }  // namespace f32
 }  // namespace oprag
