@@ -294,13 +294,9 @@ cudaError_t launch_bm25_matrix(const SparseIndex& sp, int64_t n, const int32_t* 
   constexpr size_t kRow = kDocTile * sizeof(float);
   constexpr size_t kFixed = kBm25Warps * kRow +
                             (3 * kBatchTerms + kBatchQueries + 8) * sizeof(int);
-  static bool configured = false;
-  if (!configured) {
-    e = cudaFuncSetAttribute(bm25_matrix_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             static_cast<int>(kFixed + kBm25MaxRows * kRow));
-    if (e != cudaSuccess) return e;
-    configured = true;
-  }
+  static DeviceOnce once;
+  e = allow_smem(once, bm25_matrix_kernel, kFixed + kBm25MaxRows * kRow);
+  if (e != cudaSuccess) return e;
   // One CTA per SM (its shared memory), fewer when there are fewer items.
   const int64_t items = static_cast<int64_t>(sp.ntiles) * q;
   const int grid = static_cast<int>(std::min<int64_t>(items, num_sms));

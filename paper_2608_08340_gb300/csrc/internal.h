@@ -7,9 +7,25 @@
 #include <cuda_runtime.h>
 #include <cuda_bf16.h>
 
+#include "device_once.h"
+
 namespace oprag {
 
 enum Dtype : int { kF32 = 0, kBF16 = 1 };
+
+// Raises a kernel's limit of dynamic shared memory on the current device, once
+// per device (`once`: a static of the launch function).  cudaGetDevice takes the
+// host well under a tenth of a microsecond.
+template <typename Kernel>
+inline cudaError_t allow_smem(DeviceOnce& once, Kernel* kernel, size_t bytes) {
+  int device = 0;
+  const cudaError_t e = cudaGetDevice(&device);
+  if (e != cudaSuccess) return e;
+  return once.run(device, [&] {
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                static_cast<int>(bytes));
+  });
+}
 
 // Kept-list length used for a requested k: 8, 16 or 32 (register lists), 128
 // or 256 (buffered lists).

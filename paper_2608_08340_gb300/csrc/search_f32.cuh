@@ -546,14 +546,9 @@ f32_search_kernel(const __grid_constant__ CUtensorMap map_q,
 template <int TY, int TM, bool kFine>
 cudaError_t launch_tm(const Config& c, const CUtensorMap& mq, const CUtensorMap& me,
                       const Params& p, cudaStream_t st) {
-  static bool configured = false;
-  if (!configured) {
-    cudaError_t e = cudaFuncSetAttribute(f32_search_kernel<TY, TM, kFine>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         static_cast<int>(kSmemMax));
-    if (e != cudaSuccess) return e;
-    configured = true;
-  }
+  static DeviceOnce once;
+  const cudaError_t e = allow_smem(once, f32_search_kernel<TY, TM, kFine>, kSmemMax);
+  if (e != cudaSuccess) return e;
   f32_search_kernel<TY, TM, kFine><<<dim3(c.G, c.qt), kThreads, c.smem, st>>>(mq, me, p);
   return cudaGetLastError();
 }

@@ -347,14 +347,9 @@ small_search_kernel(const __grid_constant__ CUtensorMap map_q,
 template <int N>
 cudaError_t launch_n(const CUtensorMap& mq, const CUtensorMap& me, const SmallParams& p, int grid,
                      size_t smem, cudaStream_t st) {
-  static bool configured = false;
-  if (!configured) {
-    const cudaError_t e =
-        cudaFuncSetAttribute(small_search_kernel<N>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             static_cast<int>(kSmallSmem));
-    if (e != cudaSuccess) return e;
-    configured = true;
-  }
+  static DeviceOnce once;
+  const cudaError_t e = allow_smem(once, small_search_kernel<N>, kSmallSmem);
+  if (e != cudaSuccess) return e;
   small_search_kernel<N><<<grid, kSmallThreads, smem, st>>>(mq, me, p);
   return cudaGetLastError();
 }

@@ -1651,14 +1651,9 @@ inline cudaLaunchAttribute dependent_attr() {
 template <int BN, int K, int L>
 cudaError_t launch_pair_variant(const TcMaps& m, const TcParams& prm, int grid, cudaStream_t st) {
   constexpr size_t smem = smem_for<BN, K, true, false, false, block_bar_bytes<K, L>()>();
-  static bool configured = false;
-  if (!configured) {
-    cudaError_t e = cudaFuncSetAttribute(tc_search_kernel<BN, K, L, true>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         static_cast<int>(smem));
-    if (e != cudaSuccess) return e;
-    configured = true;
-  }
+  static DeviceOnce once;
+  const cudaError_t e = allow_smem(once, tc_search_kernel<BN, K, L, true>, smem);
+  if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3(grid);
   cfg.blockDim = dim3(threads_for(K));
@@ -1683,14 +1678,9 @@ template <int BN, int K, int L>
 cudaError_t launch_variant(const TcMaps& m, const TcParams& prm, int grid, cudaStream_t st) {
   constexpr bool g = L == kLexGather;
   constexpr size_t smem = smem_for<BN, K, false, false, g, block_bar_bytes<K, L>()>();
-  static bool configured = false;
-  if (!configured) {
-    cudaError_t e = cudaFuncSetAttribute(tc_search_kernel<BN, K, L>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         static_cast<int>(smem));
-    if (e != cudaSuccess) return e;
-    configured = true;
-  }
+  static DeviceOnce once;
+  const cudaError_t e = allow_smem(once, tc_search_kernel<BN, K, L>, smem);
+  if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3(grid);
   cfg.blockDim = dim3(threads_for(K, g));
@@ -1706,14 +1696,9 @@ cudaError_t launch_variant(const TcMaps& m, const TcParams& prm, int grid, cudaS
 template <int K, int L>
 cudaError_t launch_dual_variant(const TcMaps& m, const TcParams& prm, int grid, cudaStream_t st) {
   constexpr size_t smem = smem_for<128, K, false, true, false, block_bar_bytes<K, L>()>();
-  static bool configured = false;
-  if (!configured) {
-    cudaError_t e = cudaFuncSetAttribute(tc_search_kernel<128, K, L, false, true>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         static_cast<int>(smem));
-    if (e != cudaSuccess) return e;
-    configured = true;
-  }
+  static DeviceOnce once;
+  const cudaError_t e = allow_smem(once, tc_search_kernel<128, K, L, false, true>, smem);
+  if (e != cudaSuccess) return e;
   tc_search_kernel<128, K, L, false, true><<<grid, threads_for(K), smem, st>>>(m.q, m.e, m.qb,
                                                                                m.eb, prm);
   return cudaGetLastError();
