@@ -289,11 +289,11 @@ OPRAG_API int oprag_index_set_option(oprag_index *idx, int32_t option, int32_t v
  * reads them.  0 (default) off. */
 #define OPRAG_OPT_TIMING 3
 
-/* OPRAG_OPT_WAIT_LIMIT (test hook): the number of clock cycles a wait of the
- * tensor-core search kernel on one of its pipeline barriers may spin before
- * the kernel gives up, records OPRAG_ERR_DEVICE for oprag_index_check,
- * drains its copies and tensor-core work, frees its tensor memory and
- * returns (the results of that search are then undefined).  0 (default)
+/* OPRAG_OPT_WAIT_LIMIT (test hook): the number of clock cycles a wait of a
+ * search kernel (tensor-core, small-batch or fp32) on one of its pipeline
+ * barriers may spin before the kernel gives up, records OPRAG_ERR_DEVICE for
+ * oprag_index_check, drains its copies and tensor-core work, frees its tensor
+ * memory and returns (the results of that search are then undefined).  0 (default)
  * means about 2^31 cycles (about a second); a small value lets a test make
  * the waits of a real search run out. */
 #define OPRAG_OPT_WAIT_LIMIT 7

@@ -264,6 +264,22 @@ __device__ __forceinline__ void keep_best(uint64_t* buf, int c, int k, uint64_t*
   else sort_best<16>(buf, c, k, dst);
 }
 
+// The newest block copied into a stage (-1: none), where warp w has issued the
+// blocks w, w + 8, ... up to newest[w] (-1: none).  Only that copy can still be
+// in flight: a block is issued after the one before it in its stage has landed.
+// (Its phase is the one to wait for; an older block's phase has the parity of a
+// copy that nobody will issue.)
+__host__ __device__ inline int newest_block(const int* newest, int stages, int stage) {
+  int best = -1;
+  for (int w = 0; w < kThreads / 32; ++w) {
+    int m = newest[w];
+    // the warp's blocks come back to a stage after at most `stages` steps
+    for (int i = 0; i < stages && m > best; ++i, m -= kThreads / 32)
+      if (m % stages == stage) best = m;
+  }
+  return best;
+}
+
 // The value of rank r (0-based, descending) among the 8 E values of each group
 // of eight lanes: a bitonic sort, element l E + e in lane l of the group.
 template <int E>
@@ -359,7 +375,8 @@ f32_search_kernel(const __grid_constant__ CUtensorMap map_q,
   const int blocks = tiles * nkb;
   const int lag = p.stages >= 4 ? 2 : 1;
   int ld_m = warp, ld_s = warp % p.stages, ld_kb = warp % nkb;
-  uint32_t ld_ph = (warp / p.stages) & 1, issued = 0, parity = 0;
+  uint32_t ld_ph = (warp / p.stages) & 1;
+  int ld_last = -1;            // the warp's newest block
   int64_t ld_r0 = r_begin + static_cast<int64_t>(warp / nkb) * BN;
   auto load_next = [&]() {
     if (lane == 0 && !*abort_flag &&
@@ -371,8 +388,7 @@ f32_search_kernel(const __grid_constant__ CUtensorMap map_q,
         tma_load_2d(sB + j * TX * kRowBytes, &map_e, &full[ld_s], ld_kb * kBK,
                     static_cast<int>(ld_r0) + j * TX);
       tma_load_2d(sB + p.b_bytes, &map_q, &full[ld_s], ld_kb * kBK, q0);
-      issued |= 1u << ld_s;
-      parity = (parity & ~(1u << ld_s)) | (ld_ph << ld_s);
+      ld_last = ld_m;
     }
     __syncwarp();
     ld_m += kThreads / 32;
@@ -537,10 +553,18 @@ f32_search_kernel(const __grid_constant__ CUtensorMap map_q,
       }
     }
   }
-  // After a wait gave up, copies may still fly: the CTA outlives them.
-  if (lane == 0 && *abort_flag)
-    for (int i = 0; i < p.stages; ++i)
-      if (issued & (1u << i)) mbar_drain(&full[i], (parity >> i) & 1u, p.dev_err);
+  // After a wait gave up, copies may still fly: the CTA outlives them.  Every
+  // wait lies before the last tile's barriers, so all warps read the same here.
+  if (*abort_flag) {
+    int* newest = reinterpret_cast<int*>(buf);
+    __syncthreads();           // the buffers have been read
+    if (lane == 0) newest[warp] = ld_last;
+    __syncthreads();
+    if (tid < p.stages) {
+      const int m = newest_block(newest, p.stages, tid);
+      if (m >= 0) mbar_drain(&full[tid], (m / p.stages) & 1, p.dev_err);
+    }
+  }
 }
 
 template <int TY, int TM, bool kFine>
