@@ -211,12 +211,12 @@ cudaError_t launch_r(const TIn* hidden, int batch, int tokens, int dim, const ui
     return cudaGetLastError();
   }
   const size_t smem = static_cast<size_t>(dim) * sizeof(float);
-  if (smem > 48 * 1024) {
-    const cudaError_t e =
-        cudaFuncSetAttribute(embed_pool_kernel<TIn, R, true>,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
-    if (e != cudaSuccess) return e;
-  }
+  // (for every dim: with the static shared memory, 48 KB of sums are too many
+  // for a kernel without the opt-in)
+  static DeviceOnce once;
+  const cudaError_t e =
+      allow_smem(once, embed_pool_kernel<TIn, R, true>, R * kPoolThreads * 16 / sizeof(TIn) * sizeof(float));
+  if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3(static_cast<unsigned>(batch) * split);
   cfg.blockDim = dim3(kPoolThreads);

@@ -59,6 +59,19 @@ def test_embed_pool_matches_oracle(dtype, dim, out_dtype):
     assert (out[3] == 0).all()
 
 
+@pytest.mark.parametrize("dtype,dim", [("bf16", 12272), ("bf16", 12280), ("bf16", 12288),
+                                       ("bf16", 12296), ("bf16", 16384), ("f32", 8192)])
+def test_embed_pool_of_wide_rows_in_small_batches(dtype, dim):
+    """Partial sums of a row around 48 KB, where the shared memory opt-in begins."""
+    rng = np.random.default_rng(dim)
+    h = rng.standard_normal((3, 130, dim)).astype(np.float32)
+    h_in = oracle.round_bf16(h) if dtype == "bf16" else h
+    mask = np.ones((3, 130), np.uint8)
+    mask[1, 77:] = 0
+    out = embed_pool(dev_tensor(h_in), torch.from_numpy(mask).cuda(), torch.float32)
+    np.testing.assert_allclose(out.cpu().numpy(), oracle.embed_pool(h_in, mask), rtol=0, atol=ERR)
+
+
 def test_embed_pool_feeds_the_search():
     w = workloads.config(1, n=8000, batch=4)
     rng = np.random.default_rng(11)
