@@ -197,7 +197,9 @@ OPRAG_API int oprag_hybrid_search_dense_first(oprag_index *idx, const void *quer
  *   out         device, batch x dim in out_dtype (OPRAG_BF16: round to nearest
  *               even of the fp32 result), 16-byte aligned; as queries it feeds
  *               oprag_search of an index of the same dim directly.
- * Accumulates in fp32.  Asynchronous on `stream`; needs no index.
+ * Accumulates in fp32, in an order of its own for each row: a row's result is
+ * the same in any batch and with any padding.  Asynchronous on `stream`; needs
+ * no index.
  */
 OPRAG_API int oprag_embed_pool(const void *hidden, int32_t hidden_dtype, int32_t batch,
                                int32_t tokens, int32_t dim, const uint8_t *mask, void *out,

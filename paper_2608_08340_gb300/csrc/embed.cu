@@ -2,18 +2,25 @@
 // padded batch are mean-pooled over its unmasked tokens and L2-normalised,
 // and the vector is written in the index's dtype, ready for oprag_search.
 //
-// One CTA of 256 threads per batch row when the rows fill the SMs twice: thread
-// i accumulates, in fp32, the 16-byte groups i, i + 256, ... of the row's dim
-// elements over the tokens, the loads of kTokenBatch tokens in flight at once;
-// a block reduction of the squared mean gives the norm.  HBM-bound: the
-// unmasked hidden states are read once.
+// A row's result does not depend on the batch it comes in, nor on its padding:
+// tokens belong to eight lanes by their position (eight consecutive tokens to a
+// lane), each lane is summed in order, the lanes are added in order, and the
+// squared norm is summed over the elements in a fixed order, however many CTAs
+// share the row.
 //
-// Smaller batches leave SMs without loads in flight, so a cluster of S CTAs
-// shares a row: CTA r takes the token blocks r, r + S, ... (a padded row's real
-// tokens, which come first, are spread evenly), leaves its partial sums in
-// shared memory and finishes one S-th of the row: it adds the S partial sums,
-// in CTA order, through distributed shared memory, and the squared norms of
-// the parts are exchanged the same way.
+// One CTA of 256 threads per row when the rows fill the SMs twice: thread i
+// accumulates, in fp32, the 16-byte groups i and i + 256 of the row's elements,
+// lane by lane, the loads of eight or sixteen tokens in flight at once; a block
+// reduction of the squared mean gives the norm.  HBM-bound: the unmasked hidden
+// states are read once.
+//
+// Wide rows need more threads and smaller batches leave SMs without loads in
+// flight: then a cluster of SD x ST CTAs shares a row, an SD-th of its elements
+// and an ST-th of its lanes each (a padded row's real tokens, which come first,
+// are spread evenly).  With ST > 1 a CTA leaves its lanes' sums in shared memory
+// and finishes an ST-th of its elements: it adds the eight lanes through
+// distributed shared memory.  Every CTA then forms the whole norm from the squared
+// norms of the groups of all.
 #include <cooperative_groups.h>
 #include <cuda_bf16.h>
 
@@ -25,7 +32,9 @@ namespace oprag {
 namespace {
 
 constexpr int kPoolThreads = 256;
-constexpr int kTokenBatch = 8;
+constexpr int kLanes = 8;               // partial sums of a row
+constexpr int kTokenBlock = 8;          // consecutive tokens of a lane
+constexpr int kMaxShare = 2 * kPoolThreads;      // 16-byte groups of a token per CTA
 
 template <typename TIn>
 struct Group;                                   // one 16-byte group of inputs
@@ -52,198 +61,262 @@ struct Group<float> {
   }
 };
 
+template <int N>
+__device__ __forceinline__ void store_floats(float* dst, const float (&a)[N]) {
+#pragma unroll
+  for (int i = 0; i < N; i += 4)
+    *reinterpret_cast<float4*>(dst + i) = make_float4(a[i], a[i + 1], a[i + 2], a[i + 3]);
+}
+
+// R 16-byte groups per thread and token.  kSplit: a cluster of SD * ST CTAs per
+// row, rank = dim part * ST + lane part.
 template <typename TIn, int R, bool kSplit>
-__global__ void __launch_bounds__(kPoolThreads)
+__global__ void __launch_bounds__(kPoolThreads, 2)
 embed_pool_kernel(const TIn* __restrict__ hidden, int tokens, int dim,
-                  const uint8_t* __restrict__ mask, void* __restrict__ out, int out_bf16) {
+                  const uint8_t* __restrict__ mask, void* __restrict__ out, int out_bf16, int SD,
+                  int ST) {
   namespace cg = cooperative_groups;
   constexpr int N = Group<TIn>::kN;
-  extern __shared__ __align__(16) float part[];   // this CTA's partial sums (dim)
+  constexpr int kBlocks = R == 1 ? 2 : 1;         // of a lane, loaded together
+  extern __shared__ __align__(16) float sums[];   // lanes' sums, then squares
   __shared__ float red[kPoolThreads / 32];
-  __shared__ float part_ss;                       // squared norm of this CTA's part
   __shared__ int part_count;
   cg::cluster_group cluster = cg::this_cluster();
-  const int S = kSplit ? static_cast<int>(cluster.num_blocks()) : 1;
+  const int S = kSplit ? SD * ST : 1;
   const int rank = kSplit ? static_cast<int>(cluster.block_rank()) : 0;
-  const int b = blockIdx.x / S;
+  const int dpart = kSplit ? rank / ST : 0, tpart = kSplit ? rank % ST : 0;
+  const int lane_step = kSplit ? ST : 1;
+  const int b = blockIdx.x / S, wl = threadIdx.x & 31;
   const int groups = dim / N;
-  const uint4* row0 = reinterpret_cast<const uint4*>(hidden + static_cast<int64_t>(b) * tokens * dim);
+  const int share = kSplit ? (groups + SD - 1) / SD : groups;    // groups of a dim part
+  const int first = dpart * share;
+  const int mine = min(share, groups - first);    // (none when <= 0)
+  const uint4* row = reinterpret_cast<const uint4*>(hidden + static_cast<int64_t>(b) * tokens * dim) +
+                     first;
   const uint8_t* mrow = mask + static_cast<int64_t>(b) * tokens;
-  float acc[R][N];
+  float tot[R][N], acc[R][N];
+#pragma unroll
+  for (int r = 0; r < R; ++r)
+#pragma unroll
+    for (int i = 0; i < N; ++i) tot[r][i] = 0.f;
+  // The steps of this CTA's lanes, one after the other: step (l, t) takes the
+  // lane's blocks at t and, with kBlocks = 2, at t + kStride.  The mask of a
+  // step's tokens, a byte per thread of the warp, is read a step ahead.
+  constexpr int kStride = kLanes * kTokenBlock;
+  const int lanes = min(kLanes, (tokens + kTokenBlock - 1) / kTokenBlock);   // that hold tokens
+  auto read_mask = [&](int l, int t) -> uint32_t {
+    const int u = t + (wl & 7) + (wl >> 3) * kStride;
+    return l < lanes && wl < kBlocks * kTokenBlock && u < tokens ? mrow[u] : 0u;
+  };
+  int count = 0;
+  int l = tpart, t = l * kTokenBlock;
+  uint32_t byte = read_mask(l, t);
 #pragma unroll
   for (int r = 0; r < R; ++r)
 #pragma unroll
     for (int i = 0; i < N; ++i) acc[r][i] = 0.f;
-  // Tokens are added in increasing order (a fixed summation order for a given S).
-  constexpr int TB = R <= 2 ? kTokenBatch : kTokenBatch / 2;   // register budget
-  int count = 0;
-  for (int t = rank * TB; t < tokens; t += S * TB) {
-    bool m[TB];
-#pragma unroll
-    for (int u = 0; u < TB; ++u) {
-      m[u] = t + u < tokens && mrow[t + u] != 0;
-      count += static_cast<int>(m[u]);
+#pragma unroll 1
+  while (l < lanes) {
+    const uint32_t m = __ballot_sync(0xffffffffu, byte != 0);
+    const int at = t, lane = l;
+    t += kBlocks * kStride;
+    if (t >= tokens) {
+      l += lane_step;
+      t = l * kTokenBlock;
     }
-    uint4 v[TB][R];
+    byte = read_mask(l, t);
+    if (m != 0) {                                 // (no padding)
+      count += __popc(m);
+      uint4 v[kBlocks * kTokenBlock][R];
 #pragma unroll
-    for (int u = 0; u < TB; ++u)
+      for (int u = 0; u < kBlocks * kTokenBlock; ++u)
 #pragma unroll
-      for (int r = 0; r < R; ++r) {
-        const int g = threadIdx.x + r * kPoolThreads;
-        v[u][r] = m[u] && g < groups ? __ldg(row0 + static_cast<int64_t>(t + u) * groups + g)
-                                     : make_uint4(0, 0, 0, 0);
-      }
+        for (int r = 0; r < R; ++r) {
+          const int g = threadIdx.x + r * kPoolThreads;
+          const int token = at + u % kTokenBlock + u / kTokenBlock * kStride;
+          v[u][r] = ((m >> u) & 1u) && g < mine ? __ldg(row + static_cast<int64_t>(token) * groups + g)
+                                                : make_uint4(0, 0, 0, 0);
+        }
 #pragma unroll
-    for (int u = 0; u < TB; ++u)
+      for (int u = 0; u < kBlocks * kTokenBlock; ++u)
 #pragma unroll
-      for (int r = 0; r < R; ++r)
-        if (m[u]) Group<TIn>::add(v[u][r], acc[r]);
-  }
-  // This CTA's part of the row: groups [g0, g1), its mean and squared norm.
-  int g0 = 0, g1 = groups;
-  if constexpr (kSplit) {
+        for (int r = 0; r < R; ++r)
+          if ((m >> u) & 1u) Group<TIn>::add(v[u][r], acc[r]);
+    }
+    if (l == lane) continue;
+    // The lane is complete.
 #pragma unroll
     for (int r = 0; r < R; ++r) {
       const int g = threadIdx.x + r * kPoolThreads;
-      if (g < groups) {
+      if (kSplit && ST > 1) {
+        if (g < mine) store_floats(sums + (lane / ST * share + g) * N, acc[r]);
+      }
 #pragma unroll
-        for (int i = 0; i < N; i += 4)
-          *reinterpret_cast<float4*>(part + g * N + i) =
-              make_float4(acc[r][i], acc[r][i + 1], acc[r][i + 2], acc[r][i + 3]);
+      for (int i = 0; i < N; ++i) {
+        if (!kSplit || ST == 1) tot[r][i] += acc[r][i];
+        acc[r][i] = 0.f;
       }
     }
-    if (threadIdx.x == 0) part_count = count;
-    cluster.sync();
-    g0 = groups * rank / S;
-    g1 = groups * (rank + 1) / S;
-    count = 0;
-    for (int s = 0; s < S; ++s) count += *cluster.map_shared_rank(&part_count, s);
+  }
+  // The groups that this CTA finishes: [g0, g1) of its dim part.
+  int g0 = 0, g1 = mine;
+  const int finish = kSplit ? (share + ST - 1) / ST : share;
+  if constexpr (kSplit) {
+    if (ST > 1) {
+      if (threadIdx.x == 0) part_count = count;
+      cluster.sync();
+      g0 = tpart * finish;
+      g1 = min(mine, g0 + finish);
+      count = 0;
+      for (int p = 0; p < ST; ++p) count += *cluster.map_shared_rank(&part_count, dpart * ST + p);
 #pragma unroll
-    for (int r = 0; r < R; ++r) {
-      const int g = g0 + threadIdx.x + r * kPoolThreads;
+      for (int r = 0; r < R; ++r) {
+        const int g = g0 + threadIdx.x + r * kPoolThreads;
+        if (g >= g1) continue;
+        float4 x[kLanes][N / 4];
 #pragma unroll
-      for (int i = 0; i < N; ++i) acc[r][i] = 0.f;
-      if (g < g1) {
-        for (int s = 0; s < S; ++s) {
-          const float* p = cluster.map_shared_rank(part, s) + g * N;
+        for (int l = 0; l < kLanes; ++l) {
+          const float4* p = reinterpret_cast<const float4*>(
+              cluster.map_shared_rank(sums, dpart * ST + l % ST) + (l / ST * share + g) * N);
+#pragma unroll
+          for (int i = 0; i < N / 4; ++i)
+            x[l][i] = l < lanes ? p[i] : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+#pragma unroll
+        for (int l = 0; l < kLanes; ++l)
 #pragma unroll
           for (int i = 0; i < N; i += 4) {
-            const float4 v = *reinterpret_cast<const float4*>(p + i);
-            acc[r][i] += v.x;
-            acc[r][i + 1] += v.y;
-            acc[r][i + 2] += v.z;
-            acc[r][i + 3] += v.w;
+            tot[r][i] += x[l][i / 4].x;
+            tot[r][i + 1] += x[l][i / 4].y;
+            tot[r][i + 2] += x[l][i / 4].z;
+            tot[r][i + 3] += x[l][i / 4].w;
           }
-        }
       }
     }
   }
   const float inv_c = count > 0 ? 1.f / static_cast<float>(count) : 0.f;
+  // The squared norm: each group's squares in order, thread i adds the row's
+  // groups i, i + 256, ..., then warps and the CTA are added up.
   float ss = 0.f;
+  float* squares = sums + (kSplit && ST > 1 ? kLanes / ST * share * N : 0);   // a float per group
 #pragma unroll
-  for (int r = 0; r < R; ++r)
+  for (int r = 0; r < R; ++r) {
+    float sq = 0.f;
 #pragma unroll
     for (int i = 0; i < N; ++i) {
-      acc[r][i] *= inv_c;
-      ss = fmaf(acc[r][i], acc[r][i], ss);
+      tot[r][i] *= inv_c;
+      sq = fmaf(tot[r][i], tot[r][i], sq);
     }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = ss;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    float t = 0.f;
-    for (int w = 0; w < kPoolThreads / 32; ++w) t += red[w];
-    part_ss = t;
+    if constexpr (kSplit) {
+      const int g = g0 + threadIdx.x + r * kPoolThreads;
+      if (g < g1) squares[g - g0] = sq;
+    } else {
+      ss += sq;
+    }
   }
-  float total = 0.f;
   if constexpr (kSplit) {
     cluster.sync();
-    for (int s = 0; s < S; ++s) total += *cluster.map_shared_rank(&part_ss, s);
-  } else {
-    __syncthreads();
-    total = part_ss;
+#pragma unroll 4
+    for (int g = threadIdx.x; g < groups; g += kPoolThreads) {
+      const int d = g / share, q = (g - d * share) / finish;
+      ss += cluster.map_shared_rank(squares, d * ST + q)[g - d * share - q * finish];
+    }
+    cluster.barrier_arrive();             // this CTA reads no more
   }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
+  if (wl == 0) red[threadIdx.x >> 5] = ss;
+  __syncthreads();
+  float total = 0.f;
+#pragma unroll
+  for (int w = 0; w < kPoolThreads / 32; ++w) total += red[w];
   const float norm = sqrtf(total);
   const float scale = count > 0 && norm > 0.f ? 1.f / norm : 0.f;
 #pragma unroll
   for (int r = 0; r < R; ++r) {
     const int g = g0 + threadIdx.x + r * kPoolThreads;
     if (g >= g1) continue;
-    const int64_t e0 = static_cast<int64_t>(b) * dim + static_cast<int64_t>(g) * N;
+    const int64_t o0 = static_cast<int64_t>(b) * dim + static_cast<int64_t>(first + g) * N;
     if (out_bf16) {
-      __nv_bfloat16* o = static_cast<__nv_bfloat16*>(out) + e0;
+      __nv_bfloat16* o = static_cast<__nv_bfloat16*>(out) + o0;
 #pragma unroll
       for (int i = 0; i < N; i += 2)
         *reinterpret_cast<__nv_bfloat162*>(o + i) =
-            __floats2bfloat162_rn(acc[r][i] * scale, acc[r][i + 1] * scale);
+            __floats2bfloat162_rn(tot[r][i] * scale, tot[r][i + 1] * scale);
     } else {
-      float* o = static_cast<float*>(out) + e0;
 #pragma unroll
-      for (int i = 0; i < N; i += 4)
-        *reinterpret_cast<float4*>(o + i) = make_float4(acc[r][i] * scale, acc[r][i + 1] * scale,
-                                                        acc[r][i + 2] * scale, acc[r][i + 3] * scale);
+      for (int i = 0; i < N; ++i) tot[r][i] *= scale;
+      store_floats(static_cast<float*>(out) + o0, tot[r]);
     }
   }
-  if constexpr (kSplit) cluster.sync();   // the peers have read this CTA's shared memory
+  if constexpr (kSplit) cluster.barrier_wait();   // nor do the peers read from it
 }
 
-// CTAs per row: as many as keep the batch within two CTAs per SM, at most
-// eight (the portable cluster size) and one per block of tokens.  Measured on
-// GB300 against one CTA per row, bf16: 1 x 512 x 4096 11.8 (41.0) us, 8 x 512 x
-// 4096 13.1 (55.0) us, 64 x 512 x 4096 37.1 (82.0) us, 152 x 512 x 4096 72.5
-// (88.5) us, 1 x 64 x 768 4.3 (5.7) us; 256 x 512 x 4096 stays at one (118 us;
-// split in two 121 us).
-int split_for(int batch, int tokens, int num_sms) {
-  int s = 1;
-  while (s < 8 && static_cast<int64_t>(batch) * 2 * s <= 2 * num_sms &&
-         2 * s * kTokenBatch <= tokens)
-    s *= 2;
+// Parts of a row's elements, so that a CTA takes two groups a thread at most, and
+// of its lanes: as many as keep the batch within two CTAs per SM, with eight
+// CTAs (the portable cluster size) and one per two blocks of tokens at most.
+// Measured on GB300 with events (a pair takes 6 us of it), in brackets one CTA
+// per row and one chain of tokens, bf16: 1 x 512 x 4096 22 (85) us, 8 x 512 x 4096
+// 23 (87) us, 64 x 512 x 4096 62 (94) us, 152 x 512 x 4096 122 (116) us, or 90
+// (101) us with padded rows, 1 x 64 x 768 10 (13) us, 128 x 256 x 768 23 (37) us,
+// 20 x 512 x 8192 38 (148) us, 4 x 300 x 16384 38 (132) us; 256 x 512 x 4096 stays
+// at one CTA (134, 135 us).
+struct Split {
+  int dim, lanes;
+};
+
+Split split_for(int batch, int tokens, int groups, int num_sms) {
+  Split s{1, 1};
+  while (s.dim < 8 && groups > s.dim * kMaxShare) s.dim *= 2;
+  while (s.dim * s.lanes < 8 && static_cast<int64_t>(batch) * 2 * s.dim * s.lanes <= 2 * num_sms &&
+         2 * s.lanes * kTokenBlock <= tokens)
+    s.lanes *= 2;
   return s;
 }
 
 template <typename TIn, int R>
 cudaError_t launch_r(const TIn* hidden, int batch, int tokens, int dim, const uint8_t* mask,
-                     void* out, int out_bf16, int split, cudaStream_t st) {
-  if (split == 1) {
+                     void* out, int out_bf16, Split s, cudaStream_t st) {
+  if (s.dim * s.lanes == 1) {
     embed_pool_kernel<TIn, R, false><<<batch, kPoolThreads, 0, st>>>(hidden, tokens, dim, mask, out,
-                                                                     out_bf16);
+                                                                     out_bf16, 1, 1);
     return cudaGetLastError();
   }
-  const size_t smem = static_cast<size_t>(dim) * sizeof(float);
-  // (for every dim: with the static shared memory, 48 KB of sums are too many
-  // for a kernel without the opt-in)
+  // the lanes' sums of a part, and a float per group
+  constexpr int kGroupBytes = Group<TIn>::kN * sizeof(float);
+  const int lanes_bytes = s.lanes > 1 ? kLanes / s.lanes * kGroupBytes : 0;
   static DeviceOnce once;
-  const cudaError_t e =
-      allow_smem(once, embed_pool_kernel<TIn, R, true>, R * kPoolThreads * 16 / sizeof(TIn) * sizeof(float));
+  const cudaError_t e = allow_smem(once, embed_pool_kernel<TIn, R, true>,
+                                   R * kPoolThreads * (kLanes / 2 * kGroupBytes + sizeof(float)));
   if (e != cudaSuccess) return e;
+  const size_t share = (dim / Group<TIn>::kN + s.dim - 1) / s.dim;
   cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3(static_cast<unsigned>(batch) * split);
+  cfg.gridDim = dim3(static_cast<unsigned>(batch) * s.dim * s.lanes);
   cfg.blockDim = dim3(kPoolThreads);
-  cfg.dynamicSmemBytes = smem;
+  cfg.dynamicSmemBytes = share * (lanes_bytes + sizeof(float));
   cfg.stream = st;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = split;
+  attr[0].val.clusterDim.x = s.dim * s.lanes;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, embed_pool_kernel<TIn, R, true>, hidden, tokens, dim, mask, out,
-                            out_bf16);
+                            out_bf16, s.dim, s.lanes);
 }
 
 template <typename TIn>
 cudaError_t launch_typed(const void* hidden, int batch, int tokens, int dim, const uint8_t* mask,
-                         void* out, int out_bf16, int split, cudaStream_t st) {
+                         void* out, int out_bf16, int num_sms, cudaStream_t st) {
   const int groups = dim / Group<TIn>::kN;
-  const int r = (groups + kPoolThreads - 1) / kPoolThreads;
+  const Split s = split_for(batch, tokens, groups, num_sms);
+  const int share = (groups + s.dim - 1) / s.dim;
+  if (share > kMaxShare) return cudaErrorInvalidValue;
   const TIn* h = static_cast<const TIn*>(hidden);
-  if (r <= 1) return launch_r<TIn, 1>(h, batch, tokens, dim, mask, out, out_bf16, split, st);
-  if (r <= 2) return launch_r<TIn, 2>(h, batch, tokens, dim, mask, out, out_bf16, split, st);
-  if (r <= 4) return launch_r<TIn, 4>(h, batch, tokens, dim, mask, out, out_bf16, split, st);
-  if (r <= 8) return launch_r<TIn, 8>(h, batch, tokens, dim, mask, out, out_bf16, split, st);
-  return cudaErrorInvalidValue;
+  if (share <= kPoolThreads)
+    return launch_r<TIn, 1>(h, batch, tokens, dim, mask, out, out_bf16, s, st);
+  return launch_r<TIn, 2>(h, batch, tokens, dim, mask, out, out_bf16, s, st);
 }
 
 }  // namespace
@@ -256,10 +329,9 @@ cudaError_t launch_embed_pool(int hidden_dtype, const void* hidden, int batch, i
   cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (e != cudaSuccess) return e;
-  const int split = split_for(batch, tokens, sms);
   return hidden_dtype == kBF16
-             ? launch_typed<uint16_t>(hidden, batch, tokens, dim, mask, out, out_bf16, split, st)
-             : launch_typed<float>(hidden, batch, tokens, dim, mask, out, out_bf16, split, st);
+             ? launch_typed<uint16_t>(hidden, batch, tokens, dim, mask, out, out_bf16, sms, st)
+             : launch_typed<float>(hidden, batch, tokens, dim, mask, out, out_bf16, sms, st);
 }
 
 }  // namespace oprag

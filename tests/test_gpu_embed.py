@@ -72,6 +72,38 @@ def test_embed_pool_of_wide_rows_in_small_batches(dtype, dim):
     np.testing.assert_allclose(out.cpu().numpy(), oracle.embed_pool(h_in, mask), rtol=0, atol=ERR)
 
 
+# Batches whose rows one CTA takes alone (400 rows, or fewer than 16 tokens), and
+# two, four and eight share; widths whose groups do not divide among them.
+@pytest.mark.parametrize("b,t", [(400, 9), (3, 15), (152, 40), (60, 33), (20, 70), (1, 512)])
+@pytest.mark.parametrize("dtype,dim", [("bf16", 8), ("bf16", 136), ("bf16", 2056), ("bf16", 4104),
+                                       ("f32", 8), ("f32", 1032), ("f32", 2056)])
+def test_embed_pool_at_every_split(b, t, dtype, dim):
+    rng = np.random.default_rng(b + dim)
+    h = rng.standard_normal((b, t, dim)).astype(np.float32)
+    h_in = oracle.round_bf16(h) if dtype == "bf16" else h
+    mask = (rng.random((b, t)) < 0.7).astype(np.uint8)
+    mask[:, 0] = 1
+    out = embed_pool(dev_tensor(h_in), torch.from_numpy(mask).cuda(), torch.float32)
+    np.testing.assert_allclose(out.cpu().numpy(), oracle.embed_pool(h_in, mask), rtol=0, atol=ERR)
+
+
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+@pytest.mark.parametrize("dim,tokens", [(768, 70), (1000, 300), (4096, 128), (8192, 40)])
+def test_a_row_does_not_depend_on_its_batch(dtype, dim, tokens):
+    """The same bits alone, in batches of every split and with more padding."""
+    g = torch.Generator(device="cuda").manual_seed(dim)
+    h = torch.randn(400, tokens, dim, generator=g, device="cuda").to(dtype)
+    mask = (torch.rand(400, tokens, generator=g, device="cuda") < 0.8).to(torch.uint8)
+    whole = embed_pool(h, mask, torch.float32)
+    for b in (1, 2, 19, 40, 80, 160, 310):
+        assert torch.equal(embed_pool(h[:b], mask[:b], torch.float32), whole[:b]), b
+    wide = torch.zeros(5, tokens + 90, dim, dtype=dtype, device="cuda")
+    wide[:, :tokens] = h[:5]
+    wide_mask = torch.zeros(5, tokens + 90, dtype=torch.uint8, device="cuda")
+    wide_mask[:, :tokens] = mask[:5]
+    assert torch.equal(embed_pool(wide, wide_mask, torch.float32), whole[:5])
+
+
 def test_embed_pool_feeds_the_search():
     w = workloads.config(1, n=8000, batch=4)
     rng = np.random.default_rng(11)
