@@ -54,7 +54,7 @@ constexpr int kBatchQueries = 120;
 constexpr int kBatchTerms = 2048;
 
 // One lane's term of a query: its dense row (-1: postings [lo, hi) of the
-// tile, -2: none).
+// tile's cell, -2: none).
 struct TermSlot {
   int slot, lo, hi;
 };
@@ -65,8 +65,9 @@ __device__ __forceinline__ TermSlot load_term(const SparseIndex& sp,
   TermSlot t{-2, 0, 0};
   const int32_t term = ti < t1 ? q_terms[ti] : -1;
   if (term >= 0 && term < sp.vocab) {
-    const int32_t* tp = sp.tile_ptr + static_cast<int64_t>(term) * (sp.ntiles + 1) + tile;
+    const int64_t row = sp.row_of(term);
     t.slot = sp.dense_slot[term];
+    const int32_t* tp = tile_cell(sp.tile_ptr, row, tile);
     t.lo = tp[0];
     t.hi = tp[1];
   }
@@ -184,14 +185,19 @@ bm25_matrix_kernel(SparseIndex sp, int64_t n, const int32_t* __restrict__ q_indp
           }
 #pragma unroll
           for (int h = 0; h < kChunks; ++h) {
-            // (one term's chunks are distinct: all reads before the writes)
+            // (one term's chunks are distinct: all reads before the writes;
+            // chunk -1 and a wider cell's other tiles are outside the row)
             float v[kPostBatch];
 #pragma unroll
-            for (int u = 0; u < kPostBatch; ++u)
-              if (e[h][u].x >= 0) v[u] = row[e[h][u].x - first_doc];
+            for (int u = 0; u < kPostBatch; ++u) {
+              const uint32_t at = static_cast<uint32_t>(e[h][u].x) - static_cast<uint32_t>(first_doc);
+              if (at < kDocTile) v[u] = row[at];
+            }
 #pragma unroll
-            for (int u = 0; u < kPostBatch; ++u)
-              if (e[h][u].x >= 0) row[e[h][u].x - first_doc] = v[u] + __int_as_float(e[h][u].y);
+            for (int u = 0; u < kPostBatch; ++u) {
+              const uint32_t at = static_cast<uint32_t>(e[h][u].x) - static_cast<uint32_t>(first_doc);
+              if (at < kDocTile) row[at] = v[u] + __int_as_float(e[h][u].y);
+            }
             __syncwarp();
           }
         }

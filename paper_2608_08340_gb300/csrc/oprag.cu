@@ -108,6 +108,7 @@ struct oprag_index {
   int dense_rows = 0;
   int64_t dense_ld = 0;
   int32_t* tile_ptr = nullptr;
+  int64_t* tile_row = nullptr;
   int ntiles = 0;
   void* wsplit = nullptr;      // n x kLexK bf16 head-term weights (high | low halves)
   int32_t* lex_class = nullptr;  // vocab: epilogue class of each term (see rebuild_sparse)
@@ -191,6 +192,7 @@ struct oprag_index {
     if (dense_slot) cudaFree(dense_slot);
     if (dense_w) cudaFree(dense_w);
     if (tile_ptr) cudaFree(tile_ptr);
+    if (tile_row) cudaFree(tile_row);
     if (wsplit) cudaFree(wsplit);
     if (lex_class) cudaFree(lex_class);
     if (mid_w) cudaFree(mid_w);
@@ -202,6 +204,7 @@ struct oprag_index {
     dense_slot = nullptr;
     dense_w = nullptr;
     tile_ptr = nullptr;
+    tile_row = nullptr;
     has_sparse = false;
   }
 };
@@ -1051,6 +1054,36 @@ int oprag_search_host(oprag_index* idx, const void* queries, int32_t q, int32_t 
   return *static_cast<volatile int*>(idx->err_host) != 0 ? oprag_index_check(idx) : ok();
 }
 
+// Each term's row of the tile table (see SparseIndex; left empty when all rows
+// are full); returns the table's entries.  A full row, an entry per tile of 1024 chunks, for every term would
+// take 125 MB at a million chunks and 30522 terms and 12 GB at a hundred million,
+// most of it for rare terms.  So unless it is small, the table is held to 8
+// bytes per term and 8192 chunks: rows get a cell per P postings at most, with
+// the smallest power of two P that fits (a cell per term, the least, always
+// does).  A tile then also reads its cell's other postings, some P of them where
+// it would have read none.
+size_t tile_rows(const std::vector<int64_t>& df, const std::vector<int32_t>& slot, int64_t n,
+                 int ntiles, std::vector<int64_t>* rows) {
+  constexpr int64_t kSmallTable = int64_t(8) << 20;
+  const int64_t vocab = static_cast<int64_t>(df.size());
+  const int64_t limit = std::max(kSmallTable, vocab * (n / 8192 + 2) * 8);
+  rows->clear();
+  const int64_t full = vocab * (ntiles + 1);
+  if (full * 4 <= limit) return static_cast<size_t>(full);
+  rows->resize(df.size());
+  for (int64_t P = 1;; P *= 2) {
+    int64_t entries = 0;
+    for (size_t t = 0; t < df.size(); ++t) {
+      const int64_t postings = slot[t] < 0 ? df[t] : 0;
+      int shift = 0, cells = ntiles;
+      while (cells > 1 && cells * P > postings) cells = ((ntiles - 1) >> ++shift) + 1;
+      (*rows)[t] = tile_row_of(entries, shift);
+      entries += cells + 1;
+    }
+    if (entries * 4 + vocab * 8 <= limit || P > n) return static_cast<size_t>(entries);
+  }
+}
+
 // Builds the device side of BM25 from the index's host copy of the token
 // bags.  Called whenever the bags or the chunk count change, so that df,
 // avgdl and every weight follow the current corpus.  The host does the
@@ -1188,7 +1221,8 @@ int rebuild_sparse(oprag_index* idx) {
   const size_t dense_elems = std::max<size_t>(static_cast<size_t>(n_dense) * dld, 4);
   const size_t wsplit_elems = static_cast<size_t>(n) * kLexK;
   const size_t mid_elems = static_cast<size_t>(std::max(n_mid, 1)) * mld;
-  const size_t tptr_elems = static_cast<size_t>(vocab) * (ntiles + 1);
+  std::vector<int64_t> tile_row;
+  const size_t tptr_elems = tile_rows(df, slot, n, ntiles, &tile_row);
   // temporaries of the build: the inverted index, term offsets, idf, lengths
   int2* d_inv = nullptr;
   int64_t* d_start = nullptr;
@@ -1205,6 +1239,8 @@ int rebuild_sparse(oprag_index* idx) {
       cudaMalloc(&idx->dense_slot, slot.size() * sizeof(int32_t)) != cudaSuccess ||
       cudaMalloc(&idx->dense_w, dense_elems * sizeof(float)) != cudaSuccess ||
       cudaMalloc(&idx->tile_ptr, tptr_elems * sizeof(int32_t)) != cudaSuccess ||
+      (!tile_row.empty() &&
+       cudaMalloc(&idx->tile_row, tile_row.size() * sizeof(int64_t)) != cudaSuccess) ||
       cudaMalloc(&idx->wsplit, wsplit_elems * sizeof(uint16_t)) != cudaSuccess ||
       cudaMalloc(&idx->lex_class, lex_class.size() * sizeof(int32_t)) != cudaSuccess ||
       cudaMalloc(&idx->mid_w, mid_elems * sizeof(float)) != cudaSuccess ||
@@ -1222,6 +1258,9 @@ int rebuild_sparse(oprag_index* idx) {
     e = cudaMemcpy(idx->dense_slot, slot.data(), slot.size() * sizeof(int32_t), cudaMemcpyHostToDevice);
   if (e == cudaSuccess)
     e = cudaMemcpy(idx->lex_class, lex_class.data(), lex_class.size() * sizeof(int32_t),
+                   cudaMemcpyHostToDevice);
+  if (e == cudaSuccess && !tile_row.empty())
+    e = cudaMemcpy(idx->tile_row, tile_row.data(), tile_row.size() * sizeof(int64_t),
                    cudaMemcpyHostToDevice);
   if (e == cudaSuccess)
     e = cudaMemcpy(d_inv, inv.data(), inv.size() * sizeof(int2), cudaMemcpyHostToDevice);
@@ -1241,7 +1280,7 @@ int rebuild_sparse(oprag_index* idx) {
                       idx->dense_slot, idx->lex_class, idx->post_ptr, idx->post,
                       idx->dense_w, dld,
                       reinterpret_cast<__nv_bfloat16*>(idx->wsplit), idx->mid_w, mld};
-    e = launch_lex_build(lb, ntiles, idx->tile_ptr, nullptr);
+    e = launch_lex_build(lb, ntiles, idx->tile_row, idx->tile_ptr, nullptr);
   }
   if (e == cudaSuccess) e = cudaDeviceSynchronize();
   free_tmp();
@@ -1343,7 +1382,7 @@ int oprag_hybrid_search(oprag_index* idx, const void* queries, int32_t q, const 
   if ((rc = begin_call(idx, st))) return rc;
   const SparseIndex sp{idx->vocab,      idx->nnz,     idx->post_ptr, idx->post,
                        idx->dense_slot, idx->dense_w, idx->dense_rows, idx->dense_ld,
-                       idx->tile_ptr,   idx->ntiles};
+                       idx->tile_ptr,   idx->tile_row, idx->ntiles};
   char* lex = reinterpret_cast<char*>(idx->lex);
   if (gather) {
     // Gathered form (Sec. 4.4 fusion in the dense epilogue): per-query
@@ -1434,7 +1473,7 @@ int oprag_hybrid_search_dense_first(oprag_index* idx, const void* queries, int32
   if ((rc = run_search(idx, queries, q, nc, none, cid, csc, st))) return rc;
   const SparseIndex sp{idx->vocab,      idx->nnz,     idx->post_ptr, idx->post,
                        idx->dense_slot, idx->dense_w, idx->dense_rows, idx->dense_ld,
-                       idx->tile_ptr,   idx->ntiles};
+                       idx->tile_ptr,   idx->tile_row, idx->ntiles};
   cudaError_t e = launch_rerank(sp, q, nc, cid, csc, q_indptr, q_terms, alpha, k, out_ids,
                                 out_scores, st);
   if (e != cudaSuccess) return cuda_fail(e, "rerank kernel");

@@ -6,8 +6,8 @@
 // One CTA of four warps per query; a thread holds one or two candidates.  A
 // candidate's BM25 is the sum of its query terms' weights: a dense term's
 // weight is read from its row, a sparse term's is found by a binary search of
-// the term's postings in the candidate's 1024-chunk tile (the table of the BM25
-// pass gives their range).  The searches' scattered reads of L2 bound the
+// the term's postings around the candidate's 1024-chunk tile (the table of the
+// BM25 pass gives their range).  The searches' scattered reads of L2 bound the
 // kernel, and their latency, so a thread searches kTermBatch terms at once.
 // The sums and the fused score are formed exactly as in the BM25 pass and the
 // fused search epilogue, so with every chunk a candidate the result equals the
@@ -33,7 +33,7 @@ rerank_kernel(SparseIndex sp, int ncand, const int64_t* __restrict__ cand_ids,
               const int32_t* __restrict__ q_terms, float alpha, int k,
               int64_t* __restrict__ out_ids, float* __restrict__ out_scores) {
   __shared__ int term_slot[kTermBatch];            // dense row, -1: postings, -2: no term
-  __shared__ int64_t term_row[kTermBatch];         // the term's row of the tile table
+  __shared__ int64_t term_row[kTermBatch];         // the term's tile_row
   __shared__ uint64_t keys[kRerankThreads * E];
   __shared__ float warp_max[kRerankThreads / 32];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -54,20 +54,23 @@ rerank_kernel(SparseIndex sp, int ncand, const int64_t* __restrict__ cand_ids,
     __syncthreads();        // the previous batch's term table has been read
     if (tid < kTermBatch) {
       int slot = -2;
+      int64_t row = 0;
       const int32_t term = base + tid < t1 ? q_terms[base + tid] : -1;
-      if (term >= 0 && term < sp.vocab) slot = sp.dense_slot[term];
+      if (term >= 0 && term < sp.vocab) {
+        slot = sp.dense_slot[term];
+        row = sp.row_of(term);
+      }
       term_slot[tid] = slot >= 0 ? (with_dense ? slot : -2) : (with_sparse ? slot : -2);
-      term_row[tid] = static_cast<int64_t>(term) * (sp.ntiles + 1);
+      term_row[tid] = row;
     }
     __syncthreads();
     // Dense weights, and each candidate's part of the sparse terms' postings:
-    // those of the candidate's tile of chunks.
+    // those of the cell of the candidate's tile of chunks.
     float w[kTermBatch][E];
     int lo[kTermBatch][E], hi[kTermBatch][E], end[kTermBatch][E];
 #pragma unroll
     for (int b = 0; b < kTermBatch; ++b) {
       const int slot = term_slot[b];
-      const int32_t* tp = sp.tile_ptr + term_row[b];
 #pragma unroll
       for (int e = 0; e < E; ++e) {
         w[b][e] = 0.f;
@@ -75,8 +78,9 @@ rerank_kernel(SparseIndex sp, int ncand, const int64_t* __restrict__ cand_ids,
         if (doc[e] < 0) continue;
         if (slot >= 0) w[b][e] = __ldg(sp.dense_w + slot * sp.dense_ld + doc[e]);
         if (slot == -1) {
-          lo[b][e] = __ldg(tp + doc[e] / kBm25DocTile);
-          hi[b][e] = __ldg(tp + doc[e] / kBm25DocTile + 1);
+          const int32_t* tp = tile_cell(sp.tile_ptr, term_row[b], doc[e] / kBm25DocTile);
+          lo[b][e] = __ldg(tp);
+          hi[b][e] = __ldg(tp + 1);
         }
       }
     }

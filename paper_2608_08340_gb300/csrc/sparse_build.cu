@@ -56,35 +56,42 @@ __global__ void lex_weights_kernel(LexBuild lb) {
   }
 }
 
-// One thread per (term, tile boundary b): the first posting of the term whose
-// chunk is >= b * kBm25DocTile.
+// One warp per term (grid-stride over terms): the entries of its row, each the
+// first posting whose chunk is in the cell or behind it.
 __global__ void tile_ptr_kernel(const int64_t* __restrict__ post_ptr, const int2* __restrict__ post,
-                                int vocab, int ntiles, int32_t* __restrict__ tile_ptr) {
-  const int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
-  const int64_t per = ntiles + 1;
-  if (i >= static_cast<int64_t>(vocab) * per) return;
-  const int64_t t = i / per, b = i % per;
-  const int64_t doc0 = b * kBm25DocTile;
-  int64_t lo = post_ptr[t], hi = post_ptr[t + 1];
-  while (lo < hi) {
-    const int64_t mid = (lo + hi) >> 1;
-    if (post[mid].x < doc0) lo = mid + 1; else hi = mid;
+                                int vocab, int ntiles, const int64_t* __restrict__ tile_row,
+                                int32_t* __restrict__ tile_ptr) {
+  const int lane = threadIdx.x & 31;
+  const int64_t warp0 = (static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
+  const int64_t nwarps = (static_cast<int64_t>(gridDim.x) * blockDim.x) >> 5;
+  for (int64_t t = warp0; t < vocab; t += nwarps) {
+    const int64_t row = tile_row != nullptr ? tile_row[t] : tile_row_of(t * (ntiles + 1), 0);
+    const int shift = static_cast<int>(row & ((1 << kTileShiftBits) - 1));
+    const int cells = ((ntiles - 1) >> shift) + 1;
+    for (int c = lane; c <= cells; c += 32) {
+      const int64_t doc0 = (static_cast<int64_t>(c) << shift) * kBm25DocTile;
+      int64_t lo = post_ptr[t], hi = post_ptr[t + 1];
+      while (lo < hi) {
+        const int64_t mid = (lo + hi) >> 1;
+        if (post[mid].x < doc0) lo = mid + 1; else hi = mid;
+      }
+      tile_ptr[(row >> kTileShiftBits) + c] = static_cast<int32_t>(lo);
+    }
   }
-  tile_ptr[i] = static_cast<int32_t>(lo);
 }
 
 }  // namespace
 
-cudaError_t launch_lex_build(const LexBuild& lb, int ntiles, int32_t* tile_ptr, cudaStream_t st) {
+cudaError_t launch_lex_build(const LexBuild& lb, int ntiles, const int64_t* tile_row,
+                             int32_t* tile_ptr, cudaStream_t st) {
   if (lb.vocab <= 0) return cudaSuccess;
   const int64_t warps = lb.vocab;
   const int blocks = static_cast<int>(std::min<int64_t>((warps + 7) / 8, 8192));
   lex_weights_kernel<<<blocks, 256, 0, st>>>(lb);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  const int64_t cells = static_cast<int64_t>(lb.vocab) * (ntiles + 1);
-  tile_ptr_kernel<<<static_cast<unsigned>((cells + 255) / 256), 256, 0, st>>>(
-      lb.post_ptr, lb.post, lb.vocab, ntiles, tile_ptr);
+  tile_ptr_kernel<<<blocks, 256, 0, st>>>(lb.post_ptr, lb.post, lb.vocab, ntiles, tile_row,
+                                          tile_ptr);
   return cudaGetLastError();
 }
 
