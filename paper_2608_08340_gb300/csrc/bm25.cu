@@ -3,7 +3,7 @@
 // term and giving the same scores as a scan of the whole corpus.
 //
 // The per-posting weight idf(t) * tf (k1 + 1) / (tf + k1 (1 - b + b |d| / avgdl))
-// does not depend on the query, so it is computed once on the host when the
+// does not depend on the query, so it is computed once on the device when the
 // sparse side is attached; a query's BM25 for chunk d is then the sum of the
 // weights of its terms' postings at d (a repeated term counts again).
 //
@@ -21,8 +21,9 @@
 // folds the tile maximum into the per-query maximum that normalises the
 // lexical score.
 //
-// A query holds about four of the thirty or so dense terms, so a CTA with
-// several queries of a tile copies that tile of all dense rows to shared
+// A query holds about four of the thirty or so dense terms, so with many queries
+// (kFewQueries) a CTA looks the terms of a tile's queries up together and copies
+// that tile of all dense rows to shared
 // memory once and the items read them there: 1024 queries on 32768 chunks read
 // 19 MB of dense rows from L2 instead of 530 MB.  What is left is the write of
 // the block (134 MB) and the shared-memory passes (about 30 KB per item).
@@ -49,6 +50,13 @@ constexpr int kBm25MaxRows = 29;
 // Queries of a tile in one CTA from which its dense rows are copied: a query
 // reads about four of them, so below that direct reads move fewer bytes.
 constexpr int kStageMinQueries = 8;
+// Queries up to which a warp takes its item's terms and dense rows by itself, so
+// that no barrier and no tile boundary holds the other warps up.  Measured, 500000
+// / 32768 chunks: 4 queries 15 / 12 us against 31 / 12 us, 16 queries 31 / 12
+// against 54 / 16, 64 queries 79 / 14 against 98 / 19, 128 queries 142 / 19
+// against 157 / 22; from 192 on 500000 chunks take the same (204, 204 us), and with
+// a thousand queries the copies of the dense rows tell (see above).
+constexpr int kFewQueries = 160;
 // Queries and terms of one batch whose lookups are done together.
 constexpr int kBatchQueries = 120;
 constexpr int kBatchTerms = 2048;
@@ -74,6 +82,7 @@ __device__ __forceinline__ TermSlot load_term(const SparseIndex& sp,
   return t;
 }
 
+template <bool kFew>
 __global__ void __launch_bounds__(kBm25Threads, 1)
 bm25_matrix_kernel(SparseIndex sp, int64_t n, const int32_t* __restrict__ q_indptr,
                    const int32_t* __restrict__ q_terms, int q, float* __restrict__ out, int64_t ld,
@@ -92,43 +101,56 @@ bm25_matrix_kernel(SparseIndex sp, int64_t n, const int32_t* __restrict__ q_indp
   const int64_t w1 = total * (blockIdx.x + 1) / gridDim.x;
   int loaded = -1;             // tile whose dense rows are in shared memory
   for (int64_t w = total * blockIdx.x / gridDim.x; w < w1;) {
-    const int tile = static_cast<int>(w / q);
-    const int qa = static_cast<int>(w - static_cast<int64_t>(tile) * q);
+    // A batch: queries of one tile, or with few queries the share's next items,
+    // a warp each.
+    const int64_t wa = w;
+    const int tile_a = static_cast<int>(w / q);
+    const int qa = static_cast<int>(w - static_cast<int64_t>(tile_a) * q);
     const int q_tile = static_cast<int>(min(static_cast<int64_t>(q), qa + (w1 - w)));
-    const int qb = min(q_tile, qa + kBatchQueries);
-    w += qb - qa;
-    const int64_t d0 = static_cast<int64_t>(tile) * kDocTile;
-    const int first_doc = static_cast<int>(d0);
-    const int nv = static_cast<int>((min(n - d0, static_cast<int64_t>(kDocTile)) + 3) / 4);
-    __syncthreads();           // the previous batch has been computed
-    for (int i = threadIdx.x; i <= qb - qa; i += kBm25Threads) q_ptr[i] = q_indptr[qa + i];
-    if (loaded != tile && q_tile - qa >= kStageMinQueries) {
-      for (int i = threadIdx.x; i < rows * (kDocTile / 4); i += kBm25Threads) {
-        const int r = i / (kDocTile / 4), v = i % (kDocTile / 4);
-        if (v < nv)
-          dense4[i] = __ldg(reinterpret_cast<const float4*>(sp.dense_w + r * sp.dense_ld + d0) + v);
+    const int items = kFew ? static_cast<int>(min(w1 - w, static_cast<int64_t>(kBm25Warps)))
+                           : min(q_tile - qa, kBatchQueries);
+    w += items;
+    int staged = 0, tb = 0;
+    bool listed = false;       // else the terms are looked up per item
+    if constexpr (!kFew) {
+      const int64_t d0 = static_cast<int64_t>(tile_a) * kDocTile;
+      const int nv = static_cast<int>((min(n - d0, static_cast<int64_t>(kDocTile)) + 3) / 4);
+      __syncthreads();         // the previous batch has been computed
+      for (int i = threadIdx.x; i <= items; i += kBm25Threads) q_ptr[i] = q_indptr[qa + i];
+      if (loaded != tile_a && q_tile - qa >= kStageMinQueries) {
+        for (int i = threadIdx.x; i < rows * (kDocTile / 4); i += kBm25Threads) {
+          const int r = i / (kDocTile / 4), v = i % (kDocTile / 4);
+          if (v < nv)
+            dense4[i] = __ldg(reinterpret_cast<const float4*>(sp.dense_w + r * sp.dense_ld + d0) + v);
+        }
+        loaded = tile_a;
       }
-      loaded = tile;
-    }
-    const int staged = loaded == tile ? rows : 0;
-    __syncthreads();
-    const int tb = q_ptr[0];
-    const bool listed = q_ptr[qb - qa] - tb <= kBatchTerms;    // else looked up per item
-    if (listed) {
-      for (int i = threadIdx.x; i < q_ptr[qb - qa] - tb; i += kBm25Threads) {
-        const TermSlot t = load_term(sp, q_terms, tb + i, tb + i + 1, tile);
-        t_slot[i] = t.slot;
-        t_lo[i] = t.lo;
-        t_hi[i] = t.hi;
-      }
+      staged = loaded == tile_a ? rows : 0;
       __syncthreads();
+      tb = q_ptr[0];
+      listed = q_ptr[items] - tb <= kBatchTerms;
+      if (listed) {
+        for (int i = threadIdx.x; i < q_ptr[items] - tb; i += kBm25Threads) {
+          const TermSlot t = load_term(sp, q_terms, tb + i, tb + i + 1, tile_a);
+          t_slot[i] = t.slot;
+          t_lo[i] = t.lo;
+          t_hi[i] = t.hi;
+        }
+        __syncthreads();
+      }
     }
-    auto term = [&](int ti, int t1) {
-      if (!listed) return load_term(sp, q_terms, ti, t1, tile);
-      return ti < t1 ? TermSlot{t_slot[ti - tb], t_lo[ti - tb], t_hi[ti - tb]} : TermSlot{-2, 0, 0};
-    };
-    for (int qi = qa + warp; qi < qb; qi += kBm25Warps) {
-      const int b0 = q_ptr[qi - qa], b1 = q_ptr[qi - qa + 1];
+    for (int item = warp; item < items; item += kBm25Warps) {
+      const int tile = kFew ? static_cast<int>((wa + item) / q) : tile_a;
+      const int qi = kFew ? static_cast<int>((wa + item) % q) : qa + item;
+      const int64_t d0 = static_cast<int64_t>(tile) * kDocTile;
+      const int first_doc = static_cast<int>(d0);
+      const int nv = static_cast<int>((min(n - d0, static_cast<int64_t>(kDocTile)) + 3) / 4);
+      const int b0 = kFew ? q_indptr[qi] : q_ptr[item];
+      const int b1 = kFew ? q_indptr[qi + 1] : q_ptr[item + 1];
+      auto term = [&](int ti, int t1) {
+        if (!listed) return load_term(sp, q_terms, ti, t1, tile);
+        return ti < t1 ? TermSlot{t_slot[ti - tb], t_lo[ti - tb], t_hi[ti - tb]} : TermSlot{-2, 0, 0};
+      };
       float4 acc[kVec];
 #pragma unroll
       for (int u = 0; u < kVec; ++u) acc[u] = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -300,13 +322,21 @@ cudaError_t launch_bm25_matrix(const SparseIndex& sp, int64_t n, const int32_t* 
   constexpr size_t kRow = kDocTile * sizeof(float);
   constexpr size_t kFixed = kBm25Warps * kRow +
                             (3 * kBatchTerms + kBatchQueries + 8) * sizeof(int);
-  static DeviceOnce once;
-  e = allow_smem(once, bm25_matrix_kernel, kFixed + kBm25MaxRows * kRow);
-  if (e != cudaSuccess) return e;
   // One CTA per SM (its shared memory), fewer when there are fewer items.
   const int64_t items = static_cast<int64_t>(sp.ntiles) * q;
   const int grid = static_cast<int>(std::min<int64_t>(items, num_sms));
-  bm25_matrix_kernel<<<grid, kBm25Threads, kFixed + rows * kRow, st>>>(
+  if (q <= kFewQueries) {
+    static DeviceOnce once;
+    e = allow_smem(once, bm25_matrix_kernel<true>, kFixed);
+    if (e != cudaSuccess) return e;
+    bm25_matrix_kernel<true><<<grid, kBm25Threads, kFixed, st>>>(sp, n, q_indptr, q_terms, q, out,
+                                                                 ld, out_max, 0);
+    return cudaGetLastError();
+  }
+  static DeviceOnce once;
+  e = allow_smem(once, bm25_matrix_kernel<false>, kFixed + kBm25MaxRows * kRow);
+  if (e != cudaSuccess) return e;
+  bm25_matrix_kernel<false><<<grid, kBm25Threads, kFixed + rows * kRow, st>>>(
       sp, n, q_indptr, q_terms, q, out, ld, out_max, rows);
   return cudaGetLastError();
 }

@@ -1,6 +1,6 @@
 """GPU parity of the BM25 pass (one warp per query and 1024-chunk tile) at its
 edges: corpora around the tile size, batches below and above the number of
-queries from which a CTA stages the dense rows, queries longer than one round
+queries from which a CTA looks terms up and stages dense rows for all, queries longer than one round
 of 32 terms, corpora without dense terms and with more dense terms than the
 shared memory holds, terms with more postings than one batch of loads."""
 import numpy as np
@@ -58,3 +58,29 @@ def test_more_dense_terms_than_staged():
 def test_postings_longer_than_a_batch_of_loads():
     # terms in up to half of the chunks: hundreds of postings per tile
     _check(4000, 20, vocab=120, zipf=0.3, terms=6, alpha=0.4, lens=(30, 60))
+
+
+# More than 160 queries: the terms of a tile's queries are looked up together
+# (up to 2048 of them), the dense rows copied to shared memory.
+@pytest.mark.parametrize("n,vocab,zipf,terms,lens", [
+    (1024, 500, 1.1, 5, (20, 60)),
+    (300, 300, 1.0, 70, (20, 60)),
+    (3000, 5000, 0.2, 6, (20, 60)),
+    (2100, 90, 0.1, 9, (150, 250)),
+    (4000, 120, 0.3, 6, (30, 60)),
+])
+def test_many_queries(n, vocab, zipf, terms, lens):
+    _check(n, 161, vocab, zipf, terms, alpha=0.3, lens=lens)
+
+
+@pytest.mark.parametrize("n", [1000, 1025, 30000, 200000])
+def test_a_query_scores_the_same_in_any_batch(n):
+    w = workloads.make_dense("bm", n, 64, 200, 9, "bf16", 2)
+    workloads.add_sparse(w, 2, vocab=900, s=1.0, len_lo=10, len_hi=30, terms_per_query=7)
+    idx = Index(dev_tensor(w.E_data))
+    idx.set_sparse(w.doc_indptr, w.doc_terms, 900, w.k1, w.b)
+    Q, ptr, terms = dev_tensor(w.Q_data), torch.from_numpy(w.q_indptr), torch.from_numpy(w.q_terms)
+    ids, sc = idx.hybrid_search(Q, ptr, terms, 0.0, 9)
+    for q in (1, 19, 160, 161):
+        i, s = idx.hybrid_search(Q[:q], ptr[:q + 1], terms, 0.0, 9)
+        assert torch.equal(i, ids[:q]) and torch.equal(s, sc[:q])
