@@ -3,7 +3,7 @@
 // and the vector is written in the index's dtype, ready for oprag_search.
 //
 // A row's result does not depend on the batch it comes in, nor on its padding:
-// tokens belong to eight lanes by their position (eight consecutive tokens to a
+// tokens belong to eight lanes by their position (sixteen consecutive tokens to a
 // lane), each lane is summed in order, the lanes are added in order, and the
 // squared norm is summed over the elements in a fixed order, however many CTAs
 // share the row.
@@ -33,7 +33,9 @@ namespace {
 
 constexpr int kPoolThreads = 256;
 constexpr int kLanes = 8;               // partial sums of a row
-constexpr int kTokenBlock = 8;          // consecutive tokens of a lane
+// Consecutive tokens of a lane (with eight, rows that one CTA reads alone are read
+// with more jumps: 256 x 512 x 4096 without padding 178 instead of 174 us).
+constexpr int kTokenBlock = 16;
 constexpr int kMaxShare = 2 * kPoolThreads;      // 16-byte groups of a token per CTA
 
 template <typename TIn>
@@ -77,7 +79,8 @@ embed_pool_kernel(const TIn* __restrict__ hidden, int tokens, int dim,
                   int ST) {
   namespace cg = cooperative_groups;
   constexpr int N = Group<TIn>::kN;
-  constexpr int kBlocks = R == 1 ? 2 : 1;         // of a lane, loaded together
+  constexpr int kStep = 16 / R;                   // tokens loaded together
+  static_assert(kTokenBlock % kStep == 0, "a step lies in one block");
   extern __shared__ __align__(16) float sums[];   // lanes' sums, then squares
   __shared__ float red[kPoolThreads / 32];
   __shared__ int part_count;
@@ -99,14 +102,11 @@ embed_pool_kernel(const TIn* __restrict__ hidden, int tokens, int dim,
   for (int r = 0; r < R; ++r)
 #pragma unroll
     for (int i = 0; i < N; ++i) tot[r][i] = 0.f;
-  // The steps of this CTA's lanes, one after the other: step (l, t) takes the
-  // lane's blocks at t and, with kBlocks = 2, at t + kStride.  The mask of a
-  // step's tokens, a byte per thread of the warp, is read a step ahead.
-  constexpr int kStride = kLanes * kTokenBlock;
+  // The steps of this CTA's lanes, one after the other.  The mask of a step's
+  // tokens, a byte per thread of the warp, is read a step ahead.
   const int lanes = min(kLanes, (tokens + kTokenBlock - 1) / kTokenBlock);   // that hold tokens
   auto read_mask = [&](int l, int t) -> uint32_t {
-    const int u = t + (wl & 7) + (wl >> 3) * kStride;
-    return l < lanes && wl < kBlocks * kTokenBlock && u < tokens ? mrow[u] : 0u;
+    return l < lanes && wl < kStep && t + wl < tokens ? mrow[t + wl] : 0u;
   };
   int count = 0;
   int l = tpart, t = l * kTokenBlock;
@@ -119,7 +119,8 @@ embed_pool_kernel(const TIn* __restrict__ hidden, int tokens, int dim,
   while (l < lanes) {
     const uint32_t m = __ballot_sync(0xffffffffu, byte != 0);
     const int at = t, lane = l;
-    t += kBlocks * kStride;
+    t += kStep;
+    if (t % kTokenBlock == 0) t += (kLanes - 1) * kTokenBlock;
     if (t >= tokens) {
       l += lane_step;
       t = l * kTokenBlock;
@@ -127,18 +128,17 @@ embed_pool_kernel(const TIn* __restrict__ hidden, int tokens, int dim,
     byte = read_mask(l, t);
     if (m != 0) {                                 // (no padding)
       count += __popc(m);
-      uint4 v[kBlocks * kTokenBlock][R];
+      uint4 v[kStep][R];
 #pragma unroll
-      for (int u = 0; u < kBlocks * kTokenBlock; ++u)
+      for (int u = 0; u < kStep; ++u)
 #pragma unroll
         for (int r = 0; r < R; ++r) {
           const int g = threadIdx.x + r * kPoolThreads;
-          const int token = at + u % kTokenBlock + u / kTokenBlock * kStride;
-          v[u][r] = ((m >> u) & 1u) && g < mine ? __ldg(row + static_cast<int64_t>(token) * groups + g)
+          v[u][r] = ((m >> u) & 1u) && g < mine ? __ldg(row + static_cast<int64_t>(at + u) * groups + g)
                                                 : make_uint4(0, 0, 0, 0);
         }
 #pragma unroll
-      for (int u = 0; u < kBlocks * kTokenBlock; ++u)
+      for (int u = 0; u < kStep; ++u)
 #pragma unroll
         for (int r = 0; r < R; ++r)
           if ((m >> u) & 1u) Group<TIn>::add(v[u][r], acc[r]);
@@ -254,13 +254,13 @@ embed_pool_kernel(const TIn* __restrict__ hidden, int tokens, int dim,
 
 // Parts of a row's elements, so that a CTA takes two groups a thread at most, and
 // of its lanes: as many as keep the batch within two CTAs per SM, with eight
-// CTAs (the portable cluster size) and one per two blocks of tokens at most.
+// CTAs (the portable cluster size) and one per 8 tokens at most.
 // Measured on GB300 with events (a pair takes 6 us of it), in brackets one CTA
-// per row and one chain of tokens, bf16: 1 x 512 x 4096 22 (85) us, 8 x 512 x 4096
-// 23 (87) us, 64 x 512 x 4096 62 (94) us, 152 x 512 x 4096 122 (116) us, or 90
-// (101) us with padded rows, 1 x 64 x 768 10 (13) us, 128 x 256 x 768 23 (37) us,
-// 20 x 512 x 8192 38 (148) us, 4 x 300 x 16384 38 (132) us; 256 x 512 x 4096 stays
-// at one CTA (134, 135 us).
+// per row and one chain of tokens, bf16: 1 x 512 x 4096 21 (85) us, 64 x 512 x 4096
+// with padding 48 (92) us, 152 x 512 x 4096 121 (116) us, with padding 90 (101) us,
+// 1 x 64 x 768 10 (13) us, 128 x 256 x 768 23 (37) us, 512 x 1024 x 512 158 (205)
+// us, 20 x 512 x 8192 38 (148) us, 4 x 300 x 16384 38 (132) us; 256 x 512 x 4096
+// stays at one CTA (133, 135 us).
 struct Split {
   int dim, lanes;
 };
@@ -269,7 +269,7 @@ Split split_for(int batch, int tokens, int groups, int num_sms) {
   Split s{1, 1};
   while (s.dim < 8 && groups > s.dim * kMaxShare) s.dim *= 2;
   while (s.dim * s.lanes < 8 && static_cast<int64_t>(batch) * 2 * s.dim * s.lanes <= 2 * num_sms &&
-         2 * s.lanes * kTokenBlock <= tokens)
+         16 * s.lanes <= tokens)
     s.lanes *= 2;
   return s;
 }
