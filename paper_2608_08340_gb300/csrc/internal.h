@@ -71,7 +71,8 @@ struct ListSet {
 // Optional lexical part of the fused score (Sec. 4.4 weighted fusion):
 // f = alpha * dense + (1 - alpha) * BM25(q, id) / max_q, zero lexical part when
 // max_q <= 0.  Two forms:
-//  * materialised (SIMT kernel): bm25 is a q x ld block of BM25 values;
+//  * materialised: bm25 is a q x ld block of BM25 values, read by the
+//    tensor-core (kLexBlock), fp32 and SIMT kernels;
 //  * gathered in the tensor-core epilogue (bm25 == nullptr, lex_qcount set).
 //    Each term of the sparse side has a class (lex_class):
 //    - head (class s in [0, kLexHeadTerms)): one more K block of tensor-core
@@ -233,14 +234,14 @@ cudaError_t launch_group_select(const float* gmax, int64_t gld, int groups, int 
 
 // --- final merge of partial lists into the sorted top-k per query.
 constexpr int kLevels = 4;
-// Ranks k/16, k/8, k/4, k/2 (at least 1): candidate floors for a search of
-// k > 32 that a first pass over a sample of the corpus tiles proposes.
+// Ranks k/16, k/8, k/4, k/2 (at least 1) among the group maxima of a search of
+// k > 32: the candidate floors that its group pass proposes.
 inline __host__ __device__ int level_rank(int k, int i) {
   const int r = k >> (kLevels - i);
   return r < 1 ? 1 : r;
 }
 cudaError_t launch_merge(const ListSet& ls, int q, int k, int64_t* out_ids, float* out_scores,
-                         cudaStream_t st);
+                         int num_sms, cudaStream_t st);
 
 // Two ranked lists per query (a: q x ka, b: q x kb, each sorted score
 // descending then id ascending) into the top-k of both, score descending,

@@ -181,11 +181,11 @@ merge_small_kernel(ListSet ls, int q, int k, int64_t* __restrict__ out_ids,
 constexpr int kUnsortedLoads = 4;
 constexpr int kRankMax = 256;       // keys that rank_buffer takes
 static_assert(kRankMax >= OPRAG_K_MAX, "the k best can be ranked");
-// Up to this many queries, whose CTAs the SMs hold all at once (ten of four
-// warps each), four warps a query; above, two.  Four against two warps,
+// Up to this many queries per SM, whose CTAs the SMs hold all at once, four warps
+// a query; above, two.  Four against two warps,
 // event-timed, k = 100: 300 queries of 300000 x 128 12 / 16 us, 1024 queries 16
 // / 16 us, 4000 queries 35 / 31 us; 2048 queries of 1048576 x 768 27 / 23 us.
-constexpr int kUnsortedWideQueries = 1520;
+constexpr int kUnsortedWideQueries = 10;
 
 template <int W>
 struct Unsorted {
@@ -500,11 +500,13 @@ cudaError_t launch_merge_two(int q, const int64_t* a_ids, const float* a_sc, int
   return cudaGetLastError();
 }
 
-cudaError_t launch_merge(const ListSet& ls, int q, int k, int64_t* out_ids, float* out_scores, cudaStream_t st) {
+cudaError_t launch_merge(const ListSet& ls, int q, int k, int64_t* out_ids, float* out_scores,
+                         int num_sms, cudaStream_t st) {
   if (q <= 0) return cudaSuccess;
   if (ls.counts != nullptr)
-    return q <= kUnsortedWideQueries ? launch_unsorted<4>(ls, q, k, out_ids, out_scores, st)
-                                     : launch_unsorted<2>(ls, q, k, out_ids, out_scores, st);
+    return q <= kUnsortedWideQueries * num_sms
+               ? launch_unsorted<4>(ls, q, k, out_ids, out_scores, st)
+               : launch_unsorted<2>(ls, q, k, out_ids, out_scores, st);
   if (ls.P <= 32)
     return launch_warp_per_query(merge_kway_kernel, kWayWarps, ls, q, k, out_ids, out_scores, st);
   return launch_small(ls, q, k, out_ids, out_scores, st);

@@ -493,7 +493,7 @@ int launch_search(oprag_index* idx, const SearchLayout& L, const void* Q, int q,
     lists.out_src = out_src;
   }
   if (!L.small || !L.splan_small.inline_merge) {
-    e = launch_merge(lists, q, k, out_ids, out_scores, st);
+    e = launch_merge(lists, q, k, out_ids, out_scores, idx->num_sms, st);
     if (e != cudaSuccess) return cuda_fail(e, "merge kernel");
   }
   if (idx->timing) cudaEventRecord(idx->ev[3], st);

@@ -214,11 +214,7 @@ __device__ __forceinline__ void redo_overflowed(const Params& p, int64_t r0, int
   }
 }
 
-// The warp puts the min(c, k) best of the c keys of a buffer, best first, into
-// dst (which may be the buffer).  Up to 64 keys -- the usual case, a good
-// floor leaves few more than k -- every lane counts the keys above its own
-// ones: no chain of dependent exchanges (14 queries a warp at the end of a
-// search: 1 us instead of 10 us of bitonic sorts).  More keys are sorted.
+// keep_best for c <= 32 E keys: a bitonic sort.
 template <int E>
 __device__ __noinline__ void sort_best(uint64_t* buf, int c, int k, uint64_t* dst) {
   const int lane = threadIdx.x & 31;
@@ -233,6 +229,7 @@ __device__ __noinline__ void sort_best(uint64_t* buf, int c, int k, uint64_t* ds
   __syncwarp();
 }
 
+// keep_best for c <= 32 E keys, by counting.
 template <int E>
 __device__ __forceinline__ void rank_best(const uint64_t* buf, int c, int k, uint64_t* dst) {
   const int lane = threadIdx.x & 31;
@@ -256,6 +253,11 @@ __device__ __forceinline__ void rank_best(const uint64_t* buf, int c, int k, uin
   __syncwarp();
 }
 
+// The warp puts the min(c, k) best of the c keys of a buffer, best first, into
+// dst (which may be the buffer).  Up to 64 keys -- the usual case, a good
+// floor leaves few more than k -- every lane counts the keys above its own
+// ones: no chain of dependent exchanges (14 queries a warp at the end of a
+// search: 1 us instead of 10 us of bitonic sorts).  More keys are sorted.
 __device__ __forceinline__ void keep_best(uint64_t* buf, int c, int k, uint64_t* dst) {
   if (c <= 32) rank_best<1>(buf, c, k, dst);
   else if (c <= 64) rank_best<2>(buf, c, k, dst);

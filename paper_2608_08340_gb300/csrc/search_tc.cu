@@ -121,7 +121,15 @@ TcPlan tc_plan(const SearchShape& s, int num_sms, int force_block_n, int tile_st
   pl.sets = pl.dual ? 1 : epi_sets(list_len_of(s), s.fused_lex);
   pl.pmax = per_tile * pl.sets;
   const int K = list_len_of(s);
-  // Shared memory of the launch (the same sum as smem_for<BN, K, pair, dual>).
+  // Shared memory of the launch (the same sum as smem_for<BN, K, pair, dual>;
+  // the barriers of the BM25 block form cost no stage).
+  constexpr int kBlockBar = block_bar_bytes<8, kLexBlock>();
+  static_assert(stages_for<256, true, false, false, kBlockBar>() == stages_for<256, true>() &&
+                    stages_for<128, false, true, false, kBlockBar>() ==
+                        stages_for<128, false, true>() &&
+                    stages_for<128, false, false, false, kBlockBar>() == stages_for<128>() &&
+                    stages_for<256, false, false, false, kBlockBar>() == stages_for<256>(),
+                "stages of the BM25 block form");
   const size_t b_stage = static_cast<size_t>(pair ? bn / 2 : bn) * 128;
   const size_t a_stage = kAStageBytes * (pl.dual ? 2 : 1);
   pl.stages = pair        ? stages_for<256, true>()
@@ -130,7 +138,7 @@ TcPlan tc_plan(const SearchShape& s, int num_sms, int force_block_n, int tile_st
                             : (bn == 128 ? stages_for<128>() : stages_for<256>());
   pl.smem = static_cast<size_t>(pl.stages) * (a_stage + b_stage) +
             static_cast<size_t>(epi_sets(K, s.fused_lex)) * 128 * kStageRowBytes +
-            lex_land_bytes(s.fused_lex) + 1024 + 256;
+            lex_land_bytes(s.fused_lex) + (s.lex_block ? kBlockBar : 0) + 1024 + 256;
   return pl;
 }
 

@@ -299,3 +299,28 @@ def test_merge_regimes(q, k):
     rows = np.sort(rng.choice(q, min(q, 40), replace=False))
     check_dense(ids, sc, E, Q, k, f"merge q={q} k={k}", rows=rows)
     idx.check()
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "f32"])
+@pytest.mark.parametrize("q,k", [
+    (1, 1), (6, 8),          # the search kernel's own merge writes to host memory
+    (7, 8), (32, 16),
+    (170, 32), (171, 32),    # 65280 and 65664 bytes: written by the device, copied
+    (40, 200),
+])
+def test_host_results_are_the_device_results(dtype, q, k):
+    rng = np.random.default_rng(q + k)
+    cast = torch.bfloat16 if dtype == "bf16" else torch.float32
+    E = torch.from_numpy(rng.standard_normal((5003, 96)).astype(np.float32)).to(cast)
+    Q = torch.from_numpy(rng.standard_normal((q, 96)).astype(np.float32)).to(cast)
+    idx = Index(E)
+    ref_ids, ref_sc = idx.search(Q.cuda(), k)
+    for pinned in (False, True):
+        for _ in range(2):
+            out = (torch.full((q, k), -7, dtype=torch.int64), torch.full((q, k), 7.0))
+            if pinned:
+                out = tuple(t.pin_memory() for t in out)
+            ids, sc = idx.search_host(Q.pin_memory() if pinned else Q, k, out=out)
+            assert ids is out[0] and torch.equal(ids, ref_ids.cpu())
+            assert torch.equal(sc, ref_sc.cpu())
+    idx.close()
