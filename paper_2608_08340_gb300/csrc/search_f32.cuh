@@ -163,6 +163,13 @@ __device__ __forceinline__ void mul_block(const unsigned char* a0, const unsigne
       for (int j = TN; j < kRowsPerThread; ++j) mid[i][j] = 0.f;
 }
 
+// The fused score of query qg and row r (Sec. 4.4), the dense one without a block.
+__device__ __forceinline__ float fuse(const Fusion& fu, float s, int qg, int64_t r) {
+  if (fu.bm25 == nullptr) return s;
+  const float m = fu.bm25_max[qg], inv_max = m > 0.f ? 1.f / m : 0.f;
+  return fmaf(fu.alpha, s, (1.f - fu.alpha) * (fu.bm25[qg * fu.ld + r] * inv_max));
+}
+
 // max(m, |a|, |b|), NaN when one of them is.
 __device__ __forceinline__ float max_abs_nan(float m, float a, float b) {
   asm("max.NaN.f32 %0, %0, %1, %2;" : "+f"(m) : "f"(fabsf(a)), "f"(fabsf(b)));
@@ -172,45 +179,55 @@ __device__ __forceinline__ float max_abs_nan(float m, float a, float b) {
 // Scores that passed the fp32 range: the carried errors of the sums turn an
 // infinite sum into NaN, so those scores are formed again as plain sums in the
 // order of the dimensions, where an overflowed sum of finite products keeps its
-// infinity.  Looked for once per tile (a check in each K block, to drop the
-// carried errors there, took 6 of 204 us at 100 queries of 32768 x 768).
-// r0, q0: the thread's first corpus row and query; rows end at r_end.
-template <int TY, int TM>
-__device__ __forceinline__ void redo_overflowed(const Params& p, int64_t r0, int64_t r_end, int q0,
-                                                float (&tot)[TM][kRowsPerThread]) {
-  constexpr int TX = kThreads / TY;
-  float worst = 0.f;
+// infinity.  They are looked for once per tile, behind the pushes of the other
+// scores.  Measured against no such care, 32768 x 768: 100 queries 194 (194) us, 60
+// 118 (114), 32 77 (73), 20 51 (49), and 414 (418) us at 256 queries of 65536 x 384;
+// with a check in each K block, to drop the carried errors there, 100 queries took
+// 6 us more, and with the scores formed before the selection 2 us (32 queries 80).
+// Returns bit 4 i + j for each.
+template <int TM>
+__device__ __forceinline__ uint32_t find_overflowed(const float (&score)[TM][kRowsPerThread]) {
+  float any = 0.f;
 #pragma unroll
   for (int i = 0; i < TM; ++i)
 #pragma unroll
     for (int j = 0; j < kRowsPerThread; j += 2)
-      worst = max_abs_nan(worst, tot[i][j], tot[i][j + 1]);
-  if (worst <= FLT_MAX) return;
-  uint32_t redo = 0;                   // bit 4 i + j
+      any = max_abs_nan(any, score[i][j], score[i][j + 1]);
+  uint32_t redo = 0;
+  if (any != any) {
 #pragma unroll
-  for (int i = 0; i < TM; ++i)
+    for (int i = 0; i < TM; ++i)
 #pragma unroll
-    for (int j = 0; j < kRowsPerThread; ++j)
-      if (!(fabsf(tot[i][j]) <= FLT_MAX) && r0 + TX * j < r_end && q0 + TY * i < p.q)
-        redo |= 1u << (kRowsPerThread * i + j);
+      for (int j = 0; j < kRowsPerThread; ++j)
+        if (score[i][j] != score[i][j]) redo |= 1u << (kRowsPerThread * i + j);
+  }
+  return redo;
+}
+
+// Forms the scores of `redo` (all of rows and queries that exist) and pushes those
+// that reach their query's floor.  r0, ql0: the thread's first corpus row, and its
+// first query of the tile at q0.
+template <int TY>
+static __device__ __noinline__ void push_overflowed(const Params& p, uint32_t redo, int64_t r0,
+                                                    int q0, int ql0, uint64_t* buf, int* cnt,
+                                                    const uint32_t* flo) {
+  constexpr int TX = kThreads / TY;
 #pragma unroll 1
   for (; redo != 0; redo &= redo - 1) {
     const int at = __ffs(redo) - 1;
-    const float4* e = reinterpret_cast<const float4*>(
-        p.E + (r0 + TX * (at % kRowsPerThread)) * p.d);
-    const float4* q = reinterpret_cast<const float4*>(
-        p.Q + static_cast<int64_t>(q0 + TY * (at / kRowsPerThread)) * p.d);
+    const int64_t r = r0 + TX * (at % kRowsPerThread);
+    const int ql = ql0 + TY * (at / kRowsPerThread), qg = q0 + ql;
+    const float4* e = reinterpret_cast<const float4*>(p.E + r * p.d);
+    const float4* q = reinterpret_cast<const float4*>(p.Q + static_cast<int64_t>(qg) * p.d);
     float s = 0.f;
 #pragma unroll 2
     for (int t = 0; t < p.d / 4; ++t) {
       const float4 x = __ldg(e + t), y = __ldg(q + t);
       s = fmaf(x.w, y.w, fmaf(x.z, y.z, fmaf(x.y, y.y, fmaf(x.x, y.x, s))));
     }
-#pragma unroll
-    for (int i = 0; i < TM; ++i)
-#pragma unroll
-      for (int j = 0; j < kRowsPerThread; ++j)
-        if (at == kRowsPerThread * i + j) tot[i][j] = s;
+    s = fuse(p.fu, s, qg, r);
+    if (s >= order_score(flo[ql]))
+      buf[ql * p.cap + atomicAdd(cnt + ql, 1)] = make_key(s, static_cast<uint32_t>(r));
   }
 }
 
@@ -321,7 +338,7 @@ __device__ __forceinline__ float rank_of_8(float (&v)[E], int r) {
 template <int TY, int TM, bool kFine>
 __global__ void __launch_bounds__(kThreads, 1)
 f32_search_kernel(const __grid_constant__ CUtensorMap map_q,
-                  const __grid_constant__ CUtensorMap map_e, const Params p) {
+                  const __grid_constant__ CUtensorMap map_e, const __grid_constant__ Params p) {
   constexpr int TX = kThreads / TY;
   constexpr int BM = TY * TM, BN = TX * kRowsPerThread;
   constexpr int WY = TY / 4;                          // warps along the queries
@@ -442,8 +459,6 @@ f32_search_kernel(const __grid_constant__ CUtensorMap map_q,
       if (!kFine) add_sums<TM, kRowsPerThread>(acc, tot, lost);
     }
 
-    redo_overflowed<TY, TM>(p, r0 + tx, r_end, q0 + ty, tot);
-
     // ---- selection
     // The scores (in the accumulators' place), -inf where there is none.
 #pragma unroll
@@ -473,19 +488,21 @@ f32_search_kernel(const __grid_constant__ CUtensorMap map_q,
 #pragma unroll
       for (int i = 0; i < TM; ++i) {
         const int ql = ty + TY * i;
-        float b, v[kRowsPerThread];
-        // NaN counts for nothing: the sorts' minima and maxima would put a
-        // second copy of another score in its place.
-#pragma unroll
-        for (int j = 0; j < kRowsPerThread; ++j) v[j] = fmaxf(acc[i][j], -INFINITY);
+        // NaN counts for nothing (fmaxf with -inf): the sorts' minima and maxima
+        // would put a second copy of another score in its place.
+        const float none = -INFINITY;
+        float b;
         if (p.k <= 8) {
-          float m[1] = {fmaxf(fmaxf(v[0], v[1]), fmaxf(v[2], v[3]))};
+          float m[1] = {fmaxf(fmaxf(fmaxf(acc[i][0], acc[i][1]), fmaxf(acc[i][2], acc[i][3])), none)};
           b = rank_of_8<1>(m, p.k - 1);
         } else if (p.k <= 16) {
-          float m[2] = {fmaxf(v[0], v[1]), fmaxf(v[2], v[3])};
+          float m[2] = {fmaxf(fmaxf(acc[i][0], acc[i][1]), none),
+                        fmaxf(fmaxf(acc[i][2], acc[i][3]), none)};
           b = rank_of_8<2>(m, p.k - 1);
         } else {
-          b = rank_of_8<4>(v, p.k - 1);
+          float m[4] = {fmaxf(acc[i][0], none), fmaxf(acc[i][1], none), fmaxf(acc[i][2], none),
+                        fmaxf(acc[i][3], none)};
+          b = rank_of_8<4>(m, p.k - 1);
         }
         if ((lane & 7) == 0 && b > -INFINITY) atomicMax(flo + ql, score_order(b));
       }
@@ -527,6 +544,8 @@ f32_search_kernel(const __grid_constant__ CUtensorMap map_q,
         if ((take >> (kRowsPerThread * i + j)) & 1u)
           *b++ = make_key(acc[i][j], static_cast<uint32_t>(r0 + tx + TX * j));
     }
+    const uint32_t redo = find_overflowed<TM>(acc);
+    if (redo != 0) push_overflowed<TY>(p, redo, r0 + tx, q0, ty, buf, cnt, flo);
     __syncthreads();
     // Buffers without room for another tile, or of the last tile: keep the k
     // best.

@@ -147,6 +147,24 @@ def test_overflowing_scores_keep_their_infinity(q, d, k):
     assert ids.cpu().tolist() == [list(range(k))] * q and torch.isposinf(sc).all()
 
 
+@pytest.mark.parametrize("q", [3, 100])
+def test_overflowing_scores_in_the_hybrid_search(q):
+    n, d = 2000, 96
+    rng = np.random.default_rng(q)
+    E = rng.standard_normal((n, d)).astype(np.float32)
+    E[[3, 1100, 1999]] = 3e38
+    E[700] = -3e38
+    terms = rng.integers(0, 40, 5 * n).astype(np.int32)
+    idx = Index(dev_tensor(E))
+    idx.set_sparse(np.arange(n + 1, dtype=np.int32) * 5, terms, 40)
+    ids, sc = idx.hybrid_search(dev_tensor(np.ones((q, d), np.float32)),
+                                torch.arange(q + 1, dtype=torch.int32),
+                                torch.arange(q, dtype=torch.int32) % 40, 0.5, 12)
+    assert ids.cpu()[:, :3].tolist() == [[3, 1100, 1999]] * q
+    assert torch.isposinf(sc[:, :3]).all() and torch.isfinite(sc[:, 3:]).all()
+    assert not (ids == 700).any()
+
+
 @pytest.mark.parametrize("q", [3, 40, 100])
 @pytest.mark.parametrize("n", [20, 30000])
 def test_scores_of_minus_infinity_are_no_results(q, n):
