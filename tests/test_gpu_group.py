@@ -54,6 +54,27 @@ def test_equal_scores(n, k):
     assert (sc.cpu().numpy() == 64).all()
 
 
+@pytest.mark.parametrize("reps,k,q", [(30, 40, 3), (80, 100, 3), (80, 100, 300)])
+def test_ties_at_rank_k_with_counted_floors(reps, k, q):
+    """1500 distinct rows, each stored `reps` times, a group pass over every
+    fourth tile: rank k falls inside a group of equal scores, and the merge,
+    which drops keys below the best counted floor, must keep its lowest ids."""
+    rng = np.random.default_rng(reps)
+    base = _rows(rng, 1500, 128)
+    E = np.ascontiguousarray(np.tile(base, (reps, 1)))
+    Q = np.ascontiguousarray(base[rng.choice(1500, q, replace=False)])
+    scores = oracle.bf16_to_f32(Q).astype(np.float64) @ oracle.bf16_to_f32(base).astype(np.float64).T
+    order = np.argsort(-scores, axis=1)
+    best = np.take_along_axis(scores, order, axis=1)
+    apart = (-np.diff(best[:, :k // reps + 2], axis=1)).min(axis=1) > 10 * TOL
+    assert apart.sum() >= q // 2             # only ties within a group are ambiguous there
+    want = (order[:, :k // reps + 1, None] + 1500 * np.arange(reps)).reshape(q, -1)[:, :k]
+    idx = Index(dev_tensor(E))
+    ids, _ = idx.search(dev_tensor(Q), k)
+    assert (ids.cpu().numpy()[apart] == want[apart]).all()
+    idx.check()
+
+
 @pytest.mark.parametrize("gather", [False, True])
 def test_hybrid(gather):
     w = workloads.config(3, n=9000, batch=70)

@@ -109,8 +109,8 @@ def test_search_two_matches_the_stacked_oracle(nk, nm, k):
                                        (20000, 45000, 130, 100), (256, 70000, 600, 7),
                                        (1000, 1, 3, 2)])
 def test_search_two_is_one_search_over_the_stacked_rows(nk, nm, q, k):
-    """The two-index search runs one search pass (and, for k > 32 over many
-    tiles, one sampled pass) over the knowledge rows followed by the memory
+    """The two-index search runs one search pass (and, for k > 32, one
+    group pass) over the knowledge rows followed by the memory
     rows: its results equal a search of one index holding the stacked rows,
     with memory ids shifted by the knowledge size (scores within 1e-6, ids
     equal outside 1e-6 near-ties: the two runs may tile the rows

@@ -2,7 +2,7 @@
 issuing M = 256 MMAs, each CTA loading half of every 256-row corpus tile),
 against the fp64 oracle and against the single-CTA kernel: odd numbers of
 query tiles (the last pair's second tile empty or ragged), one query tile
-forced onto a pair, buffered lists (k > 32) with the sampled floor, and the
+forced onto a pair, buffered lists (k > 32) with the group pass, and the
 fused hybrid score."""
 import numpy as np
 import pytest

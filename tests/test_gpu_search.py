@@ -202,7 +202,7 @@ def test_config4_scale_with_upserts_sampled():
             oracle.upsert(E, up_ids, up_rows)
         Qb = w.Q_data[b * 2048:(b + 1) * 2048]
         ids, sc = idx.search(dev_tensor(Qb), w.k)
-        # the full-size path: CTA pairs, sampled first pass and counted floors
+        # the full-size path: CTA pairs, group pass and counted floors
         assert idx.last_launch["cluster"] == 2
         assert idx.last_timing()["sample_ms"] > 0.0
         # 128 rows: two in every lane quarter of all 16 query tiles
@@ -217,9 +217,9 @@ def test_config4_scale_with_upserts_sampled():
 
 @pytest.mark.parametrize("k", [33, 100, 256])
 def test_large_k_with_sampled_floor(k):
-    """k > 32 over many corpus tiles: the search first scans every 32nd tile
-    to get a lower bound of each query's k-th best score, then the full scan
-    admits only scores above it.  Results must still be exact."""
+    """k > 32 over many corpus tiles: the group pass scans some of them to get
+    a lower bound of each query's k-th best score, then the full scan admits
+    only scores that reach it.  Results must still be exact."""
     rng = np.random.default_rng(k)
     n, d, q = 160000, 128, 130
     E = workloads.to_bf16_bits(workloads._normalise(rng.standard_normal((n, d)).astype(np.float32)))
@@ -233,10 +233,10 @@ def test_large_k_with_sampled_floor(k):
 
 
 def test_large_k_exact_ties_at_kth():
-    """k = 100 over 1500 distinct rows, each stored 30 times (45000 rows, so
-    the sampled first pass and the counted floors run): the 100th result
-    falls inside a group of 30 equal scores, and the merge, which drops keys
-    below the proven floor, must still return the group's lowest ids."""
+    """k = 100 over 1500 distinct rows, each stored 30 times (45000 rows): the
+    100th result falls inside a group of 30 equal scores, and the search, which
+    drops scores below the group pass's floor, must still return the group's
+    lowest ids (with counted floors: test_gpu_group.py)."""
     rng = np.random.default_rng(0)
     m, reps, d = 1500, 30, 128
     base = oracle.round_bf16(workloads._normalise(rng.standard_normal((m, d)).astype(np.float32)))

@@ -249,9 +249,9 @@ def test_hybrid_more_head_terms_than_tensor_core_slots(gather):
 @pytest.mark.parametrize("gather", [False, True])
 @pytest.mark.parametrize("k", [33, 100])
 def test_hybrid_large_k_with_sampled_floor(k, gather):
-    """k > 32 over 313 corpus tiles: the sampled first pass (every 32nd tile,
-    so the postings cursors are placed again at every unit) runs the fused
-    epilogue too."""
+    """k > 32 over 313 corpus tiles: the group pass (every fourth tile for
+    k = 33, so the gathered form places its postings cursors again at every
+    unit) runs the fused epilogue too."""
     w = workloads.config(3, n=40000, batch=130)
     idx = Index(dev_tensor(w.E_data))
     idx.set_sparse(w.doc_indptr, w.doc_terms, w.vocab, w.k1, w.b)

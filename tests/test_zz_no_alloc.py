@@ -1,7 +1,7 @@
 """oprag_search_noalloc: the search entry point for callers that must not
 allocate device memory while serving (a process whose memory pool already
 holds the GPU, or one that cannot take the device-wide synchronisation a
-cudaMalloc or cudaFree may cause).  Its partial lists, sampled first pass and
+cudaMalloc or cudaFree may cause).  Its partial lists, group pass and
 shared bounds live in a static 16 MiB device array instead of the index's
 growable scratch buffer.
 
