@@ -1066,7 +1066,7 @@ size_t tile_rows(const std::vector<int64_t>& df, const std::vector<int32_t>& slo
                  int ntiles, std::vector<int64_t>* rows) {
   constexpr int64_t kSmallTable = int64_t(8) << 20;
   const int64_t vocab = static_cast<int64_t>(df.size());
-  const int64_t limit = std::max(kSmallTable, vocab * (n / 8192 + 2) * 8);
+  const int64_t limit = std::max(kSmallTable, vocab * ((n + 8191) / 8192 + 1) * 8);
   rows->clear();
   const int64_t full = vocab * (ntiles + 1);
   if (full * 4 <= limit) return static_cast<size_t>(full);
@@ -1075,7 +1075,9 @@ size_t tile_rows(const std::vector<int64_t>& df, const std::vector<int32_t>& slo
     int64_t entries = 0;
     for (size_t t = 0; t < df.size(); ++t) {
       const int64_t postings = slot[t] < 0 ? df[t] : 0;
-      int shift = 0, cells = ntiles;
+      // (a wider P only widens cells: go on from the last one's)
+      int shift = P == 1 ? 0 : static_cast<int>((*rows)[t] & ((1 << kTileShiftBits) - 1));
+      int64_t cells = ((ntiles - 1) >> shift) + 1;
       while (cells > 1 && cells * P > postings) cells = ((ntiles - 1) >> ++shift) + 1;
       (*rows)[t] = tile_row_of(entries, shift);
       entries += cells + 1;
